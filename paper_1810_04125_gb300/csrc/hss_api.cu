@@ -323,6 +323,15 @@ struct PhaseTimer {
 };
 enum { PH_SAMPLE = 0, PH_ID = 1, PH_TEST = 2, PH_MERGE = 3, PH_OTHER = 4, PH_RNG = 5, PH_N = 7 };
 
+// Digits of a generated source's entries (exact-split sampling), kept from
+// the first sampling pass of a compression to its end: per orientation the
+// packed digits, and the largest entry of every row (2 n).
+struct XsKeep {
+  unsigned char* pa[2] = {nullptr, nullptr};
+  unsigned* ea = nullptr;   // 2 n
+  bool have = false;
+};
+
 }  // namespace
 
 struct hss_matrix_s {
@@ -346,6 +355,7 @@ struct hss_matrix_s {
   int pack_decided = -1;   // mixed forms, generated A: packed tiles (1) or not (0)
   bool sym = false;        // symmetric option: the column side mirrors the row side
   void* packA = nullptr;   // packed tensor-core tiles of a dense A (during compress)
+  XsKeep xs;               // digits of a generated source (during compress, plain form)
   void* toep_terms = nullptr; // a Toeplitz source's diagonals split into terms (during compress)
   bool usable = false;
   bool partial = false;    // not converged; the uncompressed part kept dense (F12, F21)
@@ -356,6 +366,7 @@ struct hss_matrix_s {
   ~hss_matrix_s() {
     if (packA) cudaFree(packA);
     if (toep_terms) cudaFree(toep_terms);
+    if (xs.pa[0]) cudaFree(xs.pa[0]);
     arena.release();
   }
 };
@@ -394,19 +405,22 @@ struct DevBuf {
 // scratch, the job-list buffer, the device flags and the pinned read-back
 // buffer, the phase timer and the counters.
 //   d_flag[0..7]: [1] tensor-core sampling wait, [2] QRCP barrier,
-//   [3] tensor-core tile product wait, [4] Incrementing test barrier;
+//   [3] tensor-core tile product wait, [4] Incrementing test barrier,
+//   [5] exact-split product wait;
 //   d_flag[8 + i]: non-finite samples of matrix i.
 struct Ctx {
   cudaStream_t st = nullptr;
   Scratch scratch;
   DevBuf jobs;
   DevBuf gpack;   // operands of the tensor-core tile products split into their terms
+  DevBuf xz, xp;  // exact-split products: zeroed bookkeeping, digits of the operands
   int* d_flag = nullptr;
   int nflag = 0;
   int* h_pinned = nullptr;
   size_t h_pinned_cap = 0;
   PhaseTimer timer;
   long long launches = 0, sample_launches = 0, bytes_h2d = 0, bytes_d2h = 0;
+  size_t xs_kept = 0;      // bytes of digits kept by the matrices of the call (XsKeep)
   bool trace = false;      // HSS_TRACE=1: one stderr line per launch of the batched phases
   cudaEvent_t trace_ev[2] = {nullptr, nullptr};
   int qrcp_cap = -1, qrcp_cap_d = -1, qrcp_cap_w = -1, qrcp_nsm = 0, qrcp_per = 0;
@@ -423,6 +437,8 @@ struct Ctx {
       if (e) cudaEventDestroy(e);
     jobs.release(st);
     gpack.release(st);
+    xz.release(st);
+    xp.release(st);
     if (d_flag) cudaFreeAsync(d_flag, st);
     scratch.release();
     if (h_pinned) cudaFreeHost(h_pinned);
@@ -580,6 +596,41 @@ GemmJob gemm_job() {
   j.c_split = 0x7fffffff;
   j.alpha = 1.0;
   return j;
+}
+
+// ---- exact-split FP64 products (k_gemm_xs.cu)
+constexpr size_t kXsCap = size_t(2) << 30;   // digits of the operands of one launch
+constexpr int kSms = 152;
+constexpr size_t kXsKeep = size_t(4) << 30;  // digits of generated sources kept over a compression
+
+// k-tiles per CTA of launches whose tiles (count, k-tiles each) are given:
+// the split of K that takes the fewest waves x (k-tiles + the fixed cost of a
+// CTA, about six k-tiles; partial sums cost two more).
+int xs_seg_ktiles(const std::vector<std::pair<long long, int>>& tiles) {
+  long long work = 0;
+  int kmax = 1;
+  for (auto& t : tiles) {
+    work += t.first * t.second;
+    kmax = std::max(kmax, t.second);
+  }
+  auto cost = [&](int g) {
+    long long ctas = 0;
+    for (auto& t : tiles) ctas += t.first * ((t.second + g - 1) / g);
+    return (double)((ctas + kSms - 1) / kSms) * (std::min(g, kmax) + (g < kmax ? 8 : 6));
+  };
+  int best = kmax;
+  double bc = cost(kmax);
+  for (int w = 1; w <= 8; ++w) {
+    for (int up = 0; up < 3; ++up) {
+      const int g = (int)std::min<long long>(kmax, std::max<long long>(4, (work + (long long)w * kSms - 1) / ((long long)w * kSms) + up));
+      const double q = cost(g);
+      if (q < 0.97 * bc) {
+        bc = q;
+        best = g;
+      }
+    }
+  }
+  return best;
 }
 
 // Runs a list of tile-product jobs (one launch).  tc_prec: HSS_PREC_FP64 for
@@ -801,6 +852,150 @@ bool use_packed(hss_matrix_s* H) {
   return H->pack_decided == 1;
 }
 
+// A = A^T by the definition of the source: the point kernels depend on
+// |x_i - x_j| only (entry (i, j) and (j, i) are the same bits), a Toeplitz
+// matrix has one table for both halves.
+bool symmetric_source(const SrcDev& s) {
+  return s.kind == HSS_SRC_GAUSS || s.kind == HSS_SRC_LAPLACE || (s.kind == HSS_SRC_TOEPLITZ && s.a == s.b);
+}
+
+// The FP64 sampling Sr = (A - D^(L)) R, Sc = (A - D^(L))^T R (either may be
+// NULL) by the exact-split product.  The digits of A are made per call in row
+// chunks of at most kXsCap bytes; keep: storage that outlives the call
+// (a compression of a generated source, whose entries then are evaluated once).
+// False: nothing done (too small, or no memory for the digits); the caller
+// takes the FP64 kernel.
+hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long ldr, double* Sr, double* Sc,
+                     long long lds, XsKeep* keep, int* err, bool* done) {
+  *done = false;
+  const int n = s.n;
+  if (n < 192 || w <= 0 || n > (1 << 22) || (n + 127) / 128 > 65535) return HSS_OK;
+  cudaStream_t st = c.st;
+  const bool sym = symmetric_source(s);
+  struct Orient { int trans; double* S; double* dup; };
+  std::vector<Orient> O;
+  if (sym && Sr && Sc) O.push_back({0, Sr, Sc});
+  else {
+    if (Sr) O.push_back({0, Sr, nullptr});
+    if (Sc) O.push_back({sym ? 0 : 1, Sc, nullptr});
+  }
+  if (O.empty()) { *done = true; return HSS_OK; }
+  const int nkt = (n + XS_BK - 1) / XS_BK, nrb = (n + XS_TM - 1) / XS_TM, ncb = (w + XS_TN - 1) / XS_TN;
+  const size_t row_bytes = (size_t)nkt * xs_tile_bytes(0);
+  // row blocks of every orientation per launch
+  const int no = (int)O.size();
+  const int chunk = keep ? nrb : (int)std::max<size_t>(1, std::min<size_t>((size_t)nrb, kXsCap / (row_bytes * no)));
+  const int g = xs_seg_ktiles({{(long long)no * std::min(chunk, nrb) * ncb, nkt}});
+  const int nseg = (nkt + g - 1) / g;
+  const int nchunk = (nrb + chunk - 1) / chunk;
+  // zeroed region: flag, maxima of A (both orientations) and R, counts, tile
+  // counters and partial sums of every launch
+  size_t nz = 8;
+  const size_t oea = nz; nz += 2 * (size_t)n;
+  const size_t oeb = nz; nz += w;
+  const size_t onb = nz; nz += w;
+  const size_t per_cnt = (size_t)chunk * ncb;
+  const size_t ocnt = nz; nz += per_cnt * no * nchunk;
+  const size_t per_ws = nseg > 1 ? per_cnt * 2 * XS_TM * XS_TN : 0;
+  const size_t zw = Scratch::rnd(sizeof(unsigned) * nz);
+  const size_t zb = zw + sizeof(unsigned long long) * per_ws * no;
+  const size_t bB = (size_t)ncb * nkt * xs_tile_bytes(1);
+  if (c.xz.ensure(zb, st) != cudaSuccess ||
+      c.xp.ensure(bB + (keep ? 0 : chunk * row_bytes * no), st) != cudaSuccess) {
+    cudaGetLastError();   // no memory for the digits
+    return HSS_OK;
+  }
+  unsigned* z = (unsigned*)c.xz.p;
+  unsigned long long* ws = (unsigned long long*)(c.xz.p + zw);
+  unsigned char* pB = (unsigned char*)c.xp.p;
+  unsigned char* pA = pB + bB;
+  unsigned* ea = keep ? keep->ea : z + oea;
+  std::vector<GemmJob> jobs;
+  GemmJob jr = gemm_job();   // R alone: maxima and digits
+  jr.M = 0; jr.N = w; jr.K = n;
+  jr.B = opnd(R, 1, ldr);
+  jr.eb = z + oeb; jr.nb = z + onb; jr.pb = pB; jr.nkt = nkt;
+  jobs.push_back(jr);
+  std::vector<int> pre;   // unit prefixes: R's maxima, R's digits, the products of every chunk
+  pre.push_back(0); pre.push_back(xs_max_units(0, w, n));
+  pre.push_back(0); pre.push_back(xs_pack_units(0, w, n));
+  for (int q = 0; q < nchunk; ++q) {
+    const int r0 = q * chunk * XS_TM, rows = std::min(n - r0, chunk * XS_TM);
+    int units = 0;
+    pre.push_back(0);
+    for (int o = 0; o < no; ++o) {
+      GemmJob j = jr;
+      j.M = rows;
+      j.C = O[o].S + (long long)r0 * lds; j.c_rs = lds; j.c_cs = 1;
+      j.dup = O[o].dup ? O[o].dup + (long long)r0 * lds : nullptr;
+      j.ea = ea + (size_t)O[o].trans * n + r0;
+      j.pa = keep ? keep->pa[O[o].trans] : pA + (size_t)o * chunk * row_bytes;
+      j.nseg = nseg;
+      j.cnt = z + ocnt + (size_t)(q * no + o) * per_cnt;
+      j.ws = ws + (size_t)o * per_ws;
+      jobs.push_back(j);
+      units += (rows + XS_TM - 1) / XS_TM * ncb * nseg;
+      pre.push_back(units);
+    }
+  }
+  Staging sg;
+  const size_t oj = sg.put(jobs.data(), jobs.size() * sizeof(GemmJob));
+  const size_t op = sg.put(pre.data(), pre.size() * sizeof(int));
+  char* dev;
+  CKS(sg.send(c, &dev));
+  const GemmJob* dj = (const GemmJob*)(dev + oj);
+  const int* dp = (const int*)(dev + op);
+  CK(cudaMemsetAsync(c.xz.p, 0, zb, st));
+  bool need_t = false;
+  for (auto& x : O) need_t = need_t || x.trans;
+  const bool fresh = !keep || !keep->have;
+  if (fresh) {
+    if (keep) CK(cudaMemsetAsync(keep->ea, 0, sizeof(unsigned) * 2 * (size_t)n, st));
+    CK(launch_xs_src_max(s, ea, need_t ? ea + n : nullptr, st));
+    c.launches++;
+  }
+  CK(launch_xs_max(dj, dp, 1, pre[1], st));
+  CK(launch_xs_pack(dj, dp + 2, 1, pre[3], st));
+  c.launches += 2;
+  for (int q = 0; q < nchunk; ++q) {
+    const GemmJob* hj = jobs.data() + 1 + (size_t)q * no;
+    for (int o = 0; o < no && fresh; ++o) {
+      CK(launch_xs_src_pack(s, O[o].trans, q * chunk * XS_TM, hj[o].M, ea + (size_t)O[o].trans * n, hj[o].pa, st));
+      c.launches++;
+    }
+    if (nseg > 1 && q > 0) CK(cudaMemsetAsync(ws, 0, sizeof(unsigned long long) * per_ws * no, st));
+    const size_t op_q = 4 + (size_t)q * (no + 1);
+    CK(launch_xs_mm(dj + 1 + (size_t)q * no, dp + op_q, no, pre[op_q + no], (int*)z, err ? err : (int*)z + 1, st));
+    c.launches++;
+  }
+  if (keep) keep->have = true;
+  // operands that the digits cannot hold: the FP64 kernel instead
+  CK(launch_sample_fp64(s, w, R, ldr, Sr, Sc, lds, st, (const int*)z));
+  c.launches += (Sr ? 1 : 0) + (Sc ? 1 : 0);
+  *done = true;
+  return HSS_OK;
+}
+
+// Storage for the digits of a generated source over a whole compression
+// (made at its first sampling pass): up to kXsKeep bytes for all matrices of
+// the call; NULL: not kept, made again by every pass.
+XsKeep* xs_keep(Ctx& c, hss_matrix_s* H) {
+  if (H->src.kind != HSS_SRC_GAUSS && H->src.kind != HSS_SRC_LAPLACE) return nullptr;
+  if (H->xs.pa[0]) return &H->xs;
+  const size_t one = (size_t)((H->n + XS_TM - 1) / XS_TM) * ((H->n + XS_BK - 1) / XS_BK) * xs_tile_bytes(0);
+  const size_t need = one + Scratch::rnd(sizeof(unsigned) * 2 * (size_t)H->n);
+  if (H->n < 192 || c.xs_kept + need > kXsKeep) return nullptr;
+  char* p = nullptr;
+  if (dmalloc_async(&p, need, c.st) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  c.xs_kept += need;
+  H->xs.pa[0] = H->xs.pa[1] = (unsigned char*)p;   // a point kernel's two orientations are one
+  H->xs.ea = (unsigned*)(p + one);
+  return &H->xs;
+}
+
 // S^r = A R, S^c = A^T R for columns [c0, c1) of matrix H, the leaf diagonal
 // blocks removed (eq. sample_off_diag); the non-finite check writes the
 // matrix's flag.  No read-back here: sample_check reads every matrix's flags
@@ -845,8 +1040,13 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
     CK(cudaFreeAsync(T, st));
   } else if (H->o.precision == HSS_PREC_FP64) {
     CK(c.timer.mark(PH_SAMPLE, st));
-    CK(launch_sample_fp64(s, w, Rc, n, H->Sg_r + c0, H->sym ? nullptr : H->Sg_c + c0, H->dmax, st));
-    c.launches += norient;
+    double* Sc = H->sym ? nullptr : H->Sg_c + c0;
+    bool xs = false;
+    CKS(xs_sample(c, s, w, Rc, n, H->Sg_r + c0, Sc, H->dmax, xs_keep(c, H), c.d_flag + 5, &xs));
+    if (!xs) {
+      CK(launch_sample_fp64(s, w, Rc, n, H->Sg_r + c0, Sc, H->dmax, st));
+      c.launches += norient;
+    }
     c.sample_launches += norient;
     H->st.sample_launches += norient;
   } else if (use_packed(H)) {
@@ -932,7 +1132,8 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
 // One read-back of the sampling flags of every matrix after a sampling round.
 hss_status sample_check(Ctx& c, const std::vector<hss_matrix_s*>& Hs) {
   CKS(readback(c, c.d_flag, sizeof(int) * c.nflag));
-  if (c.h_pinned[1]) return fail(HSS_ERR_TIMEOUT, "tensor-core sampling gave up waiting (code %d)", c.h_pinned[1]);
+  for (int i : {1, 5})
+    if (c.h_pinned[i]) return fail(HSS_ERR_TIMEOUT, "tensor-core sampling gave up waiting (code %d)", c.h_pinned[i]);
   for (hss_matrix_s* H : Hs)
     if (c.h_pinned[8 + H->slot])
       return fail(HSS_ERR_NONFINITE, "NaN or Inf in the random samples (columns up to %d)", H->d);
@@ -1860,10 +2061,16 @@ hss_status compress_all(Ctx& c, const std::vector<const hss_source*>& A, const s
       CK(cudaFreeAsync(H->toep_terms, c.st));
       H->toep_terms = nullptr;
     }
+    if (H->xs.pa[0]) {
+      CK(cudaFreeAsync(H->xs.pa[0], c.st));
+      H->xs = XsKeep();
+    }
     if (!H->converged) CKS(keep_dense_blocks(c, H));
   }
-  CKS(readback(c, c.d_flag + 3, sizeof(int)));
-  if (c.h_pinned[0]) return fail(HSS_ERR_TIMEOUT, "tensor-core tile product gave up waiting (code %d)", c.h_pinned[0]);
+  CKS(readback(c, c.d_flag + 3, 3 * sizeof(int)));
+  for (int i : {0, 2})
+    if (c.h_pinned[i])
+      return fail(HSS_ERR_TIMEOUT, "tensor-core tile product gave up waiting (code %d)", c.h_pinned[i]);
   double ph[PH_N];
   c.timer.sum(ph, PH_N);
   for (size_t i = 0; i < Hs.size(); ++i) {
@@ -2707,9 +2914,13 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   CK(cudaMemcpyAsync(d_lid, lid.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
   SrcDev s = make_src(*A, d_lid);
   if (precision == HSS_PREC_FP64) {
-    CK(launch_sample_fp64(s, ncols, R, ldr, Sr, Sc, lds, st));
-    CK(cudaFreeAsync(d_lid, st));
-    return HSS_OK;
+    Ctx c(st);
+    bool xs = false;
+    hss_status e = xs_sample(c, s, ncols, R, ldr, Sr, Sc, lds, nullptr, nullptr, &xs);
+    if (e == HSS_OK && !xs && launch_sample_fp64(s, ncols, R, ldr, Sr, Sc, lds, st) != cudaSuccess)
+      e = fail(HSS_ERR_CUDA, "FP64 sampling launch failed");
+    cudaFreeAsync(d_lid, st);
+    return e;
   }
   // mixed forms: R rounded once to the tensor format, K split with atomics
   double* Rr = nullptr;

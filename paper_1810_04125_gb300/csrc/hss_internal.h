@@ -17,7 +17,7 @@ struct SrcDev {
   const double* b;
   long long ld;
   double p0, p1;
-  const int* leaf_id;   // n entries, nondecreasing
+  const int* leaf_id;   // n entries (leaves numbered level by level)
 };
 
 // Entry A(i, j) in FP64 (the definitions of HSS_SRC_*).
@@ -76,6 +76,17 @@ struct GemmJob {
   unsigned char* pa;
   unsigned char* pb;
   int nkt;
+  // exact-split form (k_gemm_xs.cu): the largest |element| (high word) of
+  // every row of A and column of B, the number of elements of a column of B
+  // near its largest, and, when K is split over nseg CTAs, the 128-bit partial
+  // sums and arrival counter of every output tile; dup: second copy of C
+  unsigned* ea;
+  unsigned* eb;
+  unsigned* nb;
+  unsigned long long* ws;
+  unsigned* cnt;
+  double* dup;
+  int nseg;
 };
 // One tile of an operand to pack: job, operand (0 = A, 1 = B), row tile, k tile.
 struct PackUnit { int job, which, tile, kt; };
@@ -183,8 +194,10 @@ struct EntryNode {
 // Launch wrappers (return cudaError_t of the launch).
 cudaError_t launch_random_normal(unsigned long long seed, int n, int col0, int ncols,
                                  double* R, long long ldr, int round_mode, cudaStream_t st);
+// only_if: device flag (may be null); the launch does nothing while it is 0
 cudaError_t launch_sample_fp64(const SrcDev& src, int ncols, const double* R, long long ldr,
-                               double* Sr, double* Sc, long long lds, cudaStream_t st);
+                               double* Sr, double* Sc, long long lds, cudaStream_t st,
+                               const int* only_if = nullptr);
 // tcgen05 mixed-precision sampling with entries generated in the kernel
 // (k_sample_tc.cu); Rp is R packed by launch_pack_r; *used_atomic tells
 // whether S had to be zeroed beforehand (K split across CTAs).  toep: for a
@@ -213,6 +226,30 @@ cudaError_t launch_round_copy(const double* in, long long ldin, double* out, lon
 cudaError_t launch_extract(const ExtractJob* jobs_dev, int njobs, int max_tiles, cudaStream_t st);
 cudaError_t launch_gemm(const GemmJob* jobs_dev, const GemmTile* tiles_dev, int ntiles,
                         cudaStream_t st);
+// FP64 products on the tensor cores from operands cut into eight 8-bit
+// digits (k_gemm_xs.cu): tiles of XS_TM x XS_TN, k-tiles of XS_BK.  Every
+// launch finds the job of a CTA in a prefix array (njobs + 1 entries: maxima
+// units, pack units, tile segments).  xs_max_units / xs_pack_units: CTAs a
+// job takes in the first two launches.
+constexpr int XS_TM = 128, XS_TN = 64, XS_BK = 32;
+size_t xs_tile_bytes(int which);            // packed bytes per k-tile of A (0) or B (1)
+int xs_max_units(int M, int N, int K);
+int xs_pack_units(int M, int N, int K);
+cudaError_t launch_xs_max(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, cudaStream_t st);
+cudaError_t launch_xs_pack(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, cudaStream_t st);
+// flag == nullptr: a tile whose operands the digits cannot hold (non-finite,
+// or a column of B of uneven magnitude) is computed by FP64 FMAs in the same
+// launch; otherwise it is left out and *flag set (for the sampling, whose A
+// has no operand view).
+cudaError_t launch_xs_mm(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, int* flag, int* err,
+                         cudaStream_t st);
+// The sampling operand A - D^(L) (trans 0) or its transpose (1), rows
+// [row0, row0 + rows): the largest entry of every row (zeroed by the caller),
+// of both orientations in one read when out_t is given, and the digits
+// (ea: the maxima of all n rows of that orientation).
+cudaError_t launch_xs_src_max(const SrcDev& src, unsigned* out, unsigned* out_t, cudaStream_t st);
+cudaError_t launch_xs_src_pack(const SrcDev& src, int trans, int row0, int rows, const unsigned* ea,
+                               unsigned char* out, cudaStream_t st);
 // The same contract with the product on tcgen05 tensor cores, operands split
 // into three TF32 terms (k_gemm_tc.cu): tiles of 128 rows x tile_n columns
 // (gemm_tc_tile_n); *err records a wait that gave up.

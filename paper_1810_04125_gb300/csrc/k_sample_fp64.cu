@@ -20,7 +20,9 @@ constexpr int BM = 64, BN = 64, BK = 16;
 
 template <bool TRANS>
 __global__ void __launch_bounds__(256) k_sample_fp64(SrcDev src, int ncols, const double* __restrict__ R,
-                                                     long long ldr, double* __restrict__ S, long long lds) {
+                                                     long long ldr, double* __restrict__ S, long long lds,
+                                                     const int* only_if) {
+  if (only_if && *only_if == 0) return;
   __shared__ double As[BK][BM + 2];
   __shared__ double Rs[BK][BN + 2];
   const int n = src.n;
@@ -80,12 +82,12 @@ __global__ void __launch_bounds__(256) k_sample_fp64(SrcDev src, int ncols, cons
 }  // namespace
 
 cudaError_t launch_sample_fp64(const SrcDev& src, int ncols, const double* R, long long ldr,
-                               double* Sr, double* Sc, long long lds, cudaStream_t st) {
+                               double* Sr, double* Sc, long long lds, cudaStream_t st, const int* only_if) {
   if (src.kind < HSS_SRC_DENSE || src.kind > HSS_SRC_LAPLACE) return cudaErrorInvalidValue;   // no entries on the device
   if (src.n <= 0 || ncols <= 0) return cudaSuccess;
   dim3 grid((src.n + BM - 1) / BM, (ncols + BN - 1) / BN);
-  if (Sr) k_sample_fp64<false><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sr, lds);
-  if (Sc) k_sample_fp64<true><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sc, lds);
+  if (Sr) k_sample_fp64<false><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sr, lds, only_if);
+  if (Sc) k_sample_fp64<true><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sc, lds, only_if);
   return cudaGetLastError();
 }
 
