@@ -602,6 +602,7 @@ GemmJob gemm_job() {
 constexpr size_t kXsCap = size_t(2) << 30;   // digits of the operands of one launch
 constexpr int kSms = 152;
 constexpr size_t kXsKeep = size_t(4) << 30;  // digits of generated sources kept over a compression
+constexpr double kXsMinUs = 30.0;            // FP64-pipe time from which the exact-split launches pay
 
 // k-tiles per CTA of launches whose tiles (count, k-tiles each) are given:
 // the split of K that takes the fewest waves x (k-tiles + the fixed cost of a
@@ -633,12 +634,122 @@ int xs_seg_ktiles(const std::vector<std::pair<long long, int>>& tiles) {
   return best;
 }
 
+// One launch set (maxima, digits, product) over jobs[b0..b1).
+hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs) {
+  const int nj = (int)jobs.size();
+  std::vector<std::pair<long long, int>> tl;
+  for (const GemmJob& j : jobs)
+    tl.push_back({(long long)((j.M + XS_TM - 1) / XS_TM) * ((j.N + XS_TN - 1) / XS_TN), (j.K + XS_BK - 1) / XS_BK});
+  const int g = xs_seg_ktiles(tl);
+  size_t nz = 8, np = 0;   // words of the zeroed region (word 0: the wait flag of calls without flags); packed bytes
+  std::vector<size_t> oea(nj), oeb(nj), onb(nj), ocnt(nj), ows(nj), opa(nj), opb(nj);
+  std::vector<int> pm(nj + 1, 0), pp(nj + 1, 0), pt(nj + 1, 0);
+  size_t nws = 0;
+  for (int i = 0; i < nj; ++i) {
+    GemmJob& j = jobs[i];
+    j.nkt = (j.K + XS_BK - 1) / XS_BK;
+    j.nseg = (j.nkt + g - 1) / g;
+    const size_t nrb = (j.M + XS_TM - 1) / XS_TM, ncb = (j.N + XS_TN - 1) / XS_TN;
+    oea[i] = nz; nz += j.M;
+    oeb[i] = nz; nz += j.N;
+    onb[i] = nz; nz += j.N;
+    ocnt[i] = nz; nz += nrb * ncb;
+    ows[i] = nws;
+    if (j.nseg > 1) nws += nrb * ncb * 2 * XS_TM * XS_TN;
+    opa[i] = np; np += nrb * j.nkt * xs_tile_bytes(0);
+    opb[i] = np; np += ncb * j.nkt * xs_tile_bytes(1);
+    pm[i + 1] = pm[i] + xs_max_units(j.M, j.N, j.K);
+    pp[i + 1] = pp[i] + xs_pack_units(j.M, j.N, j.K);
+    pt[i + 1] = pt[i] + (int)(nrb * ncb) * j.nseg;
+  }
+  const size_t zb = Scratch::rnd(sizeof(unsigned) * nz) + sizeof(unsigned long long) * nws;
+  CK(c.xz.ensure(zb, c.st));
+  CK(c.xp.ensure(np, c.st));
+  unsigned* z = (unsigned*)c.xz.p;
+  for (int i = 0; i < nj; ++i) {
+    GemmJob& j = jobs[i];
+    j.ea = z + oea[i];
+    j.eb = z + oeb[i];
+    j.nb = z + onb[i];
+    j.cnt = z + ocnt[i];
+    j.ws = (unsigned long long*)(c.xz.p + Scratch::rnd(sizeof(unsigned) * nz)) + ows[i];
+    j.pa = (unsigned char*)c.xp.p + opa[i];
+    j.pb = (unsigned char*)c.xp.p + opb[i];
+  }
+  Staging sg;
+  const size_t oj = sg.put(jobs.data(), jobs.size() * sizeof(GemmJob));
+  const size_t om = sg.put(pm.data(), sizeof(int) * (nj + 1));
+  const size_t op = sg.put(pp.data(), sizeof(int) * (nj + 1));
+  const size_t ot = sg.put(pt.data(), sizeof(int) * (nj + 1));
+  char* dev;
+  CKS(sg.send(c, &dev));
+  CK(cudaMemsetAsync(c.xz.p, 0, zb, c.st));
+  const GemmJob* dj = (const GemmJob*)(dev + oj);
+  CK(launch_xs_max(dj, (const int*)(dev + om), nj, pm[nj], c.st));
+  CK(launch_xs_pack(dj, (const int*)(dev + op), nj, pp[nj], c.st));
+  CK(launch_xs_mm(dj, (const int*)(dev + ot), nj, pt[nj], nullptr, c.d_flag ? c.d_flag + 5 : (int*)z, c.st));
+  c.launches += 3;
+  return HSS_OK;
+}
+
+size_t xs_job_bytes(const GemmJob& j) {
+  const size_t nkt = (j.K + XS_BK - 1) / XS_BK;
+  return nkt * ((size_t)((j.M + XS_TM - 1) / XS_TM) * xs_tile_bytes(0) +
+                (size_t)((j.N + XS_TN - 1) / XS_TN) * xs_tile_bytes(1));
+}
+
 // Runs a list of tile-product jobs (one launch).  tc_prec: HSS_PREC_FP64 for
 // the FP64 tile kernel; a mixed precision sends the products that only form
 // samples (merge, reduce, test projections) to the tensor-core kernel.
-hss_status run_gemms(Ctx& c, const std::vector<GemmJob>& jobs, const char* tag = "gemm",
+hss_status run_gemms(Ctx& c, const std::vector<GemmJob>& all_jobs, const char* tag = "gemm",
                      int tc_prec = HSS_PREC_FP64) {
   const bool tc = tc_prec != HSS_PREC_FP64;
+  // FP64: the products go to the exact-split kernel where the FP64 pipe would
+  // take longer than that kernel's launches: a 64 x 64 tile costs the pipe
+  // 1.07 us per unit of K on one SM, whatever part of the tile is in use.
+  std::vector<GemmJob> rest;
+  bool split = false;
+  if (!tc) {
+    double pipe = 0.0;
+    int kmx = 0;
+    for (const GemmJob& j : all_jobs) {
+      if (j.M <= 0 || j.N <= 0 || j.K <= 0 || xs_job_bytes(j) > kXsCap) continue;
+      pipe += 1.07 * j.K * ((j.M + 63) / 64) * ((j.N + 63) / 64);
+      kmx = std::max(kmx, j.K);
+    }
+    if (std::max(1.07 * kmx, pipe / kSms) > kXsMinUs) {
+      split = true;
+      if (c.trace) CK(cudaEventRecord(c.trace_ev[0], c.st));
+      std::vector<GemmJob> xs;
+      size_t bytes = 0;
+      double flop = 0.0;
+      for (const GemmJob& j : all_jobs) {
+        if (j.M <= 0 || j.N <= 0) continue;
+        if (j.K < 8 || xs_job_bytes(j) > kXsCap) {
+          rest.push_back(j);
+          continue;
+        }
+        if (bytes + xs_job_bytes(j) > kXsCap) {
+          CKS(xs_launch(c, std::move(xs)));
+          xs.clear();
+          bytes = 0;
+        }
+        xs.push_back(j);
+        bytes += xs_job_bytes(j);
+        flop += 2.0 * j.M * j.N * j.K;
+      }
+      const size_t nxs = xs.size();
+      if (!xs.empty()) CKS(xs_launch(c, std::move(xs)));
+      if (c.trace) {
+        CK(cudaEventRecord(c.trace_ev[1], c.st));
+        CK(cudaEventSynchronize(c.trace_ev[1]));
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, c.trace_ev[0], c.trace_ev[1]);
+        fprintf(stderr, "[hss trace] %s exact-split jobs %zu  %.3f ms  %.1f GFLOP/s\n", tag, nxs, ms, flop / (ms * 1e6));
+      }
+    }
+  }
+  const std::vector<GemmJob>& jobs = split ? rest : all_jobs;
   int max_n = 0;
   for (const GemmJob& j : jobs) max_n = std::max(max_n, j.N);
   const int tm = tc ? 128 : 64, tn = tc ? gemm_tc_tile_n(max_n) : 64;
