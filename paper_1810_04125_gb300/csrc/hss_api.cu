@@ -353,7 +353,7 @@ struct hss_matrix_s {
   int* iota = nullptr;
   int d_final = 0, n_adapt = 0, converged = 0;
   int pack_decided = -1;   // mixed forms, generated A: packed tiles (1) or not (0)
-  bool sym = false;        // symmetric option: the column side mirrors the row side
+  bool sym = false;        // the column side is a copy of the row side (find_symmetric)
   void* packA = nullptr;   // packed tensor-core tiles of a dense A (during compress)
   XsKeep xs;               // digits of a generated source (during compress, plain form)
   void* toep_terms = nullptr; // a Toeplitz source's diagonals split into terms (during compress)
@@ -407,7 +407,8 @@ struct DevBuf {
 //   d_flag[0..7]: [1] tensor-core sampling wait, [2] QRCP barrier,
 //   [3] tensor-core tile product wait, [4] Incrementing test barrier,
 //   [5] exact-split product wait;
-//   d_flag[8 + i]: non-finite samples of matrix i.
+//   d_flag[8 + i]: non-finite samples of matrix i;
+//   d_flag[8 + count + i]: a dense matrix i that is not symmetric.
 struct Ctx {
   cudaStream_t st = nullptr;
   Scratch scratch;
@@ -444,7 +445,7 @@ struct Ctx {
     if (h_pinned) cudaFreeHost(h_pinned);
   }
   hss_status flags(int nmat) {
-    nflag = 8 + std::max(nmat, 0);
+    nflag = 8 + 2 * std::max(nmat, 0);
     CK(dmalloc_async((void**)&d_flag, sizeof(int) * nflag, st));
     CK(cudaMemsetAsync(d_flag, 0, sizeof(int) * nflag, st));
     return HSS_OK;
@@ -464,6 +465,15 @@ SrcDev make_src(const hss_source& s, const int* leaf_id) {
   d.p1 = s.p1;
   d.leaf_id = leaf_id;
   return d;
+}
+
+// A = A^T by the definition of the source: the point kernels depend on
+// |x_i - x_j| only (entry (i, j) and (j, i) are the same bits), a Toeplitz
+// matrix has one table for both halves.
+template <class S>
+bool symmetric_source(const S& s) {
+  return s.kind == HSS_SRC_GAUSS || s.kind == HSS_SRC_LAPLACE ||
+         (s.kind == HSS_SRC_TOEPLITZ && (s.a == s.b || !s.b));
 }
 
 hss_status check_source(const hss_source* A) {
@@ -963,13 +973,6 @@ bool use_packed(hss_matrix_s* H) {
   return H->pack_decided == 1;
 }
 
-// A = A^T by the definition of the source: the point kernels depend on
-// |x_i - x_j| only (entry (i, j) and (j, i) are the same bits), a Toeplitz
-// matrix has one table for both halves.
-bool symmetric_source(const SrcDev& s) {
-  return s.kind == HSS_SRC_GAUSS || s.kind == HSS_SRC_LAPLACE || (s.kind == HSS_SRC_TOEPLITZ && s.a == s.b);
-}
-
 // The FP64 sampling Sr = (A - D^(L)) R, Sc = (A - D^(L))^T R (either may be
 // NULL) by the exact-split product.  The digits of A are made per call in row
 // chunks of at most kXsCap bytes; keep: storage that outlives the call
@@ -1224,7 +1227,7 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
     CK(cudaFreeAsync(packR, st));
   }
   CK(c.timer.mark(PH_RNG, st));
-  H->st.flop_sample += 2.0 * norient * (double)n * (double)n * (double)w;
+  H->st.flop_sample += (H->o.symmetric ? 2.0 : 4.0) * (double)n * (double)n * (double)w;
   // algorithmic bytes of the sampling kernels: A read once per orientation
   // (FP64: 8 B per entry; packed TF32x2: 8 B; packed BF16x3: 6 B), R read,
   // S written
@@ -2048,7 +2051,7 @@ hss_status keep_dense_blocks(Ctx& c, hss_matrix_s* H) {
 
 // Everything a compression needs before its first pass: tree, leaf labels,
 // sample and R buffers, and (with a user operator) the packed leaf blocks D.
-hss_status setup(Ctx& c, const hss_source* A, const hss_opts* o, hss_matrix_s* H, ExtractSet& leafD) {
+hss_status setup(Ctx& c, const hss_source* A, const hss_opts* o, hss_matrix_s* H, bool sym, ExtractSet& leafD) {
   const int n = A->n;
   H->n = n;
   H->o = *o;
@@ -2075,7 +2078,7 @@ hss_status setup(Ctx& c, const hss_source* A, const hss_opts* o, hss_matrix_s* H
   H->leaf_id = (int*)H->arena.alloc(sizeof(int) * n);
   H->iota = (int*)H->arena.alloc(sizeof(int) * n);
   H->Sg_r = (double*)H->arena.alloc(sizeof(double) * nd);
-  H->sym = o->symmetric != 0;
+  H->sym = sym;
   H->Sg_c = H->sym ? H->Sg_r : (double*)H->arena.alloc(sizeof(double) * nd);
   const bool mixed = o->precision != HSS_PREC_FP64;
   H->own_R = (o->R == nullptr) || mixed;
@@ -2122,6 +2125,40 @@ hss_status setup(Ctx& c, const hss_source* A, const hss_opts* o, hss_matrix_s* H
   return HSS_OK;
 }
 
+// Which matrices are compressed on the row side alone, the column side being
+// its copy: those of the symmetric option, and in the plain form those that
+// are symmetric, where both sides are the same computation on the same bits
+// (Sc = Sr, so the same pivots, bases and reduced samples; B21 = B12^T).  A
+// generated source is symmetric by its definition; a dense one is compared
+// with its transpose, one read of A against one read per pass and side.  The
+// mixed forms keep their two sides: with the other split of the CTAs over the
+// sides the last bits of their QR change, and their samples, equal to 1e-7
+// only, turn that into other pivots.  A user operator is asked for both
+// products.
+hss_status find_symmetric(Ctx& c, const std::vector<const hss_source*>& A, const std::vector<const hss_opts*>& O,
+                          std::vector<char>& sym) {
+  const int m = (int)A.size();
+  sym.assign(m, 0);
+  bool any = false;
+  std::vector<char> dense(m, 0);
+  for (int i = 0; i < m; ++i) {
+    if (O[i]->symmetric) sym[i] = 1;
+    else if (O[i]->precision != HSS_PREC_FP64 || O[i]->op) continue;
+    else if (symmetric_source(*A[i])) sym[i] = 1;
+    else if (A[i]->kind == HSS_SRC_DENSE) {
+      CK(launch_asymmetric(A[i]->a, A[i]->ld, A[i]->n, c.d_flag + 8 + m + i, c.st));
+      c.launches++;
+      dense[i] = 1;
+      any = true;
+    }
+  }
+  if (!any) return HSS_OK;
+  CKS(readback(c, c.d_flag, sizeof(int) * c.nflag));
+  for (int i = 0; i < m; ++i)
+    if (dense[i] && !c.h_pinned[8 + m + i]) sym[i] = 1;
+  return HSS_OK;
+}
+
 // HSSCompressAdaptive (Algorithm 3) for a list of matrices in lockstep: all
 // first samples, then passes of the tree sweep (run_pass) over the matrices
 // that are not done, each followed by the growth of the sample of those
@@ -2133,9 +2170,11 @@ hss_status compress_all(Ctx& c, const std::vector<const hss_source*>& A, const s
   CKS(c.flags((int)Hs.size()));
   CK(c.timer.mark(PH_OTHER, c.st));
   ExtractSet leafD;
+  std::vector<char> sym;
+  CKS(find_symmetric(c, A, O, sym));
   for (size_t i = 0; i < Hs.size(); ++i) {
     Hs[i]->slot = (int)i;
-    CKS(setup(c, A[i], O[i], Hs[i], leafD));
+    CKS(setup(c, A[i], O[i], Hs[i], sym[i] != 0, leafD));
   }
   if (!leafD.per.empty()) {
     CK(c.timer.mark(PH_MERGE, c.st));

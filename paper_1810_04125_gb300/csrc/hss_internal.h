@@ -305,6 +305,9 @@ cudaError_t launch_inc_group(const IncJob* jobs_dev, const int2* map_dev, int nc
                              cudaStream_t st);
 cudaError_t launch_nonfinite(const double* S, long long lds, int n, int c0, int c1,
                              int* flag, cudaStream_t st);
+// *flag |= 1 when the dense matrix a (col-major, ld) is not its transpose bit
+// for bit
+cudaError_t launch_asymmetric(const double* a, long long ld, int n, int* flag, cudaStream_t st);
 cudaError_t launch_identity_block(double* X, int n, int c0, int w, cudaStream_t st);
 cudaError_t launch_gather_int(const GatherJob* jobs_dev, int njobs, int max_cnt, cudaStream_t st);
 // entries of a compressed handle (k_entries.cu); err: 1 = index out of

@@ -101,7 +101,45 @@ __global__ void k_identity_block(double* X, int n, int c0, int w) {
   X[e] = (i == c0 + j) ? 1.0 : 0.0;
 }
 
+// *flag |= 1 when some A(i, j) and A(j, i) differ in their bits.  A CTA
+// compares the 64 x 64 tiles (bi, bj) and (bj, bi); one read of A (n = 8192:
+// 0.1 ms), and next to none once a difference has been found.
+__global__ void __launch_bounds__(256) k_asymmetric(const double* __restrict__ a, long long ld, int n,
+                                                    int* flag) {
+  __shared__ unsigned long long t[64][65];
+  const int bi = blockIdx.x, bj = blockIdx.y;
+  if (bi > bj || *(volatile int*)flag) return;
+  const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+  const unsigned long long* p = (const unsigned long long*)a;
+  unsigned long long v[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int i = 64 * bi + tx, j = 64 * bj + ty + 4 * q;
+    v[q] = i < n && j < n ? p[(long long)i + (long long)j * ld] : 0ull;
+  }
+#pragma unroll
+  for (int q = 0; q < 16; ++q) t[ty + 4 * q][tx] = v[q];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int i = 64 * bj + tx, j = 64 * bi + ty + 4 * q;
+    v[q] = i < n && j < n ? p[(long long)i + (long long)j * ld] : 0ull;
+  }
+  __syncthreads();
+  int diff = 0;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) diff |= v[q] != t[tx][ty + 4 * q] ? 1 : 0;
+  if (__syncthreads_or(diff) && threadIdx.x == 0) atomicOr(flag, 1);
+}
+
 }  // namespace
+
+cudaError_t launch_asymmetric(const double* a, long long ld, int n, int* flag, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  const unsigned nb = (unsigned)((n + 63) / 64);
+  if (nb > 65535u) return cudaErrorInvalidValue;
+  k_asymmetric<<<dim3(nb, nb), 256, 0, st>>>(a, ld, n, flag);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_identity_block(double* X, int n, int c0, int w, cudaStream_t st) {
   const long long tot = (long long)n * w;
