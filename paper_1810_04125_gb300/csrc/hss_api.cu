@@ -334,7 +334,27 @@ struct XsKeep {
 
 }  // namespace
 
+// What the products and the entry extraction of a handle read besides its
+// generators, laid out on the device at the first such call and kept (in the
+// handle's arena) until the handle is freed: the nodes with the inverse pivot
+// orders, the leaf of every index, and for H X and H^T X the task lists of
+// every phase (first task, count, 16-row tiles of its largest).
+struct ProdPlan {
+  bool ready = false;
+  EntryNode* nodes = nullptr;
+  int* leaf_of = nullptr;
+  int kcap = 1;
+  const ProdTask* tasks[2] = {nullptr, nullptr};
+  struct Phase { int first, count, tiles; };
+  std::vector<Phase> phases[2];
+  size_t rows[2] = {0, 0};   // buffer rows of a product
+  double elems = 0.0;        // generator elements read by a product
+  int sets = 0;              // of its phases, those with sums of 8 terms or more
+};
+
 struct hss_matrix_s {
+  std::mutex plan_mu;
+  ProdPlan plan;
   int n = 0, dmax = 0, device = 0;
   hss_opts o{};
   hss_source src{};
@@ -855,7 +875,9 @@ hss_status run_gemms(Ctx& c, const std::vector<GemmJob>& all_jobs, const char* t
                       c.d_flag + 3, c.st));
     c.launches++;
   } else {
-    CK(launch_gemm((const GemmJob*)(dev + oj), (const GemmTile*)(dev + ot), (int)tiles.size(), c.st));
+    bool copies = true;
+    for (const GemmJob& j : jobs) copies = copies && j.K == 0;
+    CK(launch_gemm((const GemmJob*)(dev + oj), (const GemmTile*)(dev + ot), (int)tiles.size(), copies, c.st));
     c.launches++;
   }
   if (c.trace) {
@@ -2752,6 +2774,217 @@ hss_status hss_to_dense(hss_matrix H, double* out, long long ld, void* stream) {
   return HSS_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The tasks of H X (tr = false) or H^T X, phase by phase (up level max .. 1,
+// down level 1 .. max, leaves).
+void prod_tasks(const hss_matrix_s* H, bool tr, const std::vector<const int*>& ipr, const std::vector<const int*>& ipc,
+                std::vector<ProdTask>& tasks, std::vector<ProdPlan::Phase>& phases, size_t* rows, double* elems, int* sets) {
+  const int nn = (int)H->nodes.size();
+  auto in_side = [&](const Node& t) -> const Side& { return tr ? t.r : t.c; };
+  auto out_side = [&](const Node& t) -> const Side& { return tr ? t.c : t.r; };
+  const std::vector<const int*>& ipo = tr ? ipc : ipr;   // inverse pivots of the out side
+  std::vector<int> ox(nn, 0), oy(nn, 0);
+  int tot = 0;
+  for (int i = 1; i < nn; ++i) {
+    ox[i] = tot; tot += in_side(H->nodes[i]).k;
+    oy[i] = tot; tot += out_side(H->nodes[i]).k;
+  }
+  *rows = (size_t)tot;
+  *elems = 0.0;
+  *sets = 0;
+  int most = 0, kmax = 0, k2max = 0;
+  auto put = [&](ProdTask& t, int n) {
+    t.rows = n;
+    *elems += (double)n * (t.K + t.k2);
+    most = std::max(most, n);
+    kmax = std::max(kmax, t.K);
+    k2max = std::max(k2max, t.k2);
+    tasks.push_back(t);
+  };
+  size_t first = tasks.size();
+  auto end_phase = [&]() {
+    if (tasks.size() > first) phases.push_back({(int)first, (int)(tasks.size() - first), (most + 15) / 16});
+    first = tasks.size();
+    *sets += (kmax >= 8 ? 1 : 0) + (k2max >= 8 ? 1 : 0);
+    most = kmax = k2max = 0;
+  };
+  for (int lev = H->max_level; lev >= 1; --lev) {
+    for (int id : H->by_level[lev]) {
+      const Node& t = H->nodes[id];
+      const Side& s = in_side(t);
+      if (s.k <= 0) continue;
+      ProdTask p;
+      memset(&p, 0, sizeof p);
+      p.M = s.X; p.ld = s.k; p.K = s.m - s.k;
+      p.gather = s.piv + s.k;
+      p.in_lo = t.leaf ? t.lo : -1;
+      if (!t.leaf) { p.in0 = ox[t.ch[0]]; p.in1 = ox[t.ch[1]]; p.split = in_side(H->nodes[t.ch[0]]).k; }
+      p.out_lo = -1;
+      p.self = s.piv;
+      p.out = ox[id];
+      put(p, s.k);
+    }
+    end_phase();
+  }
+  for (int lev = 1; lev <= H->max_level; ++lev) {
+    for (int id : H->by_level[lev]) {
+      const Node& c = H->nodes[id];
+      const Side& s = out_side(c);
+      if (s.k <= 0) continue;
+      const Node& par = H->nodes[c.parent];
+      const bool a = par.ch[0] == id;   // the first child
+      const Node& na = H->nodes[par.ch[0]];
+      const Node& nb = H->nodes[par.ch[1]];
+      ProdTask p;
+      memset(&p, 0, sizeof p);
+      // y^_nu1 = B12 x^_nu2, y^_nu2 = B21 x^_nu1; transposed B21^T, B12^T
+      const bool b12 = a != tr;
+      p.M = b12 ? par.B12 : par.B21;
+      p.ld = std::max(b12 ? na.r.k : nb.r.k, 1);
+      p.trans = tr ? 1 : 0;
+      const int sib = par.ch[a ? 1 : 0];
+      p.K = in_side(H->nodes[sib]).k;
+      p.in_lo = -1;
+      p.in0 = p.in1 = ox[sib];
+      p.split = 0x7fffffff;
+      p.out_lo = -1;
+      const Side& u = out_side(par);
+      const bool nested = c.parent != 0 && u.k > 0;
+      if (nested) {
+        p.X2 = u.X; p.k2 = u.k; p.y2 = oy[c.parent];
+        p.pos = ipo[c.parent] + (a ? 0 : out_side(na).k);
+      }
+      p.out = oy[id];
+      put(p, s.k);
+    }
+    end_phase();
+  }
+  for (int id = 0; id < nn; ++id) {
+    const Node& t = H->nodes[id];
+    if (!t.leaf) continue;
+    ProdTask p;
+    memset(&p, 0, sizeof p);
+    p.M = t.D; p.ld = t.size; p.K = t.size; p.trans = tr ? 1 : 0;
+    p.in_lo = t.lo;
+    const Side& u = out_side(t);
+    const bool nested = id != 0 && u.k > 0;
+    if (nested) { p.X2 = u.X; p.k2 = u.k; p.y2 = oy[id]; p.pos = ipo[id]; }
+    p.out_lo = t.lo;
+    put(p, t.size);
+  }
+  end_phase();
+}
+
+// The handle's plan, made at the first call that needs it (from any thread;
+// it is complete on the device before the lock is given up, so that calls on
+// other streams may use it at once).  NULL when there is no memory for it, or
+// when it would have to be made during a stream capture.
+const ProdPlan* get_plan(hss_matrix_s* H, cudaStream_t st) {
+  std::lock_guard<std::mutex> lock(H->plan_mu);
+  ProdPlan& P = H->plan;
+  if (P.ready) return &P;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  const int nn = (int)H->nodes.size(), n = H->n;
+  size_t ninv = 0;
+  P.kcap = 1;
+  for (int id = 0; id < nn; ++id) {
+    const Node& t = H->nodes[id];
+    P.kcap = std::max(P.kcap, std::max(t.r.k, t.c.k));
+    if (id) ninv += (size_t)t.r.m + (size_t)t.c.m;
+  }
+  std::vector<ProdTask> tasks;
+  // device layout: error word, nodes, tasks | inverse pivots, leaf of every index
+  const size_t o_nodes = 256, o_task = o_nodes + Scratch::rnd(sizeof(EntryNode) * nn);
+  // (two passes: the tasks point into the inverse pivots, which follow them)
+  size_t ntask = 0;
+  auto make = [&](char* base) {
+    const size_t o_inv = o_task + Scratch::rnd(sizeof(ProdTask) * ntask);
+    std::vector<const int*> ipr(nn, nullptr), ipc(nn, nullptr);
+    const int* inv = (const int*)(base + o_inv);
+    for (int id = 1; id < nn; ++id) {
+      const Node& t = H->nodes[id];
+      if (t.state != HSS_COMPRESSED) continue;
+      ipr[id] = inv; inv += t.r.m;
+      ipc[id] = inv; inv += t.c.m;
+    }
+    tasks.clear();
+    size_t second = 0;
+    for (int tr = 0; tr < 2; ++tr) {
+      P.phases[tr].clear();
+      if (tr) second = tasks.size();
+      std::vector<ProdTask> q;
+      if (!H->partial) prod_tasks(H, tr != 0, ipr, ipc, q, P.phases[tr], &P.rows[tr], &P.elems, &P.sets);
+      tasks.insert(tasks.end(), q.begin(), q.end());
+    }
+    P.tasks[0] = (const ProdTask*)(base + o_task);
+    P.tasks[1] = P.tasks[0] + second;
+    return o_inv;
+  };
+  make((char*)nullptr);
+  ntask = tasks.size();
+  const size_t o_inv = o_task + Scratch::rnd(sizeof(ProdTask) * ntask);
+  const size_t o_leaf = o_inv + Scratch::rnd(sizeof(int) * std::max<size_t>(ninv, 1));
+  char* base = (char*)H->arena.alloc(o_leaf + sizeof(int) * n);
+  if (!base) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  make(base);
+  std::vector<char> host(o_inv, 0);
+  EntryNode* hn = (EntryNode*)(host.data() + o_nodes);
+  int* inv = (int*)(base + o_inv);
+  for (int id = 0; id < nn; ++id) {
+    const Node& t = H->nodes[id];
+    EntryNode& e = hn[id];
+    memset(&e, 0, sizeof e);
+    e.lo = t.lo; e.size = t.size; e.level = t.level; e.parent = t.parent; e.ch0 = t.ch[0]; e.ch1 = t.ch[1];
+    e.state = t.state;
+    e.D = t.D; e.B12 = t.B12; e.B21 = t.B21; e.F12 = t.F12; e.F21 = t.F21;
+    if (id && t.state == HSS_COMPRESSED) {
+      e.kr = t.r.k; e.kc = t.c.k; e.mr = t.r.m; e.mc = t.c.m;
+      e.pivr = t.r.piv; e.pivc = t.c.piv; e.Xr = t.r.X; e.Xc = t.c.X;
+      e.ipivr = inv; inv += t.r.m;
+      e.ipivc = inv; inv += t.c.m;
+    }
+  }
+  if (ntask) memcpy(host.data() + o_task, tasks.data(), sizeof(ProdTask) * ntask);
+  int herr = 1;
+  if (cudaMemcpyAsync(base, host.data(), o_inv, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaMemsetAsync(base + o_inv, 0xff, sizeof(int) * std::max<size_t>(ninv, 1), st) != cudaSuccess ||
+      launch_inv_piv((const EntryNode*)(base + o_nodes), nn, (int*)base, st) != cudaSuccess ||
+      launch_leaf_of((const EntryNode*)(base + o_nodes), nn, (int*)(base + o_leaf), st) != cudaSuccess ||
+      cudaMemcpyAsync(&herr, base, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess || herr) {
+    cudaGetLastError();
+    return nullptr;   // (pivots that are no permutation: the general paths report it)
+  }
+  P.nodes = (EntryNode*)(base + o_nodes);
+  P.leaf_of = (int*)(base + o_leaf);
+  P.ready = true;
+  return &P;
+}
+
+// Task by task, or by the exact-split products?  Tasks: 3 us a launch and the
+// FP64 pipe at 0.85 TFLOP/s; exact split: 60 us a set of launches (measured
+// 55 to 85) and 20 TFLOP/s.  Gaussian 8-D n = 4096 (12 sets): 16 columns 684
+// us against 650, 32 columns 1130 against 679; Gaussian 3-D n = 5003 (19
+// sets): 256 columns 793 us against 1650.
+bool prod_by_tasks(const ProdPlan& P, bool tr, int nrhs) {
+  const double flop = 2.0 * P.elems * nrhs;
+  return nrhs <= 65535 * 8 && 3.0 * P.phases[tr].size() + flop / 0.85e6 <= 60.0 * P.sets + flop / 20e6;
+}
+
+}  // namespace
+
+extern "C" {
+
 hss_status hss_matvec(hss_matrix H, int nrhs, const double* X, long long ldx, double* Y,
                       long long ldy, int transpose, void* stream) {
   if (!H || !X || !Y) return fail(HSS_ERR_ARG, "NULL argument");
@@ -2760,8 +2993,25 @@ hss_status hss_matvec(hss_matrix H, int nrhs, const double* X, long long ldx, do
   if (transpose != 0 && transpose != 1) return fail(HSS_ERR_ARG, "transpose must be 0 or 1");
   if (nrhs == 0) return HSS_OK;
   cudaStream_t st = (cudaStream_t)stream;
-  Ctx c(st);
   const bool tr = transpose != 0;
+  if (!H->partial) {
+    const ProdPlan* P = get_plan(H, st);
+    if (P && prod_by_tasks(*P, tr, nrhs)) {
+      double* buf = nullptr;
+      if (P->rows[tr]) CK(dmalloc_async(&buf, sizeof(double) * P->rows[tr] * nrhs, st));
+      cudaError_t e = cudaSuccess;
+      bool after = false;
+      for (auto& ph : P->phases[tr]) {
+        e = launch_prod(P->tasks[tr] + ph.first, ph.count, ph.tiles, after, nrhs, X, ldx, Y, ldy, buf, st);
+        after = true;
+        if (e != cudaSuccess) break;
+      }
+      if (buf) cudaFreeAsync(buf, st);
+      if (e != cudaSuccess) return fail(HSS_ERR_CUDA, "HSS product launch failed: %s", cudaGetErrorString(e));
+      return HSS_OK;
+    }
+  }
+  Ctx c(st);
   const int nn = (int)H->nodes.size();
   // H^T has the roles of U and V exchanged, D^T at the leaves and
   // B12' = B21^T, B21' = B12^T: the up-sweep runs with the "in" side
@@ -2926,64 +3176,32 @@ hss_status hss_get_entries(hss_matrix H, int nr, const int* I, int nc, const int
   if (nr == 0 || nc == 0) return HSS_OK;
   if (!I || !J || !out) return fail(HSS_ERR_ARG, "NULL argument");
   cudaStream_t st = (cudaStream_t)stream;
-  const int nn = (int)H->nodes.size(), n = H->n;
-  int kcap = 1;
-  size_t ninv = 0;
-  std::vector<int> leaf_of(n);
-  for (int id = 0; id < nn; ++id) {
-    const Node& t = H->nodes[id];
-    kcap = std::max(kcap, std::max(t.r.k, t.c.k));
-    if (id) ninv += (size_t)t.r.m + (size_t)t.c.m;
-    if (t.leaf)
-      for (int i = t.lo; i < t.lo + t.size; ++i) leaf_of[i] = id;
-  }
-  const int lp1 = H->max_level + 1;
+  const int n = H->n;
+  const ProdPlan* P = get_plan(H, st);
+  if (!P) return fail(HSS_ERR_NOMEM, "the index tables of the handle could not be laid out on the device");
+  const int kcap = P->kcap, lp1 = H->max_level + 1;
   // rows and columns in chunks whose path vectors take at most 512 MB each
   // (and at most 65535 columns: one grid row per column)
   const long long per = (long long)lp1 * kcap;
   const int chunk =
       (int)std::max<long long>(1, std::min<long long>({(long long)std::max(nr, nc), (64LL << 20) / per, 65535LL}));
-  const size_t b_nodes = Scratch::rnd(sizeof(EntryNode) * nn), b_inv = Scratch::rnd(sizeof(int) * std::max<size_t>(ninv, 1)),
-               b_leaf = Scratch::rnd(sizeof(int) * n), b_vec = Scratch::rnd(sizeof(double) * (size_t)chunk * per);
+  const size_t cr = std::min(chunk, nr), cc = std::min(chunk, nc);
+  const size_t b_row = Scratch::rnd(sizeof(double) * cr * per), b_col = Scratch::rnd(sizeof(double) * cc * per);
   char* buf = nullptr;
-  CK(dmalloc_async((void**)&buf, b_nodes + b_inv + b_leaf + 2 * b_vec + 256, st));
-  EntryNode* dn = (EntryNode*)buf;
-  int* inv = (int*)(buf + b_nodes);
-  int* dleaf = (int*)(buf + b_nodes + b_inv);
-  double* Wrow = (double*)(buf + b_nodes + b_inv + b_leaf);
-  double* Vcol = Wrow + (size_t)chunk * per;
-  int* err = (int*)(buf + b_nodes + b_inv + b_leaf + 2 * b_vec);
-  std::vector<EntryNode> hn(nn);
-  size_t o = 0;
-  for (int id = 0; id < nn; ++id) {
-    const Node& t = H->nodes[id];
-    EntryNode& e = hn[id];
-    memset(&e, 0, sizeof e);
-    e.lo = t.lo; e.size = t.size; e.level = t.level; e.parent = t.parent; e.ch0 = t.ch[0]; e.ch1 = t.ch[1];
-    e.state = t.state;
-    e.D = t.D; e.B12 = t.B12; e.B21 = t.B21; e.F12 = t.F12; e.F21 = t.F21;
-    if (id && t.state == HSS_COMPRESSED) {
-      e.kr = t.r.k; e.kc = t.c.k; e.mr = t.r.m; e.mc = t.c.m;
-      e.pivr = t.r.piv; e.pivc = t.c.piv; e.Xr = t.r.X; e.Xc = t.c.X;
-      e.ipivr = inv + o; o += t.r.m;
-      e.ipivc = inv + o; o += t.c.m;
-    }
-  }
-  hss_status s = HSS_OK;
-  Ctx c(st);
+  CK(dmalloc_async(&buf, b_row + b_col + 256, st));
+  double* Wrow = (double*)buf;
+  double* Vcol = (double*)(buf + b_row);
+  int* err = (int*)(buf + b_row + b_col);
   auto run = [&]() -> hss_status {
     CK(cudaMemsetAsync(err, 0, sizeof(int), st));
-    CK(cudaMemsetAsync(inv, 0xff, sizeof(int) * std::max<size_t>(ninv, 1), st));   // -1: no position
-    CKS(upload(c, dn, hn.data(), sizeof(EntryNode) * nn));
-    CKS(upload(c, dleaf, leaf_of.data(), sizeof(int) * n));
-    CK(launch_inv_piv(dn, nn, err, st));
     for (int c0 = 0; c0 < nc; c0 += chunk) {
       const int w = std::min(chunk, nc - c0);
-      CK(launch_entry_paths(dn, dleaf, n, J + c0, w, Vcol, kcap, lp1, 1, err, st));
       for (int r0 = 0; r0 < nr; r0 += chunk) {
         const int h = std::min(chunk, nr - r0);
-        CK(launch_entry_paths(dn, dleaf, n, I + r0, h, Wrow, kcap, lp1, 0, err, st));
-        CK(launch_entry_pairs(dn, dleaf, n, I + r0, h, J + c0, w, Wrow, Vcol, kcap, lp1,
+        // (the column vectors with the first rows, then they are there)
+        CK(launch_entry_paths(P->nodes, P->leaf_of, n, I + r0, h, J + c0, r0 == 0 ? w : 0, Wrow, Vcol, kcap, lp1, err,
+                              st));
+        CK(launch_entry_pairs(P->nodes, P->leaf_of, n, I + r0, h, J + c0, w, Wrow, Vcol, kcap, lp1,
                               out + r0 + (long long)c0 * ldo, ldo, st));
       }
     }
@@ -2994,7 +3212,7 @@ hss_status hss_get_entries(hss_matrix H, int nr, const int* I, int nc, const int
     if (herr) return fail(HSS_ERR_CUDA, "inconsistent pivots in the handle (code %d)", herr);
     return HSS_OK;
   };
-  s = run();
+  const hss_status s = run();
   cudaFreeAsync(buf, st);
   return s;
 }

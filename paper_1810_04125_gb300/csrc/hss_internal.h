@@ -191,6 +191,21 @@ struct EntryNode {
   const double* F21;
 };
 
+// One task of the HSS product (k_prod.cu): one node's result, rows i < rows,
+//   out(i) = sum_l M(i, l) v(l) [+ v(self_i)] [+ row pos_i of (I; X2^T) y2].
+struct ProdTask {
+  const double* M;       // element (i, l) at i + l ld (trans 0) or i ld + l (trans 1)
+  const int* gather;     // v is read at gather[l] (NULL: at l)
+  const int* self;       // v(self[i]) is added (up-sweep), or NULL
+  const double* X2;      // k2 x (.) col-major
+  const int* pos;        // position of the task's rows in the pivot order
+  int ld, K, trans, rows;
+  int in_lo;             // v = X(in_lo + .), or -1: the buffer rows in0 + l below split,
+  int in0, in1, split;   // in1 + l - split from there
+  int k2, y2;            // y2: buffer row; k2 = 0: no such term
+  int out_lo, out;       // Y(out_lo + i), or -1: buffer row out + i
+};
+
 // Launch wrappers (return cudaError_t of the launch).
 cudaError_t launch_random_normal(unsigned long long seed, int n, int col0, int ncols,
                                  double* R, long long ldr, int round_mode, cudaStream_t st);
@@ -224,7 +239,8 @@ cudaError_t launch_sample_tc_packed(const void* A, const void* Rp, int n, int nc
 cudaError_t launch_round_copy(const double* in, long long ldin, double* out, long long ldout, int n,
                               int ncols, int mode, cudaStream_t st);
 cudaError_t launch_extract(const ExtractJob* jobs_dev, int njobs, int max_tiles, cudaStream_t st);
-cudaError_t launch_gemm(const GemmJob* jobs_dev, const GemmTile* tiles_dev, int ntiles,
+// (copies: every job has K = 0)
+cudaError_t launch_gemm(const GemmJob* jobs_dev, const GemmTile* tiles_dev, int ntiles, bool copies,
                         cudaStream_t st);
 // FP64 products on the tensor cores from operands cut into eight 8-bit
 // digits (k_gemm_xs.cu): tiles of XS_TM x XS_TN, k-tiles of XS_BK.  Every
@@ -310,11 +326,17 @@ cudaError_t launch_nonfinite(const double* S, long long lds, int n, int c0, int 
 cudaError_t launch_asymmetric(const double* a, long long ld, int n, int* flag, cudaStream_t st);
 cudaError_t launch_identity_block(double* X, int n, int c0, int w, cudaStream_t st);
 cudaError_t launch_gather_int(const GatherJob* jobs_dev, int njobs, int max_cnt, cudaStream_t st);
+// buf: the product's node vectors, row-major with nrhs columns
+// (tiles: 16-row tiles of the largest task; at most 65535 x 8 columns; after:
+// the launch before this one on the stream belongs to the same product)
+cudaError_t launch_prod(const ProdTask* tasks, int ntasks, int tiles, bool after, int nrhs, const double* X, long long ldx,
+                        double* Y, long long ldy, double* buf, cudaStream_t st);
 // entries of a compressed handle (k_entries.cu); err: 1 = index out of
 // range, 2 = pivot out of range
+cudaError_t launch_leaf_of(const EntryNode* nodes, int nn, int* leaf_of, cudaStream_t st);
 cudaError_t launch_inv_piv(const EntryNode* nodes, int nn, int* err, cudaStream_t st);
-cudaError_t launch_entry_paths(const EntryNode* nodes, const int* leaf_of, int n, const int* idx, int count,
-                               double* out, int kcap, int lp1, int side, int* err, cudaStream_t st);
+cudaError_t launch_entry_paths(const EntryNode* nodes, const int* leaf_of, int n, const int* I, int nr, const int* J,
+                               int nc, double* Wrow, double* Vcol, int kcap, int lp1, int* err, cudaStream_t st);
 cudaError_t launch_entry_pairs(const EntryNode* nodes, const int* leaf_of, int n, const int* I, int nr, const int* J,
                                int nc, const double* Wrow, const double* Vcol, int kcap, int lp1, double* out,
                                long long ldo, cudaStream_t st);

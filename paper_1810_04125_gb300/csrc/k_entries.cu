@@ -10,11 +10,11 @@
 // v_b(j) with V.  A node that was not COMPRESSED (a partial result) keeps
 // its blocks A(I_nu1, I_nu2), A(I_nu2, I_nu1) dense.
 //
-// Three kernels: the inverse pivot orders of every node side; one CTA per
-// requested row index walking its leaf's path to the root and storing
-// W_i(level) = u_a(i) B_ab for every ancestor a (and one CTA per column index
-// storing v_b(j)); one thread per requested entry finding the common
-// ancestor and forming one dot product.
+// Kept with the handle: the nodes, the inverse pivot orders of every node side
+// and the leaf of every index.  A call is two kernels: one CTA per requested
+// index walking its leaf's path to the root (row indices store W_i(level) =
+// u_a(i) B_ab for every ancestor a, column indices v_b(j)), and a warp per
+// eight entries finding the common ancestors and forming the dot products.
 #include "hss_internal.h"
 
 namespace hss {
@@ -36,84 +36,147 @@ __global__ void k_inv_piv(const EntryNode* __restrict__ nodes, int nn, int* __re
   }
 }
 
-// Row (side 0) or column (side 1) vectors of the nested basis along the path
-// of index idx[r] to the root.  side 0 stores W(level(a)) = u_a(i) B_ab for
-// every ancestor a whose parent is COMPRESSED; side 1 stores v_a(j).
-// out: (count x (levels + 1) x kcap) doubles; shared memory 2 kcap doubles.
-__global__ void k_entry_paths(const EntryNode* __restrict__ nodes, const int* __restrict__ leaf_of, int n,
-                              const int* __restrict__ idx, int count, double* __restrict__ out, int kcap, int lp1,
-                              int side, int* __restrict__ err) {
+// leaf_of[i] = the leaf that holds i (one CTA per node)
+__global__ void k_leaf_of(const EntryNode* __restrict__ nodes, int* __restrict__ leaf_of) {
+  const EntryNode& t = nodes[blockIdx.x];
+  if (t.ch0 >= 0) return;
+  for (int i = threadIdx.x; i < t.size; i += blockDim.x) leaf_of[t.lo + i] = blockIdx.x;
+}
+
+// Eight sums over a warp at once: lane l's a[x] are its parts of sum x; the
+// return value is sum l / 4 (in all four lanes of that number).  Halving the
+// number of sums with every exchange takes 9 additions where eight butterflies
+// take 40 (an FP64 instruction of a warp occupies its scheduler's FP64 pipe
+// for 64 clocks).
+__device__ __forceinline__ double warp_sum8(double* a, int lane) {
+#pragma unroll
+  for (int h = 4; h >= 1; h /= 2) {
+    const bool up = (lane & (4 * h)) != 0;
+#pragma unroll
+    for (int x = 0; x < h; ++x) {
+      const double keep = up ? a[x + h] : a[x], give = up ? a[x] : a[x + h];
+      a[x] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+    }
+  }
+  double s = a[0];
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  return s;
+}
+
+constexpr int EW = 4;   // warps of a path CTA
+
+// Row (CTAs below nr) or column vectors of the nested basis along the path of
+// an index to the root.  A row stores W(level(a)) = u_a(i) B_ab for every
+// ancestor a whose parent is COMPRESSED, a column v_a(j).  Wrow, Vcol:
+// (count x (levels + 1) x kcap) doubles; shared memory 2 kcap doubles and kcap
+// ints.  Bound by the FP64 pipe (sum of k_a k_b + k_a k_p per level) once the
+// sums run along the blocks' contiguous direction: u B with eight columns of B
+// per warp and lanes along u, u U_p with a lane per column.  Rows and columns
+// go in one launch.
+__global__ void __launch_bounds__(32 * EW) k_entry_paths(const EntryNode* __restrict__ nodes,
+                                                         const int* __restrict__ leaf_of, int n,
+                                                         const int* __restrict__ I, int nr, const int* __restrict__ J,
+                                                         double* __restrict__ Wrow, double* __restrict__ Vcol, int kcap,
+                                                         int lp1, int* __restrict__ err) {
   extern __shared__ double sm[];
   double* u = sm;
   double* u2 = sm + kcap;
-  const int r = blockIdx.x;
-  if (r >= count) return;
-  const int i = idx[r];
+  int* sp = (int*)(sm + 2 * kcap);
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const int side = (int)blockIdx.x >= nr, r = side ? blockIdx.x - nr : blockIdx.x;
+  const int i = side ? J[r] : I[r];
   if (i < 0 || i >= n) {   // reported; the pair kernel skips the entry
-    if (threadIdx.x == 0) atomicCAS(err, 0, 1);
+    if (tid == 0) atomicCAS(err, 0, 1);
     return;
   }
   int a = leaf_of[i];
   // the root is a leaf (D only), or the leaf's parent was left uncompressed
   // (its couplings are dense blocks; the leaf has no basis)
   if (nodes[a].parent < 0 || nodes[nodes[a].parent].state != HSS_COMPRESSED) return;
-  double* base = out + (long long)r * lp1 * kcap;
+  double* base = (side ? Vcol : Wrow) + (long long)r * lp1 * kcap;
   {
     const EntryNode& t = nodes[a];
     const int k = side ? t.kc : t.kr;
-    const int* inv = side ? t.ipivc : t.ipivr;
     const double* X = side ? t.Xc : t.Xr;
-    const int pos = inv[i - t.lo];
+    const int pos = (side ? t.ipivc : t.ipivr)[i - t.lo];
     if (pos < 0 || pos >= t.size) {   // not a permutation (never from a compression)
-      if (threadIdx.x == 0) atomicCAS(err, 0, 2);
+      if (tid == 0) atomicCAS(err, 0, 2);
       return;
     }
-    for (int c = threadIdx.x; c < k; c += blockDim.x)
-      u[c] = pos < k ? (c == pos ? 1.0 : 0.0) : X[c + (long long)(pos - k) * max(k, 1)];
+    for (int c = tid; c < k; c += 32 * EW) u[c] = pos < k ? (c == pos ? 1.0 : 0.0) : X[c + (long long)(pos - k) * k];
   }
-  __syncthreads();
   for (;;) {
+    __syncthreads();   // u
     const EntryNode& t = nodes[a];
     const EntryNode& p = nodes[t.parent];
     if (p.state != HSS_COMPRESSED) break;   // dense coupling above: no basis rows needed
-    const int ka = side ? t.kc : t.kr;
-    const int first = p.ch0 == a;
+    const int ka = side ? t.kc : t.kr, first = p.ch0 == a;
     const EntryNode& b = nodes[first ? p.ch1 : p.ch0];
     double* dst = base + (long long)t.level * kcap;
+    // the rows of U_p for the up-step: positions of a's rows in p's pivot order
+    const bool top = p.parent < 0;   // a is a child of the root
+    const int kp = side ? p.kc : p.kr, mp = side ? p.mc : p.mr;
+    if (!top) {
+      const int* inv = (side ? p.ipivc : p.ipivr) + (first ? 0 : (side ? b.kc : b.kr));
+      for (int q = tid; q < ka; q += 32 * EW) {
+        int pos = inv[q];
+        if (pos < 0 || pos >= mp) {   // not a permutation (never from a compression)
+          atomicCAS(err, 0, 2);
+          pos = -1;
+        }
+        sp[q] = pos;
+      }
+      for (int c = tid; c < kp; c += 32 * EW) u2[c] = 0.0;
+    }
     if (side == 0) {
       // W = u_a(i) B_ab: B12 is kr(nu1) x kc(nu2) with ld max(kr(nu1), 1),
       // B21 is kr(nu2) x kc(nu1) with ld max(kr(nu2), 1)
       const double* B = first ? p.B12 : p.B21;
-      const int ld = max(ka, 1);
-      for (int c = threadIdx.x; c < b.kc; c += blockDim.x) {
-        double s = 0.0;
-        for (int q = 0; q < ka; ++q) s = __fma_rn(u[q], B[q + (long long)c * ld], s);
-        dst[c] = s;
+      const int ld = max(ka, 1), nb = b.kc;
+      for (int c0 = 8 * warp; c0 < nb; c0 += 8 * EW) {
+        double acc[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) acc[x] = 0.0;
+        for (int q = lane; q < ka; q += 32) {
+          const double uq = u[q];
+          const double* col = B + q + (long long)c0 * ld;
+          double m[8];
+#pragma unroll
+          for (int x = 0; x < 8; ++x) m[x] = c0 + x < nb ? col[(long long)x * ld] : 0.0;
+#pragma unroll
+          for (int x = 0; x < 8; ++x) acc[x] = __fma_rn(uq, m[x], acc[x]);
+        }
+        const double s = warp_sum8(acc, lane);
+        if ((lane & 3) == 0 && c0 + lane / 4 < nb) dst[c0 + lane / 4] = s;
       }
     } else {
-      for (int c = threadIdx.x; c < ka; c += blockDim.x) dst[c] = u[c];
+      for (int c = tid; c < ka; c += 32 * EW) dst[c] = u[c];
     }
-    if (p.parent < 0) break;   // a is a child of the root
+    if (top) break;
+    __syncthreads();   // sp, u2
     // u_parent(i) = u_a(i) U_p(off + q, :), U_p(s, c) = [pos_s == c] for the
     // skeleton rows, X_p(c, pos_s - k_p) for the others
-    const int kp = side ? p.kc : p.kr;
-    const int* inv = side ? p.ipivc : p.ipivr;
     const double* X = side ? p.Xc : p.Xr;
-    const int off = first ? 0 : (side ? b.kc : b.kr);
-    const int mp = side ? p.mc : p.mr;
-    for (int c = threadIdx.x; c < kp; c += blockDim.x) {
+    for (int c0 = 32 * warp; c0 < kp; c0 += 32 * EW) {
+      const int c = c0 + lane;
       double s = 0.0;
-      for (int q = 0; q < ka; ++q) {
-        const int pos = inv[off + q];
-        if (pos < 0 || pos >= mp) {   // not a permutation (never from a compression)
-          atomicCAS(err, 0, 2);
-          continue;
+      for (int q0 = 0; q0 < ka; q0 += 8) {
+        double m[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          const int pos = q0 + x < ka ? sp[q0 + x] : -1;
+          m[x] = pos >= kp && c < kp ? X[c + (long long)(pos - kp) * kp] : 0.0;
         }
-        s = __fma_rn(u[q], pos < kp ? (pos == c ? 1.0 : 0.0) : X[c + (long long)(pos - kp) * max(kp, 1)], s);
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          if (q0 + x < ka && sp[q0 + x] >= kp) s = __fma_rn(u[q0 + x], m[x], s);
       }
-      u2[c] = s;
+      if (c < kp) u2[c] = s;
     }
     __syncthreads();
+    for (int q = tid; q < ka; q += 32 * EW)   // the skeleton rows: each position once
+      if (sp[q] >= 0 && sp[q] < kp) u2[sp[q]] += u[q];
     double* tmp = u;
     u = u2;
     u2 = tmp;
@@ -121,47 +184,67 @@ __global__ void k_entry_paths(const EntryNode* __restrict__ nodes, const int* __
   }
 }
 
-// out(r, c) = H(I[r], J[c]) for one chunk of rows and columns
-__global__ void k_entry_pairs(const EntryNode* __restrict__ nodes, const int* __restrict__ leaf_of, int n,
-                              const int* __restrict__ I, int nr, const int* __restrict__ J, int nc,
-                              const double* __restrict__ Wrow, const double* __restrict__ Vcol, int kcap, int lp1,
-                              double* __restrict__ out, long long ldo) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int c = blockIdx.y;
-  if (r >= nr || c >= nc) return;
-  const int i = I[r], j = J[c];
-  double* dst = out + r + (long long)c * ldo;
-  if (i < 0 || i >= n || j < 0 || j >= n) { *dst = 0.0; return; }
-  int a = leaf_of[i], b = leaf_of[j];
-  if (a == b) {
-    const EntryNode& t = nodes[a];
-    *dst = t.D[(i - t.lo) + (long long)(j - t.lo) * t.size];
-    return;
+// out(r, c) = H(I[r], J[c]) for one chunk of rows and columns: a warp takes
+// eight rows of one column, lanes along the dot products (a thread per entry
+// walked 64 cache lines per step of a warp).
+__global__ void __launch_bounds__(128) k_entry_pairs(const EntryNode* __restrict__ nodes, const int* __restrict__ leaf_of,
+                                                     int n, const int* __restrict__ I, int nr,
+                                                     const int* __restrict__ J, int nc, const double* __restrict__ Wrow,
+                                                     const double* __restrict__ Vcol, int kcap, int lp1,
+                                                     double* __restrict__ out, long long ldo) {
+  const int lane = threadIdx.x % 32, r0 = (blockIdx.x * 4 + threadIdx.x / 32) * 8, c = blockIdx.y;
+  if (r0 >= nr || c >= nc) return;
+  const int j = J[c];
+  // lane l finds the place of entry l / 4: the levels of the two vectors, their
+  // length, or the entry itself
+  const int rx = r0 + lane / 4;
+  int lev = -1, kb = 0;
+  double val = 0.0;
+  if (rx < nr && j >= 0 && j < n) {
+    const int i = I[rx];
+    if (i >= 0 && i < n) {
+      int a = leaf_of[i], b = leaf_of[j];
+      if (a == b) {
+        const EntryNode& t = nodes[a];
+        val = t.D[(i - t.lo) + (long long)(j - t.lo) * t.size];
+      } else {
+        while (nodes[a].level > nodes[b].level) a = nodes[a].parent;
+        while (nodes[b].level > nodes[a].level) b = nodes[b].parent;
+        while (nodes[a].parent != nodes[b].parent) { a = nodes[a].parent; b = nodes[b].parent; }
+        const EntryNode& ta = nodes[a];
+        const EntryNode& tb = nodes[b];
+        const EntryNode& p = nodes[ta.parent];
+        if (p.state != HSS_COMPRESSED) {
+          const double* F = p.ch0 == a ? p.F12 : p.F21;   // A(I_a, I_b), ld |a|
+          val = F[(i - ta.lo) + (long long)(j - tb.lo) * ta.size];
+        } else {
+          lev = ta.level;   // (a and b are siblings: one level)
+          kb = tb.kc;
+        }
+      }
+    }
   }
-  while (nodes[a].level > nodes[b].level) a = nodes[a].parent;
-  while (nodes[b].level > nodes[a].level) b = nodes[b].parent;
-  while (nodes[a].parent != nodes[b].parent) { a = nodes[a].parent; b = nodes[b].parent; }
-  const EntryNode& ta = nodes[a];
-  const EntryNode& tb = nodes[b];
-  const EntryNode& p = nodes[ta.parent];
-  if (p.state != HSS_COMPRESSED) {
-    const double* F = p.ch0 == a ? p.F12 : p.F21;   // A(I_a, I_b), ld |a|
-    *dst = F[(i - ta.lo) + (long long)(j - tb.lo) * ta.size];
-    return;
+  double acc[8];
+#pragma unroll
+  for (int x = 0; x < 8; ++x) {
+    acc[x] = 0.0;
+    const int lx = __shfl_sync(0xffffffffu, lev, 4 * x), kx = __shfl_sync(0xffffffffu, kb, 4 * x);
+    if (lx < 0) continue;
+    const double* w = Wrow + ((long long)(r0 + x) * lp1 + lx) * kcap;
+    const double* v = Vcol + ((long long)c * lp1 + lx) * kcap;
+    for (int q = lane; q < kx; q += 32) acc[x] = __fma_rn(w[q], v[q], acc[x]);
   }
-  const double* w = Wrow + ((long long)r * lp1 + ta.level) * kcap;
-  const double* v = Vcol + ((long long)c * lp1 + tb.level) * kcap;
-  double s0 = 0.0, s1 = 0.0;
-  int q = 0;
-  for (; q + 1 < tb.kc; q += 2) {
-    s0 = __fma_rn(w[q], v[q], s0);
-    s1 = __fma_rn(w[q + 1], v[q + 1], s1);
-  }
-  if (q < tb.kc) s0 = __fma_rn(w[q], v[q], s0);
-  *dst = s0 + s1;
+  const double s = warp_sum8(acc, lane);
+  if ((lane & 3) == 0 && rx < nr) out[rx + (long long)c * ldo] = lev >= 0 ? s : val;
 }
 
 }  // namespace
+
+cudaError_t launch_leaf_of(const EntryNode* nodes, int nn, int* leaf_of, cudaStream_t st) {
+  if (nn <= 0) return cudaSuccess;
+  k_leaf_of<<<nn, 128, 0, st>>>(nodes, leaf_of);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_inv_piv(const EntryNode* nodes, int nn, int* err, cudaStream_t st) {
   if (nn <= 0) return cudaSuccess;
@@ -169,13 +252,13 @@ cudaError_t launch_inv_piv(const EntryNode* nodes, int nn, int* err, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_entry_paths(const EntryNode* nodes, const int* leaf_of, int n, const int* idx, int count,
-                               double* out, int kcap, int lp1, int side, int* err, cudaStream_t st) {
-  if (count <= 0) return cudaSuccess;
-  const size_t sm = sizeof(double) * 2 * (size_t)kcap;
+cudaError_t launch_entry_paths(const EntryNode* nodes, const int* leaf_of, int n, const int* I, int nr, const int* J,
+                               int nc, double* Wrow, double* Vcol, int kcap, int lp1, int* err, cudaStream_t st) {
+  if (nr + nc <= 0) return cudaSuccess;
+  const size_t sm = (sizeof(double) * 2 + sizeof(int)) * (size_t)kcap;
   cudaError_t e = cudaFuncSetAttribute(k_entry_paths, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_entry_paths<<<count, 128, sm, st>>>(nodes, leaf_of, n, idx, count, out, kcap, lp1, side, err);
+  k_entry_paths<<<nr + nc, 32 * EW, sm, st>>>(nodes, leaf_of, n, I, nr, J, Wrow, Vcol, kcap, lp1, err);
   return cudaGetLastError();
 }
 
@@ -183,8 +266,8 @@ cudaError_t launch_entry_pairs(const EntryNode* nodes, const int* leaf_of, int n
                                int nc, const double* Wrow, const double* Vcol, int kcap, int lp1, double* out,
                                long long ldo, cudaStream_t st) {
   if (nr <= 0 || nc <= 0) return cudaSuccess;
-  k_entry_pairs<<<dim3((nr + 127) / 128, nc), 128, 0, st>>>(nodes, leaf_of, n, I, nr, J, nc, Wrow, Vcol, kcap, lp1,
-                                                            out, ldo);
+  k_entry_pairs<<<dim3((nr + 31) / 32, nc), 128, 0, st>>>(nodes, leaf_of, n, I, nr, J, nc, Wrow, Vcol, kcap, lp1, out,
+                                                          ldo);
   return cudaGetLastError();
 }
 

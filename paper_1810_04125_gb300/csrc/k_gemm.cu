@@ -24,6 +24,52 @@ __device__ __forceinline__ double ld_op(const Opnd& o, int i, int l) {
   return b[(long long)r * o.rs + (long long)l * o.cs];
 }
 
+// A job without a product, C = beta C0 + gamma C (gathers and scatters of node
+// vectors, many of them between column- and row-major): 32 columns at a time
+// through shared memory, lanes along the contiguous direction on each side.
+// Without the product's registers eight CTAs fit an SM instead of two.
+__global__ void __launch_bounds__(256) k_copy(const GemmJob* __restrict__ jobs, const GemmTile* __restrict__ tiles) {
+  constexpr int LD = TM + 1;
+  __shared__ double sm[32 * LD];
+  const GemmTile tl = tiles[blockIdx.x];
+  const GemmJob& jb = jobs[tl.job];
+  const int i0 = tl.ti * TM, j0 = tl.tj * TN, tid = threadIdx.x;
+  const bool in_rm = jb.C0.cs == 1, out_rm = jb.c_cs == 1;
+  const double beta = jb.beta, gamma = jb.gamma;
+  for (int h = 0; h < TN; h += 32) {
+    if (j0 + h >= jb.N) break;
+    if (h) __syncthreads();
+    if (beta != 0.0) {
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int e = tid + q * 256, il = in_rm ? e / 32 : e % TM, jl = in_rm ? e % 32 : e / TM;
+        v[q] = i0 + il < jb.M && j0 + h + jl < jb.N ? ld_op(jb.C0, i0 + il, j0 + h + jl) : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int e = tid + q * 256, il = in_rm ? e / 32 : e % TM, jl = in_rm ? e % 32 : e / TM;
+        sm[jl * LD + il] = v[q];
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int e = tid + q * 256, il = out_rm ? e / 32 : e % TM, jl = out_rm ? e % 32 : e / TM;
+      const int i = i0 + il, j = j0 + h + jl;
+      if (i >= jb.M || j >= jb.N) continue;
+      int r = jb.c_rows ? jb.c_rows[i] : i;
+      double* base = jb.C;
+      if (r >= jb.c_split) { base = jb.C2; r -= jb.c_split; }
+      double* dst = base + (long long)r * jb.c_rs + (long long)j * jb.c_cs;
+      double v = 0.0;
+      if (beta != 0.0) v = beta == 1.0 ? sm[jl * LD + il] : beta * sm[jl * LD + il];
+      if (gamma != 0.0) v += gamma == 1.0 ? *dst : gamma * *dst;
+      *dst = v;
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256) k_gemm(const GemmJob* __restrict__ jobs,
                                               const GemmTile* __restrict__ tiles) {
   __shared__ double As[TK][TM + 2];
@@ -88,9 +134,13 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmJob* __restrict__ jobs,
 
 }  // namespace
 
-cudaError_t launch_gemm(const GemmJob* jobs_dev, const GemmTile* tiles_dev, int ntiles,
+cudaError_t launch_gemm(const GemmJob* jobs_dev, const GemmTile* tiles_dev, int ntiles, bool copies,
                         cudaStream_t st) {
   if (ntiles <= 0) return cudaSuccess;
+  if (copies) {
+    k_copy<<<ntiles, 256, 0, st>>>(jobs_dev, tiles_dev);
+    return cudaGetLastError();
+  }
   k_gemm<<<ntiles, 256, 0, st>>>(jobs_dev, tiles_dev);
   return cudaGetLastError();
 }

@@ -70,7 +70,7 @@ constexpr int XW = 16;                                  // drain warps
 constexpr int XMW = 3;                                  // warps that issue MMAs
 constexpr int XTHREADS = (1 + XMW + XW) * 32;
 constexpr int XNH = XS_TN / 4;                          // columns per drain thread
-constexpr int MAXK = 256;                               // k range of one maxima unit
+constexpr int MAXK = 128, MAXR = 32;                    // one maxima unit: k range, rows
 constexpr unsigned HI_INF = 0x7FF00000u;
 constexpr uint32_t MAGIC = 0x4B400000u;                 // bits of 1.5 2^23
 
@@ -149,51 +149,55 @@ __device__ __forceinline__ int find_job(const int* prefix, int njobs, int u) {
 }
 
 // ------------------------------------------------------------ operand maxima
-// One unit: 128 rows of A (or 64 columns of B) x 256 of K; memory-bound, one
-// read of the operand.
+// One unit: 32 rows of A (or columns of B) x 128 of K; one read of the operand.
+// A warp takes four rows, all their loads in flight together (with 128 rows to
+// a unit, a warp's sixteen rows one after the other took 25 us whatever the
+// size).
 __global__ void __launch_bounds__(256) k_xs_max(const GemmJob* __restrict__ jobs, const int* __restrict__ prefix,
                                                 int njobs) {
   const int ji = find_job(prefix, njobs, blockIdx.x);
   const GemmJob& j = jobs[ji];
   int u = blockIdx.x - prefix[ji];
-  const int nkc = (j.K + MAXK - 1) / MAXK, nrb = (j.M + XS_TM - 1) / XS_TM;
+  const int nkc = (j.K + MAXK - 1) / MAXK, nrb = (j.M + MAXR - 1) / MAXR;
   const int which = u >= nrb * nkc;
   if (which) u -= nrb * nkc;
-  const int tile = u / nkc, l0 = (u % nkc) * MAXK, l1 = min(j.K, l0 + MAXK);
-  const int R = which ? XS_TN : XS_TM, r0 = tile * R, nr = min(which ? j.N : j.M, r0 + R) - r0;
+  const int r0 = (u / nkc) * MAXR, l0 = (u % nkc) * MAXK, l1 = min(j.K, l0 + MAXK);
+  const int nr = min(which ? j.N : j.M, r0 + MAXR) - r0;
   const Opnd& o = which ? j.B : j.A;
   unsigned* out = (which ? j.eb : j.ea) + r0;
   const bool rows_fast = which ? o.cs == 1 : (o.rs == 1 && !o.rows);
   const long long cs = o.cs;
-  const int tid = threadIdx.x;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   auto at = [&](int r, int l) {
     return which ? op_row(o, l)[(long long)(r0 + r) * cs] : op_row(o, r0 + r)[(long long)l * cs];
   };
-  constexpr int UN = 8;   // loads in flight per thread
-  if (rows_fast) {
-    const int r = tid % R, g = tid / R, ng = 256 / R;
-    if (r < nr) {
-      unsigned k = 0u;
-      for (int l = l0 + g; l < l1; l += UN * ng) {
-        double v[UN];
+  if (rows_fast) {   // lanes along the rows, a warp every eighth l
+    unsigned k = 0u;
+    if (lane < nr)
+      for (int lb = l0 + warp; lb < l1; lb += 64) {
+        double v[8];
 #pragma unroll
-        for (int x = 0; x < UN; ++x) v[x] = l + x * ng < l1 ? at(r, l + x * ng) : 0.0;
+        for (int x = 0; x < 8; ++x) v[x] = lb + 8 * x < l1 ? at(lane, lb + 8 * x) : 0.0;
 #pragma unroll
-        for (int x = 0; x < UN; ++x) k = max(k, mag_key(v[x]));
+        for (int x = 0; x < 8; ++x) k = max(k, mag_key(v[x]));
       }
-      if (k) atomicMax(out + r, k);
+    if (k) atomicMax(out + lane, k);
+  } else {   // lanes along l
+    unsigned k[4] = {0u, 0u, 0u, 0u};
+    for (int lb = l0 + lane; lb < l1; lb += 64) {
+      double v[4][2];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+          v[q][x] = 4 * warp + q < nr && lb + 32 * x < l1 ? at(4 * warp + q, lb + 32 * x) : 0.0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) k[q] = max(k[q], max(mag_key(v[q][0]), mag_key(v[q][1])));
     }
-  } else {
-    const int warp = tid / 32, lane = tid % 32;
-    for (int r = warp; r < nr; r += 8) {
-      unsigned k = 0u;
-      double v[MAXK / 32];
 #pragma unroll
-      for (int x = 0; x < MAXK / 32; ++x) v[x] = l0 + lane + 32 * x < l1 ? at(r, l0 + lane + 32 * x) : 0.0;
-#pragma unroll
-      for (int x = 0; x < MAXK / 32; ++x) k = max(k, mag_key(v[x]));
-      k = __reduce_max_sync(0xffffffffu, k);
-      if (lane == 0 && k) atomicMax(out + r, k);
+    for (int q = 0; q < 4; ++q) {
+      const unsigned m = __reduce_max_sync(0xffffffffu, k[q]);
+      if (lane == 0 && m) atomicMax(out + 4 * warp + q, m);
     }
   }
 }
@@ -711,7 +715,7 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
 size_t xs_tile_bytes(int which) { return (size_t)XD * (which ? XB : XA); }
 
 int xs_max_units(int M, int N, int K) {
-  return ((M + XS_TM - 1) / XS_TM + (N + XS_TN - 1) / XS_TN) * ((K + MAXK - 1) / MAXK);
+  return ((M + MAXR - 1) / MAXR + (N + MAXR - 1) / MAXR) * ((K + MAXK - 1) / MAXK);
 }
 int xs_pack_units(int M, int N, int K) {
   return ((M + XS_TM - 1) / XS_TM + (N + XS_TN - 1) / XS_TN) * ((K + XS_BK - 1) / XS_BK);
