@@ -374,6 +374,7 @@ struct hss_matrix_s {
   int d_final = 0, n_adapt = 0, converged = 0;
   int pack_decided = -1;   // mixed forms, generated A: packed tiles (1) or not (0)
   bool sym = false;        // the column side is a copy of the row side (find_symmetric)
+  bool same_samples = false;   // mixed forms, A = A^T: S^c is a copy of S^r
   void* packA = nullptr;   // packed tensor-core tiles of a dense A (during compress)
   XsKeep xs;               // digits of a generated source (during compress, plain form)
   void* toep_terms = nullptr; // a Toeplitz source's diagonals split into terms (during compress)
@@ -989,7 +990,7 @@ bool use_packed(hss_matrix_s* H) {
   if (H->src.kind == HSS_SRC_DENSE) return true;
   if (H->pack_decided < 0) {
     size_t fr = 0, tot = 0;
-    const size_t pb = packed_a_bytes(H->n, H->o.precision);
+    const size_t pb = packed_a_bytes(H->n, H->o.precision, H->sym || H->same_samples ? 1 : 2);
     H->pack_decided = (cudaMemGetInfo(&fr, &tot) == cudaSuccess && (double)pb <= 0.4 * (double)fr) ? 1 : 0;
   }
   return H->pack_decided == 1;
@@ -1153,6 +1154,13 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
   SrcDev s = make_src(H->src, H->leaf_id);
   const double* Rc = H->R + (long long)c0 * n;
   const int norient = H->sym ? 1 : 2;   // A^T R is A R for a symmetric A
+  const bool one_side = H->sym || H->same_samples;
+  auto copy_samples = [&]() -> hss_status {
+    if (H->same_samples)
+      CK(cudaMemcpy2DAsync(H->Sg_c + c0, sizeof(double) * H->dmax, H->Sg_r + c0, sizeof(double) * H->dmax,
+                           sizeof(double) * w, n, cudaMemcpyDeviceToDevice, st));
+    return HSS_OK;
+  };
   if (H->o.op) {
     // the user's product A R (and A^T R), then the leaf diagonal blocks off
     CK(c.timer.mark(PH_SAMPLE, st));
@@ -1191,10 +1199,11 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
     // every pass streams them (a generated A is evaluated once, not once per
     // pass)
     if (!H->packA) {
-      const size_t pb = packed_a_bytes(n, H->o.precision);
+      const int orients = one_side ? 1 : 2;
+      const size_t pb = packed_a_bytes(n, H->o.precision, orients);
       CK(c.timer.mark(PH_SAMPLE, st));
       CK(dmalloc_async(&H->packA, pb, st));
-      CK(launch_pack_a(s, H->o.leaf, H->o.precision, H->packA, st));
+      CK(launch_pack_a(s, H->o.leaf, H->o.precision, orients, H->packA, st));
       c.launches++;
       // the split is part of the sampling work: a dense A read once, the
       // packed tiles written once
@@ -1207,16 +1216,17 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
     c.launches++;
     if (sample_tc_packed_ksplit(n, w, H->o.precision) > 1) {
       CK(cudaMemset2DAsync(H->Sg_r + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
-      if (!H->sym) CK(cudaMemset2DAsync(H->Sg_c + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
+      if (!one_side) CK(cudaMemset2DAsync(H->Sg_c + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
     }
     CK(c.timer.mark(PH_SAMPLE, st));
     CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 0, H->Sg_r + c0, H->dmax, c.d_flag + 1, st));
-    if (!H->sym)
+    if (!one_side)
       CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 1, H->Sg_c + c0, H->dmax, c.d_flag + 1,
                                  st));
-    c.launches += norient;
-    c.sample_launches += norient;
-    H->st.sample_launches += norient;
+    CKS(copy_samples());
+    c.launches += one_side ? 1 : 2;
+    c.sample_launches += one_side ? 1 : 2;
+    H->st.sample_launches += one_side ? 1 : 2;
     CK(c.timer.mark(PH_RNG, st));
     CK(cudaFreeAsync(packR, st));
   } else {
@@ -1233,18 +1243,19 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
     c.launches++;
     if (sample_tc_ksplit(n, w, H->o.precision) > 1) {
       CK(cudaMemset2DAsync(H->Sg_r + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
-      if (!H->sym) CK(cudaMemset2DAsync(H->Sg_c + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
+      if (!one_side) CK(cudaMemset2DAsync(H->Sg_c + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
     }
     CK(c.timer.mark(PH_SAMPLE, st));
     int at = 0;
     CK(launch_sample_tc(s, H->o.leaf, H->o.precision, 0, w, packR, H->Sg_r + c0, H->dmax, c.d_flag + 1, &at,
                         H->toep_terms, st));
-    if (!H->sym)
+    if (!one_side)
       CK(launch_sample_tc(s, H->o.leaf, H->o.precision, 1, w, packR, H->Sg_c + c0, H->dmax, c.d_flag + 1, &at,
                           H->toep_terms, st));
-    c.launches += norient;
-    c.sample_launches += norient;
-    H->st.sample_launches += norient;
+    CKS(copy_samples());
+    c.launches += one_side ? 1 : 2;
+    c.sample_launches += one_side ? 1 : 2;
+    H->st.sample_launches += one_side ? 1 : 2;
     CK(c.timer.mark(PH_RNG, st));
     CK(cudaFreeAsync(packR, st));
   }
@@ -2148,25 +2159,26 @@ hss_status setup(Ctx& c, const hss_source* A, const hss_opts* o, hss_matrix_s* H
 }
 
 // Which matrices are compressed on the row side alone, the column side being
-// its copy: those of the symmetric option, and in the plain form those that
+// its copy (1): those of the symmetric option, and in the plain form those that
 // are symmetric, where both sides are the same computation on the same bits
 // (Sc = Sr, so the same pivots, bases and reduced samples; B21 = B12^T).  A
 // generated source is symmetric by its definition; a dense one is compared
 // with its transpose, one read of A against one read per pass and side.  The
-// mixed forms keep their two sides: with the other split of the CTAs over the
-// sides the last bits of their QR change, and their samples, equal to 1e-7
-// only, turn that into other pivots.  A user operator is asked for both
-// products.
+// mixed forms share the samples only (2): with the other split of the CTAs
+// over the sides the last bits of their QR change, and their samples, equal
+// to 1e-7 only, turn that into other pivots.  A user operator is asked for
+// both products (0).
 hss_status find_symmetric(Ctx& c, const std::vector<const hss_source*>& A, const std::vector<const hss_opts*>& O,
                           std::vector<char>& sym) {
   const int m = (int)A.size();
   sym.assign(m, 0);
   bool any = false;
   std::vector<char> dense(m, 0);
+  auto kind = [&](int i) { return (char)(O[i]->precision == HSS_PREC_FP64 ? 1 : 2); };
   for (int i = 0; i < m; ++i) {
     if (O[i]->symmetric) sym[i] = 1;
-    else if (O[i]->precision != HSS_PREC_FP64 || O[i]->op) continue;
-    else if (symmetric_source(*A[i])) sym[i] = 1;
+    else if (O[i]->op) continue;
+    else if (symmetric_source(*A[i])) sym[i] = kind(i);
     else if (A[i]->kind == HSS_SRC_DENSE) {
       CK(launch_asymmetric(A[i]->a, A[i]->ld, A[i]->n, c.d_flag + 8 + m + i, c.st));
       c.launches++;
@@ -2177,7 +2189,7 @@ hss_status find_symmetric(Ctx& c, const std::vector<const hss_source*>& A, const
   if (!any) return HSS_OK;
   CKS(readback(c, c.d_flag, sizeof(int) * c.nflag));
   for (int i = 0; i < m; ++i)
-    if (dense[i] && !c.h_pinned[8 + m + i]) sym[i] = 1;
+    if (dense[i] && !c.h_pinned[8 + m + i]) sym[i] = kind(i);
   return HSS_OK;
 }
 
@@ -2196,7 +2208,8 @@ hss_status compress_all(Ctx& c, const std::vector<const hss_source*>& A, const s
   CKS(find_symmetric(c, A, O, sym));
   for (size_t i = 0; i < Hs.size(); ++i) {
     Hs[i]->slot = (int)i;
-    CKS(setup(c, A[i], O[i], Hs[i], sym[i] != 0, leafD));
+    Hs[i]->same_samples = sym[i] == 2;
+    CKS(setup(c, A[i], O[i], Hs[i], sym[i] == 1, leafD));
   }
   if (!leafD.per.empty()) {
     CK(c.timer.mark(PH_MERGE, c.st));
@@ -2439,7 +2452,7 @@ hss_status hss_compress_batched(const hss_source* A, const hss_opts* opts, int c
     double b = 8.0 * n * dm * (opts[i].symmetric ? 3.0 : 4.0);      // R, S^r, S^c, node samples
     if (opts[i].strategy == HSS_INCREMENTING) b += 8.0 * n * dm * 2.0;   // bases Q
     if (opts[i].precision != HSS_PREC_FP64 && A[i].kind == HSS_SRC_DENSE)
-      b += (double)packed_a_bytes(A[i].n, opts[i].precision);
+      b += (double)packed_a_bytes(A[i].n, opts[i].precision, 2);
     return b;
   };
   size_t fr = 0, tot = 0;
@@ -3304,8 +3317,8 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   CK(dmalloc_async(&pR, packed_r_bytes(n, ncols, precision), st));
   CK(launch_pack_r(Rr, n, n, ncols, precision, pR, st));
   if (packed) {
-    CK(dmalloc_async(&pA, packed_a_bytes(n, precision), st));
-    CK(launch_pack_a(s, leaf, precision, pA, st));
+    CK(dmalloc_async(&pA, packed_a_bytes(n, precision, 2), st));
+    CK(launch_pack_a(s, leaf, precision, 2, pA, st));
   } else if (A->kind == HSS_SRC_TOEPLITZ) {
     CK(dmalloc_async(&tt, toeplitz_terms_bytes(n, precision), st));
     CK(launch_toeplitz_terms(s, precision, tt, st));
@@ -3313,6 +3326,11 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   for (int side = 0; side < 2; ++side) {
     double* S = side ? Sc : Sr;
     if (!S) continue;
+    if (side == 1 && Sr && symmetric_source(*A)) {   // the same product of the same bits
+      CK(cudaMemcpy2DAsync(Sc, sizeof(double) * lds, Sr, sizeof(double) * lds, sizeof(double) * ncols, n,
+                           cudaMemcpyDeviceToDevice, st));
+      continue;
+    }
     const int ks = packed ? sample_tc_packed_ksplit(n, ncols, precision) : sample_tc_ksplit(n, ncols, precision);
     if (ks > 1) CK(cudaMemset2DAsync(S, sizeof(double) * lds, 0, sizeof(double) * ncols, n, st));
     int at = 0;

@@ -226,9 +226,10 @@ cudaError_t launch_toeplitz_terms(const SrcDev& src, int precision, void* out, c
 int sample_tc_ksplit(int n, int ncols, int precision);
 // packed form for a dense A: operands split once into canonical tiles in
 // global memory, the main loop fed by bulk copies (k_sample_tc.cu)
-size_t packed_a_bytes(int n, int precision);
+// (orients: 2, or 1 when A = A^T and the second orientation is not read)
+size_t packed_a_bytes(int n, int precision, int orients);
 size_t packed_r_bytes(int n, int ncols, int precision);
-cudaError_t launch_pack_a(const SrcDev& src, int leaf, int precision, void* out, cudaStream_t st);
+cudaError_t launch_pack_a(const SrcDev& src, int leaf, int precision, int orients, void* out, cudaStream_t st);
 cudaError_t launch_pack_r(const double* R, long long ldr, int n, int ncols, int precision, void* out,
                           cudaStream_t st);
 int sample_tc_packed_ksplit(int n, int ncols, int precision);

@@ -630,10 +630,10 @@ cudaError_t launch_toeplitz_terms(const SrcDev& src, int precision, void* out, c
   return cudaGetLastError();
 }
 
-size_t packed_a_bytes(int n, int precision) {
+size_t packed_a_bytes(int n, int precision, int orients) {
   const int T = precision == HSS_PREC_TF32X2 ? 2 : 3, bk = bk_of(precision);
   const size_t nrb = (n + BM - 1) / BM, nkt = (n + bk - 1) / bk;
-  return 2 * nrb * nkt * T * (size_t)TILE_A_BYTES;
+  return orients * nrb * nkt * T * (size_t)TILE_A_BYTES;
 }
 
 size_t packed_r_bytes(int n, int ncols, int precision) {
@@ -643,12 +643,12 @@ size_t packed_r_bytes(int n, int ncols, int precision) {
   return nct * nkt * (size_t)N * 128;
 }
 
-cudaError_t launch_pack_a(const SrcDev& src, int leaf, int precision, void* out, cudaStream_t st) {
+cudaError_t launch_pack_a(const SrcDev& src, int leaf, int precision, int orients, void* out, cudaStream_t st) {
   if (src.kind < HSS_SRC_DENSE || src.kind > HSS_SRC_LAPLACE) return cudaErrorInvalidValue;   // no entries on the device
   const int n = src.n;
   const int bk = bk_of(precision);
   const int nrb = (n + BM - 1) / BM, nkt = (n + bk - 1) / bk;
-  const long long tiles = 2LL * nrb * nkt;
+  const long long tiles = (long long)orients * nrb * nkt;
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   if (precision == HSS_PREC_TF32X2)
     k_pack_a<HSS_PREC_TF32X2><<<(unsigned)tiles, 256, 0, st>>>(src, leaf, nrb, nkt, (uint8_t*)out);
