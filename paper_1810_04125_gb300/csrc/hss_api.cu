@@ -1212,7 +1212,7 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
     }
     void* packR = nullptr;
     CK(dmalloc_async(&packR, packed_r_bytes(n, w, H->o.precision), st));
-    CK(launch_pack_r(Rc, n, n, w, H->o.precision, packR, st));
+    CK(launch_pack_r(Rc, n, n, w, H->o.precision, false, packR, st));
     c.launches++;
     if (sample_tc_packed_ksplit(n, w, H->o.precision) > 1) {
       CK(cudaMemset2DAsync(H->Sg_r + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
@@ -1239,7 +1239,7 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
     }
     void* packR = nullptr;
     CK(dmalloc_async(&packR, packed_r_bytes(n, w, H->o.precision), st));
-    CK(launch_pack_r(Rc, n, n, w, H->o.precision, packR, st));
+    CK(launch_pack_r(Rc, n, n, w, H->o.precision, H->toep_terms != nullptr, packR, st));
     c.launches++;
     if (sample_tc_ksplit(n, w, H->o.precision) > 1) {
       CK(cudaMemset2DAsync(H->Sg_r + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
@@ -3315,7 +3315,7 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   void* tt = nullptr;
   const bool packed = A->kind == HSS_SRC_DENSE;
   CK(dmalloc_async(&pR, packed_r_bytes(n, ncols, precision), st));
-  CK(launch_pack_r(Rr, n, n, ncols, precision, pR, st));
+  CK(launch_pack_r(Rr, n, n, ncols, precision, A->kind == HSS_SRC_TOEPLITZ, pR, st));
   if (packed) {
     CK(dmalloc_async(&pA, packed_a_bytes(n, precision, 2), st));
     CK(launch_pack_a(s, leaf, precision, 2, pA, st));

@@ -230,7 +230,8 @@ int sample_tc_ksplit(int n, int ncols, int precision);
 size_t packed_a_bytes(int n, int precision, int orients);
 size_t packed_r_bytes(int n, int ncols, int precision);
 cudaError_t launch_pack_a(const SrcDev& src, int leaf, int precision, int orients, void* out, cudaStream_t st);
-cudaError_t launch_pack_r(const double* R, long long ldr, int n, int ncols, int precision, void* out,
+// (toep: in the order that launch_sample_tc takes with Toeplitz terms)
+cudaError_t launch_pack_r(const double* R, long long ldr, int n, int ncols, int precision, bool toep, void* out,
                           cudaStream_t st);
 int sample_tc_packed_ksplit(int n, int ncols, int precision);
 cudaError_t launch_sample_tc_packed(const void* A, const void* Rp, int n, int ncols, int precision,

@@ -89,13 +89,11 @@ constexpr int GEN_WARPS = 16;
 // chains four k-tiles long (its samples serve tolerances >= 1e-4; measured
 // error of the samples below 5e-7), BF16 x 3 two (tolerances down to 1e-6)
 __host__ __device__ constexpr int drain_gen(int precision) { return precision == HSS_PREC_TF32X2 ? 4 : 2; }
-constexpr int TW = 80;   // window entries per term and producer warp (>= 8 + BK - 1)
 
 // The diagonals c_t of a Toeplitz matrix (A_ij = c_{i-j}: the first column
 // for i >= j, the first row for i < j), t = -(n-1) .. n-1, split into the T
 // terms of the mixed form exactly as the producers split an entry: the
-// generating kernel then assembles a tile from a window of consecutive
-// diagonals instead of evaluating and splitting every entry.  TF32 x 2: the
+// Toeplitz kernel assembles its tiles from them.  TF32 x 2: the
 // two terms of a diagonal side by side (one 8-byte word); BF16 x 3: term
 // after term (2n - 1 entries each).
 template <int PREC>
@@ -138,9 +136,6 @@ __global__ void __maxnreg__(96) k_sample_tc_gen(TcArgs a) {
   uint32_t* tmem_slot = (uint32_t*)(tempty + 2);
   int* lrow_lo = (int*)(tmem_slot + 4);
   int* lrow_hi = lrow_lo + BM;
-  // per producer warp: T window rows of TW diagonals (Toeplitz path)
-  uint32_t* win32 = (uint32_t*)(lrow_hi + BM) + (size_t)(threadIdx.x / 32) * T * TW;
-  uint16_t* win16 = (uint16_t*)win32;
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const int rb = blockIdx.x, ct = blockIdx.y;
   const int row0 = rb * BM, col0 = ct * N;
@@ -174,25 +169,11 @@ __global__ void __maxnreg__(96) k_sample_tc_gen(TcArgs a) {
 
   if (warp < GEN_WARPS) {
     const int q = warp % 4, h = warp / 4;
-    // this warp's rows (Toeplitz path): all below n, and the union of their
-    // leaf blocks [wlo, whi)
-    int wlo = 0x7fffffff, whi = -1;
-#pragma unroll
-    for (int rr = 0; rr < 8; ++rr) {
-      wlo = min(wlo, lrow_lo[8 * warp + rr]);
-      whi = max(whi, lrow_hi[8 * warp + rr]);
-    }
-    const bool rows_ok = row0 + 8 * warp + 8 <= n;
     float s[NH], e[NH];
 #pragma unroll
     for (int j = 0; j < NH; ++j) { s[j] = 0.f; e[j] = 0.f; }
     bool ok = true;
     int drained = 0;   // chains drained so far
-    // the Toeplitz diagonal terms: entry t of term k at tterm[k][t], |t| < n
-    const uint2* tterm64 = a.toep ? (const uint2*)a.toep + (n - 1) : nullptr;
-    const uint16_t* tterm16 = a.toep ? (const uint16_t*)a.toep + (n - 1) : nullptr;
-    uint2* win64 = (uint2*)win32;
-    const long long tlen = 2LL * n - 1;
     int st = 0;
     uint32_t ph = 0u;
     for (int it = 0; it < nk && ok; ++it) {
@@ -204,111 +185,26 @@ __global__ void __maxnreg__(96) k_sample_tc_gen(TcArgs a) {
         bulk_g2s(sp + T * TILE_A_BYTES, gB + (size_t)it * tileB, tileB, &full[st]);
       }
       const int k0 = (kt0 + it) * BK;
-      if (a.toep) {
-        // Toeplitz: this warp's 8 rows of the tile from a window of 8 + BK - 1
-        // consecutive diagonals (orientation 0: A(r, k) = c_{r - k}; 1:
-        // A(k, r) = c_{k - r}), masked only where the rows reach past n or a
-        // row's leaf block meets the tile's columns
-        const int rw = 8 * warp;
-        const int tb = TRANS ? k0 - row0 - rw - 7 : row0 - k0 + rw - (BK - 1);
-        __syncwarp();
-#pragma unroll
-        for (int qq0 = 0; qq0 < 8 + BK - 1; qq0 += 32) {
-          const int qq = qq0 + lane;
-          if (qq < 8 + BK - 1) {
-            const int t = tb + qq;
-            const bool in = t > -n && t < n;
-            if constexpr (PREC == HSS_PREC_TF32X2) {
-              win64[qq] = in ? tterm64[t] : make_uint2(0u, 0u);
-            } else {
-#pragma unroll
-              for (int k = 0; k < T; ++k) win16[k * TW + qq] = in ? tterm16[k * tlen + t] : (uint16_t)0;
-            }
-          }
-        }
-        __syncwarp();
-        const bool clean = rows_ok && k0 + BK <= n && (k0 + BK <= wlo || k0 >= whi);
-#pragma unroll
-        for (int i2 = 0; i2 < 2; ++i2) {
-          const int idx = lane + 32 * i2, rl = idx % 8, c = idx / 8, r = rw + rl;
-          // window position of the chunk's first entry; the next entries
-          // step by +1 (orientation 1) or -1 (orientation 0)
-          const int q0 = TRANS ? c * EV - rl + 7 : rl - c * EV + (BK - 1);
-          constexpr int dq = TRANS ? 1 : -1;
-          uint4 chunk[T];
-          if (PREC == HSS_PREC_TF32X2 && clean) {
-            uint2 w[4];
-#pragma unroll
-            for (int e2 = 0; e2 < 4; ++e2) w[e2] = win64[q0 + dq * e2];
-            chunk[0] = make_uint4(w[0].x, w[1].x, w[2].x, w[3].x);
-            chunk[T - 1] = make_uint4(w[0].y, w[1].y, w[2].y, w[3].y);
-          } else if (PREC == HSS_PREC_TF32X2) {
-            const int gr = row0 + r, lo = lrow_lo[r], hi = lrow_hi[r];
-            uint2 w[4];
-#pragma unroll
-            for (int e2 = 0; e2 < 4; ++e2) {
-              const int gk = k0 + c * EV + e2;
-              const bool keep = gr < n && gk < n && (gk < lo || gk >= hi);
-              w[e2] = keep ? win64[q0 + dq * e2] : make_uint2(0u, 0u);
-            }
-            chunk[0] = make_uint4(w[0].x, w[1].x, w[2].x, w[3].x);
-            chunk[T - 1] = make_uint4(w[0].y, w[1].y, w[2].y, w[3].y);
-          } else if (clean) {
-#pragma unroll
-            for (int k = 0; k < T; ++k) {
-              uint32_t wv[4];
-#pragma unroll
-              for (int e2 = 0; e2 < 4; ++e2)
-                wv[e2] = (uint32_t)win16[k * TW + q0 + dq * (2 * e2)] |
-                         ((uint32_t)win16[k * TW + q0 + dq * (2 * e2 + 1)] << 16);
-              chunk[k] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-            }
-          } else {
-            const int gr = row0 + r, lo = lrow_lo[r], hi = lrow_hi[r];
-#pragma unroll
-            for (int k = 0; k < T; ++k) {
-              uint32_t wv[4];
-#pragma unroll
-              for (int e2 = 0; e2 < 4; ++e2) {
-                uint32_t pair = 0u;
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                  const int x = 2 * e2 + hh;
+              for (int u = tid; u < BM * KC; u += NP) {
+                int r, c;
+                if (!TRANS) { r = u % BM; c = u / BM; }
+                else { r = (u / (8 * KC)) * 8 + (u % 8); c = (u / 8) % KC; }
+                const int gr = row0 + r, lo = lrow_lo[r], hi = lrow_hi[r];
+                double v[EV];
+      #pragma unroll
+                for (int x = 0; x < EV; ++x) {
                   const int gk = k0 + c * EV + x;
-                  const bool keep = gr < n && gk < n && (gk < lo || gk >= hi);
-                  pair |= (keep ? (uint32_t)win16[k * TW + q0 + dq * x] : 0u) << (16 * hh);
+                  double val = 0.0;
+                  if (gr < n && gk < n && (gk < lo || gk >= hi))
+                    val = TRANS ? entry_gen(a.src, gk, gr) : entry_gen(a.src, gr, gk);
+                  v[x] = val;
                 }
-                wv[e2] = pair;
+                uint4 chunk[T];
+                SP::split(v, chunk);
+                const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)c * 128u + (uint32_t)(r % 8) * 16u;
+      #pragma unroll
+                for (int t = 0; t < T; ++t) *(uint4*)(sp + t * TILE_A_BYTES + off) = chunk[t];
               }
-              chunk[k] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-            }
-          }
-          const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)c * 128u + (uint32_t)(r % 8) * 16u;
-#pragma unroll
-          for (int t = 0; t < T; ++t) *(uint4*)(sp + t * TILE_A_BYTES + off) = chunk[t];
-        }
-      } else {
-        for (int u = tid; u < BM * KC; u += NP) {
-          int r, c;
-          if (!TRANS) { r = u % BM; c = u / BM; }
-          else { r = (u / (8 * KC)) * 8 + (u % 8); c = (u / 8) % KC; }
-          const int gr = row0 + r, lo = lrow_lo[r], hi = lrow_hi[r];
-          double v[EV];
-#pragma unroll
-          for (int x = 0; x < EV; ++x) {
-            const int gk = k0 + c * EV + x;
-            double val = 0.0;
-            if (gr < n && gk < n && (gk < lo || gk >= hi))
-              val = TRANS ? entry_gen(a.src, gk, gr) : entry_gen(a.src, gr, gk);
-            v[x] = val;
-          }
-          uint4 chunk[T];
-          SP::split(v, chunk);
-          const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)c * 128u + (uint32_t)(r % 8) * 16u;
-#pragma unroll
-          for (int t = 0; t < T; ++t) *(uint4*)(sp + t * TILE_A_BYTES + off) = chunk[t];
-        }
-      }
       fence_async_smem();
       mbar_arrive(&full[st]);
       // after the last tile of chain c, drain chain c-1
@@ -350,6 +246,275 @@ __global__ void __maxnreg__(96) k_sample_tc_gen(TcArgs a) {
       mma_ktile<PREC>(smem_u32(smem + st * stage_bytes), tmem, N, b, first, id);
       mma_commit(&empty[st]);
       if (it % DR == DR - 1 || it == nk - 1) mma_commit(&tfull[b]);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == GEN_WARPS) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"((uint32_t)a.tmem_cols)
+                 : "memory");
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Toeplitz kernel.  A tile of a Toeplitz matrix is made of few different core
+// matrices (8 rows x 16 bytes): the one of row group R and K chunk c holds the
+// diagonals around 8 R - EV c (EV elements per chunk), so a 128 x BK tile has
+// 15 (8 / EV) + BK / EV of them instead of 16 BK / EV, and the tile of the next
+// k-tile shifts by BK / EV.  The producers therefore write one strip of core
+// matrices, in the order of their diagonal, for up to J k-tiles at a time (an
+// epoch), and the tensor core reads every tile out of it: stepping R by one
+// moves the shared-memory address by SBO = 8 / EV core matrices, stepping c
+// back by one moves it by LBO = one.  c runs backwards in the strip, so the two
+// chunks of an MMA come in swapped order, in R as well (packed with the chunks
+// of a pair exchanged): the sum of an MMA is the same.  What the strip cannot
+// hold, k-tiles that meet the rows' leaf blocks or reach past n, is staged
+// as whole masked tiles, one per epoch.
+//
+// Assembling every tile from a window of diagonals (sixteen warps, 2048 stores
+// of 16 bytes per k-tile) bounded the sampling at 1700 clocks per k-tile and
+// column tile; the strip takes about 100 stores per k-tile, which leaves the
+// TF32 MMAs (8 of 128 x 128 x 8, 512 clocks), the R tile's bulk copy (16 KB)
+// and the drains.  Two warps issue, one for the leading term's accumulator, one
+// for the corrections'.
+constexpr int TP_MMA = 2, TP_NSB = 6;
+constexpr int TP_THREADS = (GEN_WARPS + 1 + TP_MMA) * 32;
+
+template <int PREC>
+constexpr int toep_cores() { return 15 * (8 / Split<PREC>::EV) + Split<PREC>::BK / Split<PREC>::EV; }
+// k-tiles per epoch: the strip of a term fits the 16 KB of a whole tile
+template <int PREC>
+constexpr int toep_epoch() {
+  return (int)((TILE_A_BYTES / 128 - toep_cores<PREC>()) / (Split<PREC>::BK / Split<PREC>::EV)) + 1;
+}
+
+// The k-tiles [kt0, kt1) of a CTA cut into epochs.
+struct ToepEpochs {
+  int kt1, ku0, ku1, klast, J;   // masked: [ku0, ku1) and klast (-1: none)
+  __device__ __forceinline__ int length(int kt, bool& masked) const {
+    masked = (kt >= ku0 && kt < ku1) || kt == klast;
+    if (masked) return 1;
+    int end = kt1;
+    if (kt < ku0) end = min(end, ku0);
+    if (klast > kt) end = min(end, klast);
+    return min(J, end - kt);
+  }
+};
+
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0u;
+}
+
+template <int PREC, int NH, int TRANS>
+__global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
+  using SP = Split<PREC>;
+  constexpr int T = SP::T, EV = SP::EV, BK = SP::BK, KC = BK / EV, RS = 8 / EV;
+  constexpr int DR = drain_gen(PREC), NP = GEN_WARPS * 32;
+  constexpr uint32_t abuf = T * TILE_A_BYTES;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const int n = a.src.n, N = a.N;
+  const uint32_t tileB = (uint32_t)N * 128u;
+  uint8_t* sB = smem + 2 * abuf;
+  uint64_t* fullA = (uint64_t*)(sB + TP_NSB * tileB);
+  uint64_t* emptyA = fullA + 2;
+  uint64_t* fullB = emptyA + 2;
+  uint64_t* emptyB = fullB + TP_NSB;
+  uint64_t* tfull = emptyB + TP_NSB;
+  uint64_t* tempty = tfull + 2;
+  uint32_t* tmem_slot = (uint32_t*)(tempty + 2);
+  int* lrow_lo = (int*)(tmem_slot + 4);
+  int* lrow_hi = lrow_lo + BM;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const int rb = blockIdx.x, ct = blockIdx.y;
+  const int row0 = rb * BM, col0 = ct * N;
+  const int kt0 = (int)((long long)a.nkt * blockIdx.z / a.ksplit);
+  const int kt1 = (int)((long long)a.nkt * (blockIdx.z + 1) / a.ksplit);
+  const int nk = kt1 - kt0;
+  const int nchain = (nk + DR - 1) / DR;
+  if (tid == 0) {
+    for (int s = 0; s < 2; ++s) { mbar_init(&fullA[s], NP); mbar_init(&emptyA[s], TP_MMA); }
+    for (int s = 0; s < TP_NSB; ++s) { mbar_init(&fullB[s], 1); mbar_init(&emptyB[s], TP_MMA); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&tfull[b], TP_MMA); mbar_init(&tempty[b], GEN_WARPS); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (tid < BM) {
+    int r = row0 + tid, lo = 0x7fffffff, hi = 0x7fffffff;
+    if (r < n) leaf_range(r, n, a.leaf, lo, hi);
+    lrow_lo[tid] = lo;
+    lrow_hi[tid] = hi;
+  }
+  if (warp == GEN_WARPS) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"((uint32_t)a.tmem_cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    tc_fence_before();
+  }
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  // the leaves of the CTA's first and last row bound the masked k-tiles
+  ToepEpochs ep;
+  ep.kt1 = kt1;
+  ep.ku0 = lrow_lo[0] / BK;
+  ep.ku1 = (lrow_hi[min(BM, n - row0) - 1] + BK - 1) / BK;
+  ep.klast = n % BK ? a.nkt - 1 : -1;
+  ep.J = toep_epoch<PREC>();
+
+  if (warp < GEN_WARPS) {
+    const int q = warp % 4, h = warp / 4;
+    float s[NH], e[NH];
+#pragma unroll
+    for (int j = 0; j < NH; ++j) { s[j] = 0.f; e[j] = 0.f; }
+    const uint2* tterm64 = (const uint2*)a.toep + (n - 1);
+    const uint16_t* tterm16 = (const uint16_t*)a.toep + (n - 1);
+    const long long tlen = 2LL * n - 1;
+    // the EV elements of diagonals t, t + dt, ... as the chunks of the terms
+    auto chunk_of = [&](int t, int dt, uint4* out, auto&& keep) {
+      if constexpr (PREC == HSS_PREC_TF32X2) {
+        uint2 w[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int tx = t + dt * x;
+          w[x] = keep(x) && tx > -n && tx < n ? tterm64[tx] : make_uint2(0u, 0u);
+        }
+        out[0] = make_uint4(w[0].x, w[1].x, w[2].x, w[3].x);
+        out[T - 1] = make_uint4(w[0].y, w[1].y, w[2].y, w[3].y);
+      } else {
+#pragma unroll
+        for (int k = 0; k < T; ++k) {
+          uint32_t w[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const int ta = t + dt * (2 * x), tb = ta + dt;
+            const uint32_t lo = keep(2 * x) && ta > -n && ta < n ? tterm16[k * tlen + ta] : 0u;
+            const uint32_t hi = keep(2 * x + 1) && tb > -n && tb < n ? tterm16[k * tlen + tb] : 0u;
+            w[x] = lo | (hi << 16);
+          }
+          out[k] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+    };
+    auto produce = [&](int idx, int kt, int len, bool masked) -> bool {
+      const int buf = idx & 1;
+      if (!mbar_wait_warp(&emptyA[buf], ((uint32_t)(idx >> 1) & 1u) ^ 1u, a.err, 2)) return false;
+      uint8_t* dst = smem + buf * abuf;
+      if (!masked) {
+        // core matrix m of the strip: diagonals d + rho - x, d = row0 - (last
+        // k-tile's first column) + EV (m - (KC - 1))
+        const int d0 = row0 - (kt + len - 1) * BK - EV * (KC - 1), cores = toep_cores<PREC>() + KC * (len - 1);
+        for (int u = tid; u < cores * 8; u += NP) {
+          const int m = u / 8, rho = u % 8, d = d0 + EV * m + rho;
+          uint4 ch[T];
+          chunk_of(TRANS ? -d : d, TRANS ? 1 : -1, ch, [](int) { return true; });
+#pragma unroll
+          for (int t = 0; t < T; ++t) *(uint4*)(dst + t * TILE_A_BYTES + (uint32_t)u * 16u) = ch[t];
+        }
+      } else {
+        const int k0 = kt * BK;
+        for (int u = tid; u < BM * KC; u += NP) {
+          const int r = u % BM, c = u / BM, gr = row0 + r, lo = lrow_lo[r], hi = lrow_hi[r];
+          const int d = gr - k0 - c * EV;
+          uint4 ch[T];
+          chunk_of(TRANS ? -d : d, TRANS ? 1 : -1, ch, [&](int x) {
+            const int gk = k0 + c * EV + x;
+            return gr < n && gk < n && (gk < lo || gk >= hi);
+          });
+          const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)(c ^ 1) * 128u + (uint32_t)(r % 8) * 16u;
+#pragma unroll
+          for (int t = 0; t < T; ++t) *(uint4*)(dst + t * TILE_A_BYTES + off) = ch[t];
+        }
+      }
+      fence_async_smem();
+      mbar_arrive(&fullA[buf]);
+      return true;
+    };
+    // epoch i + 1 is written before the chains that end in epoch i are drained
+    bool ok = true, masked = false;
+    int kt = kt0, drained = 0, idx = 0;
+    int len = nk > 0 ? ep.length(kt, masked) : 0;
+    if (len > 0) ok = produce(0, kt, len, masked);
+    while (ok && len > 0) {
+      const int kn = kt + len;
+      bool nm = false;
+      const int nl = kn < kt1 ? ep.length(kn, nm) : 0;
+      if (nl > 0) ok = produce(++idx, kn, nl, nm);
+      const int done = kn == kt1 ? nchain : (kn - kt0) / DR;   // chains that end by here
+      for (; ok && drained < done; ++drained) {
+        const int b = drained & 1;
+        if (!mbar_wait_warp(&tfull[b], (uint32_t)(drained >> 1) & 1u, a.err, 6)) { ok = false; break; }
+        tc_fence_after();
+        drain_chain<NH>(tmem, N, b, q, h, s, e);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[b]);
+      }
+      kt = kn;
+      len = nl;
+    }
+    if (ok) store_row<NH>(a.S, a.lds, n, a.ncols, row0 + 32 * q + lane, col0 + h * NH, a.atomic, s, e);
+  } else if (warp == GEN_WARPS) {
+    // ---------------------------------------------------------- copies of R
+    if (lane == 0) {
+      const uint8_t* gB = a.Rp + ((size_t)ct * a.nkt + kt0) * tileB;
+      int st = 0;
+      uint32_t ph = 0u;
+      for (int it = 0; it < nk; ++it) {
+        if (it > 0 && ++st == TP_NSB) { st = 0; ph ^= 1u; }
+        if (!mbar_wait(&emptyB[st], ph ^ 1u, a.err, 4)) break;
+        mbar_expect_tx(&fullB[st], tileB);
+        bulk_g2s(sB + st * tileB, gB + (size_t)it * tileB, tileB, &fullB[st]);
+      }
+    }
+  } else {
+    // ------------------------------------------- MMA issuers: 0 HI, 1 LO
+    const int g = warp - GEN_WARPS - 1;
+    const uint32_t id = idesc(SP::FMT, (uint32_t)N);
+    const bool one = elect_one();
+    bool ok = true, masked = false;
+    int st = 0, it = 0;
+    uint32_t ph = 0u;
+    for (int kt = kt0, idx = 0; ok && kt < kt1; ++idx) {
+      const int len = ep.length(kt, masked), buf = idx & 1;
+      if (!mbar_wait_warp(&fullA[buf], (uint32_t)(idx >> 1) & 1u, a.err, 3)) break;
+      const uint32_t sa = smem_u32(smem + buf * abuf);
+      for (int j = 0; j < len; ++j, ++it) {
+        if (it > 0 && ++st == TP_NSB) { st = 0; ph ^= 1u; }
+        const int c = it / DR, b = c & 1;
+        const bool first = (it % DR) == 0;
+        if (first && !mbar_wait_warp(&tempty[b], ((uint32_t)(c >> 1) & 1u) ^ 1u, a.err, 8)) { ok = false; break; }
+        if (!mbar_wait_warp(&fullB[st], ph, a.err, 5)) { ok = false; break; }
+        tc_fence_after();
+        if (one) {
+          const uint64_t bd = sdesc(smem_u32(sB + st * tileB), 128u, 1024u);
+          // chunk 2 ks + 1 of the tile's first row group, then LBO on to 2 ks
+          const uint64_t ad = masked ? sdesc(sa, 128u, 1024u)
+                                     : sdesc(sa + 128u * (uint32_t)(KC - 2 + KC * (len - 1 - j)), 128u, RS * 128u);
+          const uint32_t d = tmem + (uint32_t)((2 * b + g) * N);
+#pragma unroll
+          for (int ks = 0; ks < BK / SP::KSTEP; ++ks) {
+            const uint64_t ak = masked ? ad + (uint64_t)(ks * 16) : ad - (uint64_t)(ks * 16);   // 256 bytes
+            const uint64_t bk = bd + (uint64_t)(ks * 16);
+            if (g == 0) {
+              mma<PREC>(d, ak, bk, id, (first && ks == 0) ? 0u : 1u);
+            } else {
+#pragma unroll
+              for (int t = 1; t < T; ++t)
+                mma<PREC>(d, ak + (uint64_t)((t * TILE_A_BYTES) >> 4), bk, id, (first && ks == 0 && t == 1) ? 0u : 1u);
+            }
+          }
+          mma_commit(&emptyB[st]);
+          if (it % DR == DR - 1 || it == nk - 1) mma_commit(&tfull[b]);
+          if (j == len - 1) mma_commit(&emptyA[buf]);
+        }
+        __syncwarp();
+      }
+      kt += len;
     }
   }
   tc_fence_before();
@@ -416,7 +581,7 @@ __global__ void __launch_bounds__(256) k_pack_a(SrcDev src, int leaf, int nrb, i
 
 template <int PREC>
 __global__ void __launch_bounds__(256) k_pack_r(const double* R, long long ldr, int n, int ncols, int N,
-                                                int nkt, uint8_t* out) {
+                                                int nkt, int swap, uint8_t* out) {
   using SP = Split<PREC>;
   constexpr int EV = SP::EV, BK = SP::BK, KC = BK / EV;
   const int tile = blockIdx.x, ct = tile / nkt, kt = tile % nkt;
@@ -430,7 +595,7 @@ __global__ void __launch_bounds__(256) k_pack_r(const double* R, long long ldr, 
       const int gk = kt * BK + c * EV + x;
       v[x] = (gc < ncols && gk < n) ? R[(long long)gk + (long long)gc * ldr] : 0.0;
     }
-    const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)c * 128u + (uint32_t)(r % 8) * 16u;
+    const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)(c ^ swap) * 128u + (uint32_t)(r % 8) * 16u;
     *(uint4*)(dst + off) = SP::pack_r(v);
   }
 }
@@ -581,25 +746,26 @@ cudaError_t launch_packed_t(const TcPackedArgs& a, int gx, int gy, cudaStream_t 
 template <int PREC>
 cudaError_t launch_gen_t(const TcArgs& a, int gx, int gy, cudaStream_t st) {
   constexpr int T = Split<PREC>::T;
-  const size_t sm = (size_t)NSTAGE * (T * TILE_A_BYTES + (size_t)a.N * 128) + 8 * (2 * NSTAGE + 4) + 16 +
-                    2 * BM * sizeof(int) + (size_t)GEN_WARPS * T * TW * sizeof(uint32_t) + 1024;
-  dim3 grid(gx, gy, a.ksplit);
-#define HSS_LAUNCH_GEN(NHV, TR)                                                                     \
-  do {                                                                                              \
-    cudaError_t e = cudaFuncSetAttribute(k_sample_tc_gen<PREC, NHV, TR>,                            \
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);     \
-    if (e != cudaSuccess) return e;                                                                 \
-    k_sample_tc_gen<PREC, NHV, TR><<<grid, GEN_THREADS, sm, st>>>(a);                               \
-  } while (0)
-  if (a.N == 64) {
-    if (a.trans) HSS_LAUNCH_GEN(16, 1);
-    else HSS_LAUNCH_GEN(16, 0);
-  } else {
-    if (a.trans) HSS_LAUNCH_GEN(32, 1);
-    else HSS_LAUNCH_GEN(32, 0);
+  const dim3 grid(gx, gy, a.ksplit);
+  const bool toep = a.toep != nullptr;
+  const size_t sm = toep ? (size_t)2 * T * TILE_A_BYTES + (size_t)TP_NSB * a.N * 128 + 8 * (2 * TP_NSB + 8) + 16 +
+                               2 * BM * sizeof(int) + 1024
+                         : (size_t)NSTAGE * (T * TILE_A_BYTES + (size_t)a.N * 128) + 8 * (2 * NSTAGE + 4) + 16 +
+                               2 * BM * sizeof(int) + 1024;
+  auto run = [&](auto* kernel, int threads) -> cudaError_t {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, threads, sm, st>>>(a);
+    return cudaGetLastError();
+  };
+  if (toep) {
+    if (a.N == 64)
+      return a.trans ? run(k_sample_tc_toep<PREC, 16, 1>, TP_THREADS) : run(k_sample_tc_toep<PREC, 16, 0>, TP_THREADS);
+    return a.trans ? run(k_sample_tc_toep<PREC, 32, 1>, TP_THREADS) : run(k_sample_tc_toep<PREC, 32, 0>, TP_THREADS);
   }
-#undef HSS_LAUNCH_GEN
-  return cudaGetLastError();
+  if (a.N == 64)
+    return a.trans ? run(k_sample_tc_gen<PREC, 16, 1>, GEN_THREADS) : run(k_sample_tc_gen<PREC, 16, 0>, GEN_THREADS);
+  return a.trans ? run(k_sample_tc_gen<PREC, 32, 1>, GEN_THREADS) : run(k_sample_tc_gen<PREC, 32, 0>, GEN_THREADS);
 }
 
 int bk_of(int precision) { return precision == HSS_PREC_TF32X2 ? 32 : 64; }
@@ -657,15 +823,15 @@ cudaError_t launch_pack_a(const SrcDev& src, int leaf, int precision, int orient
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack_r(const double* R, long long ldr, int n, int ncols, int precision, void* out,
-                          cudaStream_t st) {
+cudaError_t launch_pack_r(const double* R, long long ldr, int n, int ncols, int precision, bool toep,
+                          void* out, cudaStream_t st) {
   if (n <= 0 || ncols <= 0) return cudaSuccess;
-  const int bk = bk_of(precision);
+  const int bk = bk_of(precision), swap = toep ? 1 : 0;
   const int N = tile_n(ncols), nct = (ncols + N - 1) / N, nkt = (n + bk - 1) / bk;
   if (precision == HSS_PREC_TF32X2)
-    k_pack_r<HSS_PREC_TF32X2><<<nct * nkt, 256, 0, st>>>(R, ldr, n, ncols, N, nkt, (uint8_t*)out);
+    k_pack_r<HSS_PREC_TF32X2><<<nct * nkt, 256, 0, st>>>(R, ldr, n, ncols, N, nkt, swap, (uint8_t*)out);
   else
-    k_pack_r<HSS_PREC_BF16X3><<<nct * nkt, 256, 0, st>>>(R, ldr, n, ncols, N, nkt, (uint8_t*)out);
+    k_pack_r<HSS_PREC_BF16X3><<<nct * nkt, 256, 0, st>>>(R, ldr, n, ncols, N, nkt, swap, (uint8_t*)out);
   return cudaGetLastError();
 }
 
