@@ -277,10 +277,12 @@ __global__ void __maxnreg__(96) k_sample_tc_gen(TcArgs a) {
 // of 16 bytes per k-tile) bounded the sampling at 1700 clocks per k-tile and
 // column tile; the strip takes about 100 stores per k-tile, which leaves the
 // TF32 MMAs (8 of 128 x 128 x 8, 512 clocks), the R tile's bulk copy (16 KB)
-// and the drains.  Two warps issue, one for the leading term's accumulator, one
-// for the corrections'.
-constexpr int TP_MMA = 2, TP_NSB = 6;
-constexpr int TP_THREADS = (GEN_WARPS + 1 + TP_MMA) * 32;
+// and the drains.  Two warps write the strips (drain warps that wrote them kept
+// the tensor core waiting for its buffers: 61 -> 32 ms at n = 131072 and 256
+// columns, in warps of their own 27 ms, 0.67 of the measured tensor rate).
+constexpr int TP_NSB = 6;     // stages of R tiles
+constexpr int TP_STRIP = 2;   // strip warps
+constexpr int TP_THREADS = (GEN_WARPS + 2 + TP_STRIP) * 32;   // drains, copies, MMAs, strips
 
 template <int PREC>
 constexpr int toep_cores() { return 15 * (8 / Split<PREC>::EV) + Split<PREC>::BK / Split<PREC>::EV; }
@@ -313,7 +315,7 @@ template <int PREC, int NH, int TRANS>
 __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
   using SP = Split<PREC>;
   constexpr int T = SP::T, EV = SP::EV, BK = SP::BK, KC = BK / EV, RS = 8 / EV;
-  constexpr int DR = drain_gen(PREC), NP = GEN_WARPS * 32;
+  constexpr int DR = drain_gen(PREC);
   constexpr uint32_t abuf = T * TILE_A_BYTES;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int n = a.src.n, N = a.N;
@@ -336,9 +338,9 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
   const int nk = kt1 - kt0;
   const int nchain = (nk + DR - 1) / DR;
   if (tid == 0) {
-    for (int s = 0; s < 2; ++s) { mbar_init(&fullA[s], NP); mbar_init(&emptyA[s], TP_MMA); }
-    for (int s = 0; s < TP_NSB; ++s) { mbar_init(&fullB[s], 1); mbar_init(&emptyB[s], TP_MMA); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&tfull[b], TP_MMA); mbar_init(&tempty[b], GEN_WARPS); }
+    for (int s = 0; s < 2; ++s) { mbar_init(&fullA[s], 32 * TP_STRIP); mbar_init(&emptyA[s], 1); }
+    for (int s = 0; s < TP_NSB; ++s) { mbar_init(&fullB[s], 1); mbar_init(&emptyB[s], 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], GEN_WARPS); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < BM) {
@@ -371,6 +373,20 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
     float s[NH], e[NH];
 #pragma unroll
     for (int j = 0; j < NH; ++j) { s[j] = 0.f; e[j] = 0.f; }
+    bool ok = true;
+    for (int cd = 0; cd < nchain; ++cd) {
+      const int b = cd & 1;
+      if (!mbar_wait_warp(&tfull[b], (uint32_t)(cd >> 1) & 1u, a.err, 6)) { ok = false; break; }
+      tc_fence_after();
+      drain_chain<NH>(tmem, N, b, q, h, s, e);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[b]);
+    }
+    if (ok) store_row<NH>(a.S, a.lds, n, a.ncols, row0 + 32 * q + lane, col0 + h * NH, a.atomic, s, e);
+  } else if (warp >= GEN_WARPS + 2) {
+    // ------------------------------------------------------------ strips of A
+    const int tl = tid - (GEN_WARPS + 2) * 32;
     const uint2* tterm64 = (const uint2*)a.toep + (n - 1);
     const uint16_t* tterm16 = (const uint16_t*)a.toep + (n - 1);
     const long long tlen = 2LL * n - 1;
@@ -408,7 +424,8 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
         // core matrix m of the strip: diagonals d + rho - x, d = row0 - (last
         // k-tile's first column) + EV (m - (KC - 1))
         const int d0 = row0 - (kt + len - 1) * BK - EV * (KC - 1), cores = toep_cores<PREC>() + KC * (len - 1);
-        for (int u = tid; u < cores * 8; u += NP) {
+#pragma unroll 4
+        for (int u = tl; u < cores * 8; u += 32 * TP_STRIP) {
           const int m = u / 8, rho = u % 8, d = d0 + EV * m + rho;
           uint4 ch[T];
           chunk_of(TRANS ? -d : d, TRANS ? 1 : -1, ch, [](int) { return true; });
@@ -417,7 +434,7 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
         }
       } else {
         const int k0 = kt * BK;
-        for (int u = tid; u < BM * KC; u += NP) {
+        for (int u = tl; u < BM * KC; u += 32 * TP_STRIP) {
           const int r = u % BM, c = u / BM, gr = row0 + r, lo = lrow_lo[r], hi = lrow_hi[r];
           const int d = gr - k0 - c * EV;
           uint4 ch[T];
@@ -434,30 +451,12 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
       mbar_arrive(&fullA[buf]);
       return true;
     };
-    // epoch i + 1 is written before the chains that end in epoch i are drained
-    bool ok = true, masked = false;
-    int kt = kt0, drained = 0, idx = 0;
-    int len = nk > 0 ? ep.length(kt, masked) : 0;
-    if (len > 0) ok = produce(0, kt, len, masked);
-    while (ok && len > 0) {
-      const int kn = kt + len;
-      bool nm = false;
-      const int nl = kn < kt1 ? ep.length(kn, nm) : 0;
-      if (nl > 0) ok = produce(++idx, kn, nl, nm);
-      const int done = kn == kt1 ? nchain : (kn - kt0) / DR;   // chains that end by here
-      for (; ok && drained < done; ++drained) {
-        const int b = drained & 1;
-        if (!mbar_wait_warp(&tfull[b], (uint32_t)(drained >> 1) & 1u, a.err, 6)) { ok = false; break; }
-        tc_fence_after();
-        drain_chain<NH>(tmem, N, b, q, h, s, e);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[b]);
-      }
-      kt = kn;
-      len = nl;
+    bool masked = false;
+    for (int kt = kt0, idx = 0; kt < kt1; ++idx) {
+      const int len = ep.length(kt, masked);
+      if (!produce(idx, kt, len, masked)) break;
+      kt += len;
     }
-    if (ok) store_row<NH>(a.S, a.lds, n, a.ncols, row0 + 32 * q + lane, col0 + h * NH, a.atomic, s, e);
   } else if (warp == GEN_WARPS) {
     // ---------------------------------------------------------- copies of R
     if (lane == 0) {
@@ -472,8 +471,7 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
       }
     }
   } else {
-    // ------------------------------------------- MMA issuers: 0 HI, 1 LO
-    const int g = warp - GEN_WARPS - 1;
+    // --------------------------------------------------------- MMA issuer
     const uint32_t id = idesc(SP::FMT, (uint32_t)N);
     const bool one = elect_one();
     bool ok = true, masked = false;
@@ -495,18 +493,15 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
           // chunk 2 ks + 1 of the tile's first row group, then LBO on to 2 ks
           const uint64_t ad = masked ? sdesc(sa, 128u, 1024u)
                                      : sdesc(sa + 128u * (uint32_t)(KC - 2 + KC * (len - 1 - j)), 128u, RS * 128u);
-          const uint32_t d = tmem + (uint32_t)((2 * b + g) * N);
+          const uint32_t hi = tmem + (uint32_t)((2 * b) * N), lo = hi + (uint32_t)N;
 #pragma unroll
           for (int ks = 0; ks < BK / SP::KSTEP; ++ks) {
             const uint64_t ak = masked ? ad + (uint64_t)(ks * 16) : ad - (uint64_t)(ks * 16);   // 256 bytes
             const uint64_t bk = bd + (uint64_t)(ks * 16);
-            if (g == 0) {
-              mma<PREC>(d, ak, bk, id, (first && ks == 0) ? 0u : 1u);
-            } else {
+            mma<PREC>(hi, ak, bk, id, (first && ks == 0) ? 0u : 1u);
 #pragma unroll
-              for (int t = 1; t < T; ++t)
-                mma<PREC>(d, ak + (uint64_t)((t * TILE_A_BYTES) >> 4), bk, id, (first && ks == 0 && t == 1) ? 0u : 1u);
-            }
+            for (int t = 1; t < T; ++t)
+              mma<PREC>(lo, ak + (uint64_t)((t * TILE_A_BYTES) >> 4), bk, id, (first && ks == 0 && t == 1) ? 0u : 1u);
           }
           mma_commit(&emptyB[st]);
           if (it % DR == DR - 1 || it == nk - 1) mma_commit(&tfull[b]);
