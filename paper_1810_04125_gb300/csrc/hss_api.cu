@@ -377,6 +377,7 @@ struct hss_matrix_s {
   bool same_samples = false;   // mixed forms, A = A^T: S^c is a copy of S^r
   void* packA = nullptr;   // packed tensor-core tiles of a dense A (during compress)
   XsKeep xs;               // digits of a generated source (during compress, plain form)
+  float4* pts = nullptr;      // a Laplace source's points split for FP32 (during compress, mixed forms)
   void* toep_terms = nullptr; // a Toeplitz source's diagonals split into terms (during compress)
   bool usable = false;
   bool partial = false;    // not converged; the uncompressed part kept dense (F12, F21)
@@ -387,6 +388,7 @@ struct hss_matrix_s {
   ~hss_matrix_s() {
     if (packA) cudaFree(packA);
     if (toep_terms) cudaFree(toep_terms);
+    if (pts) cudaFree(pts);
     if (xs.pa[0]) cudaFree(xs.pa[0]);
     arena.release();
   }
@@ -485,6 +487,7 @@ SrcDev make_src(const hss_source& s, const int* leaf_id) {
   d.p0 = s.p0;
   d.p1 = s.p1;
   d.leaf_id = leaf_id;
+  d.pts = nullptr;
   return d;
 }
 
@@ -1153,6 +1156,14 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
   }
   SrcDev s = make_src(H->src, H->leaf_id);
   const double* Rc = H->R + (long long)c0 * n;
+  if (H->src.kind == HSS_SRC_LAPLACE && H->o.precision != HSS_PREC_FP64) {
+    if (!H->pts) {
+      CK(dmalloc_async(&H->pts, sizeof(float4) * 2 * (size_t)n, st));
+      CK(launch_split_points(s, H->pts, st));
+      c.launches++;
+    }
+    s.pts = H->pts;
+  }
   const int norient = H->sym ? 1 : 2;   // A^T R is A R for a symmetric A
   const bool one_side = H->sym || H->same_samples;
   auto copy_samples = [&]() -> hss_status {
@@ -1219,9 +1230,10 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
       if (!one_side) CK(cudaMemset2DAsync(H->Sg_c + c0, sizeof(double) * H->dmax, 0, sizeof(double) * w, n, st));
     }
     CK(c.timer.mark(PH_SAMPLE, st));
-    CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 0, H->Sg_r + c0, H->dmax, c.d_flag + 1, st));
+    const int ks = sample_tc_packed_ksplit(n, w, H->o.precision);
+    CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 0, ks, H->Sg_r + c0, H->dmax, c.d_flag + 1, st));
     if (!one_side)
-      CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 1, H->Sg_c + c0, H->dmax, c.d_flag + 1,
+      CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 1, ks, H->Sg_c + c0, H->dmax, c.d_flag + 1,
                                  st));
     CKS(copy_samples());
     c.launches += one_side ? 1 : 2;
@@ -2245,6 +2257,10 @@ hss_status compress_all(Ctx& c, const std::vector<const hss_source*>& A, const s
     if (H->toep_terms) {
       CK(cudaFreeAsync(H->toep_terms, c.st));
       H->toep_terms = nullptr;
+    }
+    if (H->pts) {
+      CK(cudaFreeAsync(H->pts, c.st));
+      H->pts = nullptr;
     }
     if (H->xs.pa[0]) {
       CK(cudaFreeAsync(H->xs.pa[0], c.st));
@@ -3313,12 +3329,34 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   void* pA = nullptr;
   void* pR = nullptr;
   void* tt = nullptr;
-  const bool packed = A->kind == HSS_SRC_DENSE;
+  // BF16 x 3 point kernels are packed too where the tiles take at most 4 GB and
+  // there is room for them: their chains are as long in both kernels (with the
+  // same split of K the samples are the same bits), and the pack kernel, without
+  // accumulators to hold, generates faster (Laplace, 128 columns: 6.1 ps an entry
+  // at n = 26000 packed, 8.4 at n = 27000 generated in the product kernel)
+  bool packed = A->kind == HSS_SRC_DENSE;
+  const bool both = packed;   // a point kernel is symmetric: one orientation
+  if ((A->kind == HSS_SRC_LAPLACE || A->kind == HSS_SRC_GAUSS) && precision == HSS_PREC_BF16X3) {
+    const size_t pb = packed_a_bytes(n, precision, 1);
+    if (pb <= (size_t(4) << 30)) {
+      if (dmalloc_async(&pA, pb, st) == cudaSuccess) packed = true;
+      else {
+        cudaGetLastError();
+        pA = nullptr;
+      }
+    }
+  }
+  float4* pts = nullptr;
+  if (A->kind == HSS_SRC_LAPLACE) {
+    CK(dmalloc_async(&pts, sizeof(float4) * 2 * (size_t)n, st));
+    CK(launch_split_points(s, pts, st));
+    s.pts = pts;
+  }
   CK(dmalloc_async(&pR, packed_r_bytes(n, ncols, precision), st));
   CK(launch_pack_r(Rr, n, n, ncols, precision, A->kind == HSS_SRC_TOEPLITZ, pR, st));
   if (packed) {
-    CK(dmalloc_async(&pA, packed_a_bytes(n, precision, 2), st));
-    CK(launch_pack_a(s, leaf, precision, 2, pA, st));
+    if (!pA) CK(dmalloc_async(&pA, packed_a_bytes(n, precision, 2), st));
+    CK(launch_pack_a(s, leaf, precision, both ? 2 : 1, pA, st));
   } else if (A->kind == HSS_SRC_TOEPLITZ) {
     CK(dmalloc_async(&tt, toeplitz_terms_bytes(n, precision), st));
     CK(launch_toeplitz_terms(s, precision, tt, st));
@@ -3331,13 +3369,15 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
                            cudaMemcpyDeviceToDevice, st));
       continue;
     }
-    const int ks = packed ? sample_tc_packed_ksplit(n, ncols, precision) : sample_tc_ksplit(n, ncols, precision);
+    const int ks = A->kind == HSS_SRC_DENSE ? sample_tc_packed_ksplit(n, ncols, precision)
+                                            : sample_tc_ksplit(n, ncols, precision);
     if (ks > 1) CK(cudaMemset2DAsync(S, sizeof(double) * lds, 0, sizeof(double) * ncols, n, st));
     int at = 0;
-    if (packed) CK(launch_sample_tc_packed(pA, pR, n, ncols, precision, side, S, lds, err, st));
+    if (packed) CK(launch_sample_tc_packed(pA, pR, n, ncols, precision, both ? side : 0, ks, S, lds, err, st));
     else CK(launch_sample_tc(s, leaf, precision, side, ncols, pR, S, lds, err, &at, tt, st));
   }
   if (packed) CK(cudaFreeAsync(pA, st));
+  if (pts) CK(cudaFreeAsync(pts, st));
   if (tt) CK(cudaFreeAsync(tt, st));
   CK(cudaFreeAsync(pR, st));
   int herr = 0;

@@ -18,6 +18,8 @@ struct SrcDev {
   long long ld;
   double p0, p1;
   const int* leaf_id;   // n entries (leaves numbered level by level)
+  const float4* pts;    // LAPLACE, mixed forms: the points split for the FP32
+                        // evaluation (launch_split_points), 2 per point, or NULL
 };
 
 // Entry A(i, j) in FP64 (the definitions of HSS_SRC_*).
@@ -221,6 +223,8 @@ cudaError_t launch_sample_fp64(const SrcDev& src, int ncols, const double* R, lo
 cudaError_t launch_sample_tc(const SrcDev& src, int leaf, int precision, int trans, int ncols,
                              const void* Rp, double* S, long long lds, int* err, int* used_atomic,
                              const void* toep, cudaStream_t st);
+// src.pts of a Laplace source: 2 n float4
+cudaError_t launch_split_points(const SrcDev& src, float4* out, cudaStream_t st);
 size_t toeplitz_terms_bytes(int n, int precision);
 cudaError_t launch_toeplitz_terms(const SrcDev& src, int precision, void* out, cudaStream_t st);
 int sample_tc_ksplit(int n, int ncols, int precision);
@@ -235,7 +239,7 @@ cudaError_t launch_pack_r(const double* R, long long ldr, int n, int ncols, int 
                           cudaStream_t st);
 int sample_tc_packed_ksplit(int n, int ncols, int precision);
 cudaError_t launch_sample_tc_packed(const void* A, const void* Rp, int n, int ncols, int precision,
-                                    int trans, double* S, long long lds, int* err, cudaStream_t st);
+                                    int trans, int ksplit, double* S, long long lds, int* err, cudaStream_t st);
 // out(:, c) = R rounded to the significand of the mixed format (mode 1: 11
 // bits, TF32; mode 2: 8 bits, BF16)
 cudaError_t launch_round_copy(const double* in, long long ldin, double* out, long long ldout, int n,

@@ -57,6 +57,127 @@ __device__ __forceinline__ double entry_gen(const SrcDev& s, int i, int j) {
   return y1 * (1.0 / (4.0 * 3.141592653589793));
 }
 
+// The Laplace entry rounded to FP32, from points split into pairs of floats, on
+// the FP32 pipe (64 times the FP64 pipe's rate; entry_gen takes nine FP64
+// instructions and four conversions per entry, which bounded the generation).
+// The coordinate differences, their squares and the sum are kept as unevaluated
+// pairs with error-free additions and products (Dekker, Numer. Math. 18, 1971;
+// Knuth, TAOCP 2, 4.2.2), 1/sqrt by one Newton step of third order on the FP32
+// reciprocal square root with an exact residual: relative error below 2^-44.
+// Returns false, and the caller evaluates entry_gen, where that is not certain
+// to give entry_gen's FP32 value, so that the samples are the same bit for bit:
+// where the value is closer to a rounding boundary than what the two can differ
+// by, 2^-41 of it for the arithmetic of both and 2^-43 max|coordinate| / r for
+// the coordinates (split to 2^-48 of themselves, subtracted to 2^-46), or r^2 is
+// far from 1 (or not finite).  One entry in 2^15 at max|coordinate| / r = 2.
+// About 105 instructions an entry with the split, a third of the issue slots'
+// worth below what the pack kernel takes; n = 12000, 128 columns, BF16 x 3:
+// 6.44 ms with entry_gen, 1.04 ms so.
+__device__ __forceinline__ bool laplace_f32(const float4 ah, const float4 al, const float4 bh, const float4 bl,
+                                            float* out) {
+  float p[3], pe[3];
+  const float a1[3] = {ah.x, ah.y, ah.z}, a2[3] = {al.x, al.y, al.z};
+  const float b1[3] = {bh.x, bh.y, bh.z}, b2[3] = {bl.x, bl.y, bl.z};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float s = __fsub_rn(a1[c], b1[c]), t = __fsub_rn(s, a1[c]);
+    float e = __fsub_rn(__fsub_rn(a1[c], __fsub_rn(s, t)), __fadd_rn(b1[c], t));
+    e = __fadd_rn(e, __fsub_rn(a2[c], b2[c]));
+    p[c] = __fmul_rn(s, s);
+    pe[c] = __fmaf_rn(e, e, __fmaf_rn(__fadd_rn(s, s), e, __fmaf_rn(s, s, -p[c])));
+  }
+  auto two_sum = [](float x, float y, float& e) {
+    const float s = __fadd_rn(x, y), t = __fsub_rn(s, x);
+    e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, t)), __fsub_rn(y, t));
+    return s;
+  };
+  float e1, e2;
+  const float s1 = two_sum(p[0], p[1], e1), s2 = two_sum(s1, p[2], e2);
+  const float lo = __fadd_rn(__fadd_rn(e1, e2), __fadd_rn(__fadd_rn(pe[0], pe[1]), pe[2]));
+  const float h = __fadd_rn(s2, lo), l = __fsub_rn(lo, __fsub_rn(h, s2));
+  if (!(h >= 8.6736174e-19f && h <= 1.1529215e18f)) return false;   // 2^-60, 2^60
+  const float y = rsqrtf(h);
+  const float w = __fmul_rn(y, y), we = __fmaf_rn(y, y, -w);
+  const float t = __fmul_rn(h, w), te = __fmaf_rn(h, w, -t);
+  float e = __fsub_rn(__fsub_rn(1.0f, t), te);   // 1 - (h + l) y^2
+  e = __fmaf_rn(-h, we, e);
+  e = __fmaf_rn(-l, w, e);
+  const float corr = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, __fmul_rn(0.5f, e)));
+  // times 1 / (4 pi), as a pair
+  const double c4 = 1.0 / (4.0 * 3.141592653589793);
+  const float ch = (float)c4, cl = (float)(c4 - (double)(float)c4);
+  const float v = __fmul_rn(y, ch);
+  float ve = __fmaf_rn(y, ch, -v);
+  ve = __fmaf_rn(corr, ch, ve);
+  ve = __fmaf_rn(y, cl, ve);
+  const float f = __fadd_rn(v, ve), rem = __fsub_rn(ve, __fsub_rn(f, v));
+  const uint32_t u = __float_as_uint(f);
+  const float half_ulp = __uint_as_float((u & 0x7F800000u) - (24u << 23));
+  const float margin = __fmaf_rn(__fmul_rn(fmaxf(ah.w, bh.w), y), 1.13686838e-13f, 4.54747351e-13f);   // 2^-43, 2^-41
+  *out = f;
+  return __fmaf_rn(f, margin, fabsf(rem)) < half_ulp && (u & 0x7FFFFFu) != 0u;
+}
+
+__global__ void k_split_points(SrcDev src, float4* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= src.n) return;
+  float h[3], l[3], m = 0.f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double x = src.a[i + c * src.ld];
+    h[c] = (float)x;
+    l[c] = (float)(x - (double)h[c]);
+    m = fmaxf(m, fabsf(h[c]));
+  }
+  out[2 * i] = make_float4(h[0], h[1], h[2], m);
+  out[2 * i + 1] = make_float4(l[0], l[1], l[2], 0.f);
+}
+
+// The EV entries (row, k .. k + EV - 1) of A - D^(L) (trans: of its transpose)
+// as the chunks of their terms; lo, hi: the row's leaf.
+template <int PREC, bool TRANS>
+__device__ __forceinline__ void entry_chunk(const SrcDev& src, int gr, int k, int lo, int hi, uint4* chunk) {
+  using SP = Split<PREC>;
+  constexpr int EV = SP::EV;
+  const int n = src.n;
+  if (src.pts) {   // (symmetric: one evaluation for both orientations)
+    float v[EV];
+    const int ga = min(gr, n - 1);
+    const float4 ah = src.pts[2 * ga], al = src.pts[2 * ga + 1];
+    bool redo = false;
+#pragma unroll
+    for (int x = 0; x < EV; ++x) {
+      const int gk = k + x, gp = min(gk, n - 1);
+      const bool in = gr < n && gk < n && (gk < lo || gk >= hi);
+      float f;
+      const bool ok = laplace_f32(ah, al, src.pts[2 * gp], src.pts[2 * gp + 1], &f);
+      redo |= in && !ok;
+      v[x] = in ? f : 0.f;
+    }
+    if (redo) {   // rare: the eight again, so that the common path has no branch
+#pragma unroll 1
+      for (int x = 0; x < EV; ++x) {
+        const int gk = k + x;
+        const float f = gr < n && gk < n && (gk < lo || gk >= hi) ? to_f32(entry_gen(src, gr, gk)) : 0.f;
+#pragma unroll
+        for (int y = 0; y < EV; ++y)
+          if (y == x) v[y] = f;
+      }
+    }
+    SP::split(v, chunk);
+    return;
+  }
+  double v[EV];
+#pragma unroll
+  for (int x = 0; x < EV; ++x) {
+    const int gk = k + x;
+    double val = 0.0;
+    if (gr < n && gk < n && (gk < lo || gk >= hi)) val = TRANS ? entry_gen(src, gk, gr) : entry_gen(src, gr, gk);
+    v[x] = val;
+  }
+  SP::split(v, chunk);
+}
+
 // ---------------------------------------------------------------------------
 // Generating kernel (entries computed by the producer warps).
 // Warps 0-7: generate the A tile of each stage, drain chains, write the
@@ -185,26 +306,16 @@ __global__ void __maxnreg__(96) k_sample_tc_gen(TcArgs a) {
         bulk_g2s(sp + T * TILE_A_BYTES, gB + (size_t)it * tileB, tileB, &full[st]);
       }
       const int k0 = (kt0 + it) * BK;
-              for (int u = tid; u < BM * KC; u += NP) {
-                int r, c;
-                if (!TRANS) { r = u % BM; c = u / BM; }
-                else { r = (u / (8 * KC)) * 8 + (u % 8); c = (u / 8) % KC; }
-                const int gr = row0 + r, lo = lrow_lo[r], hi = lrow_hi[r];
-                double v[EV];
-      #pragma unroll
-                for (int x = 0; x < EV; ++x) {
-                  const int gk = k0 + c * EV + x;
-                  double val = 0.0;
-                  if (gr < n && gk < n && (gk < lo || gk >= hi))
-                    val = TRANS ? entry_gen(a.src, gk, gr) : entry_gen(a.src, gr, gk);
-                  v[x] = val;
-                }
-                uint4 chunk[T];
-                SP::split(v, chunk);
-                const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)c * 128u + (uint32_t)(r % 8) * 16u;
-      #pragma unroll
-                for (int t = 0; t < T; ++t) *(uint4*)(sp + t * TILE_A_BYTES + off) = chunk[t];
-              }
+      for (int u = tid; u < BM * KC; u += NP) {
+        int r, c;
+        if (!TRANS) { r = u % BM; c = u / BM; }
+        else { r = (u / (8 * KC)) * 8 + (u % 8); c = (u / 8) % KC; }
+        uint4 chunk[T];
+        entry_chunk<PREC, TRANS != 0>(a.src, row0 + r, k0 + c * EV, lrow_lo[r], lrow_hi[r], chunk);
+        const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)c * 128u + (uint32_t)(r % 8) * 16u;
+#pragma unroll
+        for (int t = 0; t < T; ++t) *(uint4*)(sp + t * TILE_A_BYTES + off) = chunk[t];
+      }
       fence_async_smem();
       mbar_arrive(&full[st]);
       // after the last tile of chain c, drain chain c-1
@@ -557,17 +668,9 @@ __global__ void __launch_bounds__(256) k_pack_a(SrcDev src, int leaf, int nrb, i
     int r, c;
     if (!o) { r = u % BM; c = u / BM; }
     else { r = (u / (8 * KC)) * 8 + (u % 8); c = (u / 8) % KC; }
-    const int gr = row0 + r, lo = rlo[r], hi = rhi[r];
-    double v[EV];
-#pragma unroll
-    for (int x = 0; x < EV; ++x) {
-      const int gk = k0 + c * EV + x;
-      double val = 0.0;
-      if (gr < n && gk < n && (gk < lo || gk >= hi)) val = o ? entry_gen(src, gk, gr) : entry_gen(src, gr, gk);
-      v[x] = val;
-    }
     uint4 chunk[T];
-    SP::split(v, chunk);
+    if (o) entry_chunk<PREC, true>(src, row0 + r, k0 + c * EV, rlo[r], rhi[r], chunk);
+    else entry_chunk<PREC, false>(src, row0 + r, k0 + c * EV, rlo[r], rhi[r], chunk);
     const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)c * 128u + (uint32_t)(r % 8) * 16u;
 #pragma unroll
     for (int t = 0; t < T; ++t) *(uint4*)(dst + t * TILE_A_BYTES + off) = chunk[t];
@@ -777,6 +880,12 @@ int ksplit_for(int gx, int gy, int nkt, int waves) {
 
 }  // namespace
 
+cudaError_t launch_split_points(const SrcDev& src, float4* out, cudaStream_t st) {
+  if (src.kind != HSS_SRC_LAPLACE || src.n <= 0) return cudaErrorInvalidValue;
+  k_split_points<<<(src.n + 127) / 128, 128, 0, st>>>(src, out);
+  return cudaGetLastError();
+}
+
 size_t toeplitz_terms_bytes(int n, int precision) {
   return (size_t)(2LL * n - 1) * (precision == HSS_PREC_TF32X2 ? 2 * 4 : 3 * 2);
 }
@@ -843,7 +952,7 @@ int sample_tc_ksplit(int n, int ncols, int precision) {
 }
 
 cudaError_t launch_sample_tc_packed(const void* A, const void* Rp, int n, int ncols, int precision,
-                                    int trans, double* S, long long lds, int* err, cudaStream_t st) {
+                                    int trans, int ksplit, double* S, long long lds, int* err, cudaStream_t st) {
   if (n <= 0 || ncols <= 0) return cudaSuccess;
   TcPackedArgs a;
   a.A = (const uint8_t*)A;
@@ -854,7 +963,7 @@ cudaError_t launch_sample_tc_packed(const void* A, const void* Rp, int n, int nc
   a.N = tile_n(ncols);
   a.ncols = ncols;
   a.tmem_cols = tmem_cols_for(a.N);
-  a.ksplit = sample_tc_packed_ksplit(n, ncols, precision);
+  a.ksplit = ksplit;
   a.trans = trans;
   a.drain = DRAIN_PACKED;
   a.S = S;

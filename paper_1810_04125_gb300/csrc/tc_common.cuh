@@ -138,6 +138,9 @@ __device__ __forceinline__ uint16_t bf16_bits(float x) {
 }
 __device__ __forceinline__ float bf16_val(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 
+__device__ __forceinline__ float to_f32(double x) { return __double2float_rn(x); }
+__device__ __forceinline__ float to_f32(float x) { return x; }
+
 template <int PREC>
 struct Split;
 
@@ -148,12 +151,13 @@ struct Split<HSS_PREC_TF32X2> {
   static constexpr int BK = 32;    // K per stage (128 bytes per row)
   static constexpr int KSTEP = 8;  // K per MMA
   static constexpr uint32_t FMT = 2;
-  // v: EV FP64 values -> T chunks of 16 bytes
-  __device__ static void split(const double* v, uint4* out) {
+  // v: EV FP64 (or already rounded FP32) values -> T chunks of 16 bytes
+  template <class V>
+  __device__ static void split(const V* v, uint4* out) {
     uint32_t h[4], l[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      float f = __double2float_rn(v[e]);
+      float f = to_f32(v[e]);
       float hi = round_tf32(f);
       float lo = round_tf32(f - hi);
       h[e] = __float_as_uint(hi);
@@ -175,14 +179,15 @@ struct Split<HSS_PREC_BF16X3> {
   static constexpr int BK = 64;
   static constexpr int KSTEP = 16;
   static constexpr uint32_t FMT = 1;
-  __device__ static void split(const double* v, uint4* out) {
+  template <class V>
+  __device__ static void split(const V* v, uint4* out) {
     uint32_t w[3][4];
 #pragma unroll
     for (int e = 0; e < 8; e += 2) {
       uint16_t b[3][2];
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        float f = __double2float_rn(v[e + q]);
+        float f = to_f32(v[e + q]);
         uint16_t b0 = bf16_bits(f);
         float r1 = f - bf16_val(b0);
         uint16_t b1 = bf16_bits(r1);
