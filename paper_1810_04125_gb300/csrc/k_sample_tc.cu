@@ -70,9 +70,9 @@ __device__ __forceinline__ double entry_gen(const SrcDev& s, int i, int j) {
 // by, 2^-41 of it for the arithmetic of both and 2^-43 max|coordinate| / r for
 // the coordinates (split to 2^-48 of themselves, subtracted to 2^-46), or r^2 is
 // far from 1 (or not finite).  One entry in 2^15 at max|coordinate| / r = 2.
-// About 105 instructions an entry with the split, a third of the issue slots'
-// worth below what the pack kernel takes; n = 12000, 128 columns, BF16 x 3:
-// 6.44 ms with entry_gen, 1.04 ms so.
+// About 105 instructions an entry with the split: 2.8 ps at full issue, and the
+// pack kernel takes 5.8.  n = 12000, 128 columns, BF16 x 3: 6.44 ms with
+// entry_gen, 1.04 ms so.
 __device__ __forceinline__ bool laplace_f32(const float4 ah, const float4 al, const float4 bh, const float4 bl,
                                             float* out) {
   float p[3], pe[3];
