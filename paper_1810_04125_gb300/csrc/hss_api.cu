@@ -1231,14 +1231,12 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
     }
     CK(c.timer.mark(PH_SAMPLE, st));
     const int ks = sample_tc_packed_ksplit(n, w, H->o.precision);
-    CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 0, ks, H->Sg_r + c0, H->dmax, c.d_flag + 1, st));
-    if (!one_side)
-      CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 1, ks, H->Sg_c + c0, H->dmax, c.d_flag + 1,
-                                 st));
+    CK(launch_sample_tc_packed(H->packA, packR, n, w, H->o.precision, 0, ks, H->Sg_r + c0,
+                               one_side ? nullptr : H->Sg_c + c0, H->dmax, c.d_flag + 1, st));
     CKS(copy_samples());
-    c.launches += one_side ? 1 : 2;
-    c.sample_launches += one_side ? 1 : 2;
-    H->st.sample_launches += one_side ? 1 : 2;
+    c.launches += 1;
+    c.sample_launches += 1;
+    H->st.sample_launches += 1;
     CK(c.timer.mark(PH_RNG, st));
     CK(cudaFreeAsync(packR, st));
   } else {
@@ -1265,9 +1263,9 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
       CK(launch_sample_tc(s, H->o.leaf, H->o.precision, 1, w, packR, H->Sg_c + c0, H->dmax, c.d_flag + 1, &at,
                           H->toep_terms, st));
     CKS(copy_samples());
-    c.launches += one_side ? 1 : 2;
-    c.sample_launches += one_side ? 1 : 2;
-    H->st.sample_launches += one_side ? 1 : 2;
+    c.launches += 1;
+    c.sample_launches += 1;
+    H->st.sample_launches += 1;
     CK(c.timer.mark(PH_RNG, st));
     CK(cudaFreeAsync(packR, st));
   }
@@ -3332,10 +3330,12 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   // BF16 x 3 point kernels are packed too where the tiles take at most 4 GB and
   // there is room for them: their chains are as long in both kernels (with the
   // same split of K the samples are the same bits), and the pack kernel, without
-  // accumulators to hold, generates faster (Laplace, 128 columns: 6.1 ps an entry
-  // at n = 26000 packed, 8.4 at n = 27000 generated in the product kernel)
+  // accumulators to hold, generates faster and one half of the matrix (Laplace, 128 columns:
+  // 4.4 ps an entry at n = 26000 packed, 8.2 at n = 27000 in the product kernel)
   bool packed = A->kind == HSS_SRC_DENSE;
-  const bool both = packed;   // a point kernel is symmetric: one orientation
+  // A point kernel is symmetric: one orientation serves both sides; a dense A
+  // has two, unless only its own is asked for.
+  const int orients = packed && Sc ? 2 : 1;
   if ((A->kind == HSS_SRC_LAPLACE || A->kind == HSS_SRC_GAUSS) && precision == HSS_PREC_BF16X3) {
     const size_t pb = packed_a_bytes(n, precision, 1);
     if (pb <= (size_t(4) << 30)) {
@@ -3355,8 +3355,8 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   CK(dmalloc_async(&pR, packed_r_bytes(n, ncols, precision), st));
   CK(launch_pack_r(Rr, n, n, ncols, precision, A->kind == HSS_SRC_TOEPLITZ, pR, st));
   if (packed) {
-    if (!pA) CK(dmalloc_async(&pA, packed_a_bytes(n, precision, 2), st));
-    CK(launch_pack_a(s, leaf, precision, both ? 2 : 1, pA, st));
+    if (!pA) CK(dmalloc_async(&pA, packed_a_bytes(n, precision, orients), st));
+    CK(launch_pack_a(s, leaf, precision, orients, pA, st));
   } else if (A->kind == HSS_SRC_TOEPLITZ) {
     CK(dmalloc_async(&tt, toeplitz_terms_bytes(n, precision), st));
     CK(launch_toeplitz_terms(s, precision, tt, st));
@@ -3373,7 +3373,12 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
                                             : sample_tc_ksplit(n, ncols, precision);
     if (ks > 1) CK(cudaMemset2DAsync(S, sizeof(double) * lds, 0, sizeof(double) * ncols, n, st));
     int at = 0;
-    if (packed) CK(launch_sample_tc_packed(pA, pR, n, ncols, precision, both ? side : 0, ks, S, lds, err, st));
+    if (packed && side == 0 && orients == 2 && Sc) {   // both sides at once
+      if (ks > 1) CK(cudaMemset2DAsync(Sc, sizeof(double) * lds, 0, sizeof(double) * ncols, n, st));
+      CK(launch_sample_tc_packed(pA, pR, n, ncols, precision, 0, ks, S, Sc, lds, err, st));
+      break;
+    }
+    if (packed) CK(launch_sample_tc_packed(pA, pR, n, ncols, precision, orients == 2 ? side : 0, ks, S, nullptr, lds, err, st));
     else CK(launch_sample_tc(s, leaf, precision, side, ncols, pR, S, lds, err, &at, tt, st));
   }
   if (packed) CK(cudaFreeAsync(pA, st));

@@ -239,7 +239,8 @@ cudaError_t launch_pack_r(const double* R, long long ldr, int n, int ncols, int 
                           cudaStream_t st);
 int sample_tc_packed_ksplit(int n, int ncols, int precision);
 cudaError_t launch_sample_tc_packed(const void* A, const void* Rp, int n, int ncols, int precision,
-                                    int trans, int ksplit, double* S, long long lds, int* err, cudaStream_t st);
+                                    int trans, int ksplit, double* S, double* Sc, long long lds, int* err,
+                                    cudaStream_t st);
 // out(:, c) = R rounded to the significand of the mixed format (mode 1: 11
 // bits, TF32; mode 2: 8 bits, BF16)
 cudaError_t launch_round_copy(const double* in, long long ldin, double* out, long long ldout, int n,

@@ -71,8 +71,8 @@ __device__ __forceinline__ double entry_gen(const SrcDev& s, int i, int j) {
 // the coordinates (split to 2^-48 of themselves, subtracted to 2^-46), or r^2 is
 // far from 1 (or not finite).  One entry in 2^15 at max|coordinate| / r = 2.
 // About 105 instructions an entry with the split: 2.8 ps at full issue, and the
-// pack kernel takes 5.8.  n = 12000, 128 columns, BF16 x 3: 6.44 ms with
-// entry_gen, 1.04 ms so.
+// pack kernel, which evaluates one half, took 5.8 an entry of the whole.
+// n = 12000, 128 columns, BF16 x 3: 6.44 ms with entry_gen, 1.04 ms so.
 __device__ __forceinline__ bool laplace_f32(const float4 ah, const float4 al, const float4 bh, const float4 bl,
                                             float* out) {
   float p[3], pe[3];
@@ -133,6 +133,18 @@ __global__ void k_split_points(SrcDev src, float4* out) {
   out[2 * i + 1] = make_float4(l[0], l[1], l[2], 0.f);
 }
 
+// double -> float, round to nearest even, on the integer pipe (the conversion
+// instruction runs at the FP64 pipe's rate); ok is cleared where the value is
+// not a normal float before the rounding
+__device__ __forceinline__ float f32_of(double x, bool& ok) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t ax = hi & 0x7FFFFFFFu;
+  ok = ok && ax - 0x38100000u < 0x0FD00000u;   // 2^-126 .. 2^127: no overflow by the carry
+  const uint32_t t = __funnelshift_l(lo, hi, 3) - 0xC0000000u;
+  const uint32_t up = (lo << 3) + (t & 1u) > 0x80000000u ? 1u : 0u;
+  return __uint_as_float(((t + up) & 0x7FFFFFFFu) | (hi & 0x80000000u));
+}
+
 // The EV entries (row, k .. k + EV - 1) of A - D^(L) (trans: of its transpose)
 // as the chunks of their terms; lo, hi: the row's leaf.
 template <int PREC, bool TRANS>
@@ -165,6 +177,30 @@ __device__ __forceinline__ void entry_chunk(const SrcDev& src, int gr, int k, in
       }
     }
     SP::split(v, chunk);
+    return;
+  }
+  if (src.kind == HSS_SRC_DENSE) {
+    // (a chunk outside of the row's leaf, which is nearly all, without masks)
+    double v[EV];
+    const long long step = TRANS ? 1 : src.ld;
+    const double* p = src.a + (TRANS ? k + gr * src.ld : gr + k * src.ld);
+    if (gr < n && k + EV <= n && (k + EV <= lo || k >= hi)) {
+#pragma unroll
+      for (int x = 0; x < EV; ++x) v[x] = p[x * step];
+    } else {
+#pragma unroll
+      for (int x = 0; x < EV; ++x)
+        v[x] = gr < n && k + x < n && (k + x < lo || k + x >= hi) ? p[x * step] : 0.0;
+    }
+    float f[EV];
+    bool fine = true;
+#pragma unroll
+    for (int x = 0; x < EV; ++x) f[x] = f32_of(v[x], fine);
+    if (!fine) {   // (volatile: not to be computed ahead of the branch)
+#pragma unroll
+      for (int x = 0; x < EV; ++x) asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f[x]) : "d"(v[x]));
+    }
+    SP::split(f, chunk);
     return;
   }
   double v[EV];
@@ -677,6 +713,124 @@ __global__ void __launch_bounds__(256) k_pack_a(SrcDev src, int leaf, int nrb, i
   }
 }
 
+// Packing by 128 x 128 blocks of A, each entry read (or evaluated), masked and
+// rounded to FP32 once and then written to both tiles that hold it: the tile of
+// its row, and the tile of its column, which belongs to the transposed
+// orientation or, for a symmetric source (sym, blocks on and below the
+// diagonal), to the same one.  k_pack_a reads a dense A once per orientation
+// and evaluates every entry of a symmetric source twice.
+// Bound by memory: dense, both orientations, TF32 x 2, n = 8192: 400 us by
+// k_pack_a, 269 us here (0.53 GB read, 1.07 GB written: 5.9 TB/s); the Laplace
+// samples of n = 12000, 128 columns, BF16 x 3: 1.00 to 0.78 ms.
+template <int PREC, int KIND>
+__global__ void __launch_bounds__(256, 3) k_pack_pair(SrcDev src, int leaf, int nb, int nkt, int sym, uint8_t* out) {
+  using SP = Split<PREC>;
+  constexpr int T = SP::T, EV = SP::EV, BK = SP::BK, KC = BK / EV, LD = BM + 4, U = 8;
+  extern __shared__ float blk[];   // column j of the block at j LD: its rows contiguous, as in A
+  __shared__ int ij[2];
+  const int n = src.n, tid = threadIdx.x;
+  if (tid == 0) {
+    const unsigned t = blockIdx.x;
+    int I, J;
+    if (!sym) {   // neighbours in the grid read neighbouring rows of the same columns
+      I = t % nb;
+      J = t / nb;
+    } else {      // column J holds the blocks I = J .. nb - 1
+      const float b = 2.0f * nb + 1.0f;
+      J = (int)((b - sqrtf(fmaxf(b * b - 8.0f * t, 0.0f))) * 0.5f);
+      J = max(0, min(J, nb - 1));
+      auto start = [&](int j) { return (unsigned)j * nb - (unsigned)j * (j - 1u) / 2u; };
+      while (J > 0 && start(J) > t) --J;
+      while (J + 1 < nb && start(J + 1) <= t) ++J;
+      I = J + (int)(t - start(J));
+    }
+    ij[0] = I;
+    ij[1] = J;
+  }
+  __syncthreads();
+  const int I = ij[0], J = ij[1];
+  {
+    const int r = tid % BM, i = I * BM + r, ic = min(i, n - 1);
+    int lo = 0, hi = 0x7fffffff;   // (a row past the end: all of it masked)
+    if (i < n) leaf_range(i, n, leaf, lo, hi);
+    const bool lap = KIND != HSS_SRC_DENSE && src.pts != nullptr;
+    float4 ah = make_float4(0.f, 0.f, 0.f, 0.f), al = ah;
+    if (lap) { ah = src.pts[2 * ic]; al = src.pts[2 * ic + 1]; }
+#pragma unroll 1
+    for (int c = tid / BM; c < BM; c += 2 * U) {
+      float f[U];
+      bool redo = false;
+      if (KIND == HSS_SRC_DENSE) {
+        double v[U];
+#pragma unroll
+        for (int x = 0; x < U; ++x) {
+          const int j = J * BM + c + 2 * x;
+          v[x] = j < n && (j < lo || j >= hi) ? src.a[ic + j * src.ld] : 0.0;
+        }
+        bool fine = true;
+#pragma unroll
+        for (int x = 0; x < U; ++x) f[x] = f32_of(v[x], fine);
+        if (!fine) {   // (volatile: not to be computed ahead of the branch)
+#pragma unroll
+          for (int x = 0; x < U; ++x) asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f[x]) : "d"(v[x]));
+        }
+      } else if (lap) {
+#pragma unroll
+        for (int x = 0; x < U; ++x) {
+          const int j = J * BM + c + 2 * x, jc = min(j, n - 1);
+          const bool in = j < n && (j < lo || j >= hi);
+          float w;
+          const bool ok = laplace_f32(ah, al, src.pts[2 * jc], src.pts[2 * jc + 1], &w);
+          redo |= in && !ok;
+          f[x] = in ? w : 0.f;
+        }
+      } else {
+        redo = true;
+      }
+#pragma unroll
+      for (int x = 0; x < U; ++x) blk[(c + 2 * x) * LD + r] = f[x];
+      if (KIND != HSS_SRC_DENSE && redo) {
+#pragma unroll 1
+        for (int x = 0; x < U; ++x) {
+          const int j = J * BM + c + 2 * x;
+          blk[(c + 2 * x) * LD + r] = j < n && (j < lo || j >= hi) ? to_f32(entry_gen(src, ic, j)) : 0.f;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  constexpr int NT = BM / BK;   // k-tiles of a block
+  for (int u = tid; u < NT * BM * KC; u += 256) {   // rows of the block as tile rows
+    const int r = u % BM, c = (u / BM) % KC, t = u / (BM * KC), kt = J * NT + t;
+    if (kt >= nkt) break;
+    float f[EV];
+#pragma unroll
+    for (int x = 0; x < EV; ++x) f[x] = blk[(t * BK + c * EV + x) * LD + r];
+    uint4 chunk[T];
+    SP::split(f, chunk);
+    uint8_t* dst = out + ((size_t)I * nkt + kt) * (T * TILE_A_BYTES) + (r / 8) * 1024 + c * 128 + (r % 8) * 16;
+#pragma unroll
+    for (int p = 0; p < T; ++p) *(uint4*)(dst + p * TILE_A_BYTES) = chunk[p];
+  }
+  if (sym && I == J) return;
+  const size_t o1 = sym ? 0 : (size_t)nb * nkt;
+  for (int u = tid; u < NT * BM * KC; u += 256) {   // columns of the block as tile rows
+    const int r = (u / (8 * KC)) % (BM / 8) * 8 + u % 8, c = (u / 8) % KC, t = u / (BM * KC), kt = I * NT + t;
+    if (kt >= nkt) break;
+    float f[EV];
+#pragma unroll
+    for (int x = 0; x < EV; x += 4) {
+      const float4 d = *(const float4*)(blk + r * LD + t * BK + c * EV + x);
+      f[x] = d.x; f[x + 1] = d.y; f[x + 2] = d.z; f[x + 3] = d.w;
+    }
+    uint4 chunk[T];
+    SP::split(f, chunk);
+    uint8_t* dst = out + (o1 + (size_t)J * nkt + kt) * (T * TILE_A_BYTES) + (r / 8) * 1024 + c * 128 + (r % 8) * 16;
+#pragma unroll
+    for (int p = 0; p < T; ++p) *(uint4*)(dst + p * TILE_A_BYTES) = chunk[p];
+  }
+}
+
 template <int PREC>
 __global__ void __launch_bounds__(256) k_pack_r(const double* R, long long ldr, int n, int ncols, int N,
                                                 int nkt, int swap, uint8_t* out) {
@@ -703,6 +857,7 @@ struct TcPackedArgs {
   const uint8_t* Rp;
   int n, nrb, nkt, N, ncols, tmem_cols, ksplit, trans, drain;
   double* S;
+  double* Sc;         // the transposed orientation (trans = 0), or NULL: only S
   long long lds;
   int atomic;
   int* err;
@@ -730,7 +885,9 @@ __global__ void __maxnreg__(96) k_sample_tc_packed(TcPackedArgs a) {
   // column tiles vary fastest across the grid: the CTAs that stream one
   // row block of A for different column tiles run together and share it
   // through L2, so A crosses HBM once per pass
-  const int rb = blockIdx.y, ct = blockIdx.x;
+  // (both orientations, where both are wanted, in one launch: one last wave
+  // instead of two)
+  const int side = blockIdx.y >= (unsigned)a.nrb ? 1 : 0, rb = blockIdx.y - side * a.nrb, ct = blockIdx.x;
   const int kt0 = (int)((long long)a.nkt * blockIdx.z / a.ksplit);
   const int kt1 = (int)((long long)a.nkt * (blockIdx.z + 1) / a.ksplit);
   const int nk = kt1 - kt0, DR = a.drain;
@@ -751,7 +908,7 @@ __global__ void __maxnreg__(96) k_sample_tc_packed(TcPackedArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint8_t* gA = a.A + ((size_t)(a.trans * a.nrb + rb) * a.nkt + kt0) * (T * TILE_A_BYTES);
+  const uint8_t* gA = a.A + ((size_t)((a.trans + side) * a.nrb + rb) * a.nkt + kt0) * (T * TILE_A_BYTES);
   const uint8_t* gB = a.Rp + ((size_t)ct * a.nkt + kt0) * tileB;
   if (warp == 0) {
     if (lane == 0) {
@@ -801,7 +958,7 @@ __global__ void __maxnreg__(96) k_sample_tc_packed(TcPackedArgs a) {
       if (lane == 0) mbar_arrive(&tempty[b]);
     }
     if (ok && nk > 0)
-      store_row<NH>(a.S, a.lds, a.n, a.ncols, rb * BM + 32 * q + lane, ct * N + h * NH, a.atomic, s, e);
+      store_row<NH>(side ? a.Sc : a.S, a.lds, a.n, a.ncols, rb * BM + 32 * q + lane, ct * N + h * NH, a.atomic, s, e);
   }
   tc_fence_before();
   __syncthreads();
@@ -827,7 +984,7 @@ template <int PREC>
 cudaError_t launch_packed_t(const TcPackedArgs& a, int gx, int gy, cudaStream_t st) {
   constexpr int T = Split<PREC>::T, NS = packed_stages<PREC>();
   const size_t sm = (size_t)NS * (T * TILE_A_BYTES + (size_t)a.N * 128) + 8 * (2 * NS + 4) + 16 + 1024;
-  dim3 grid(gy, gx, a.ksplit);   // x: column tiles, y: row blocks
+  dim3 grid(gy, gx, a.ksplit);   // x: column tiles, y: row blocks (of both orientations)
 #define HSS_LAUNCH_PK(NHV)                                                                          \
   do {                                                                                              \
     cudaError_t e = cudaFuncSetAttribute(k_sample_tc_packed<PREC, NHV>,                             \
@@ -920,6 +1077,22 @@ cudaError_t launch_pack_a(const SrcDev& src, int leaf, int precision, int orient
   const int nrb = (n + BM - 1) / BM, nkt = (n + bk - 1) / bk;
   const long long tiles = (long long)orients * nrb * nkt;
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  // by blocks where a block serves two tiles; a dense A wanted in one
+  // orientation is read once either way (and may be symmetric only in name)
+  const bool dense = src.kind == HSS_SRC_DENSE, sym = src.kind == HSS_SRC_GAUSS || src.kind == HSS_SRC_LAPLACE;
+  if ((dense && orients == 2) || (sym && orients == 1)) {
+    auto run = [&](auto* kernel) -> cudaError_t {
+      const int sm = BM * (BM + 4) * (int)sizeof(float);
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+      if (e != cudaSuccess) return e;
+      const long long grid = dense ? (long long)nrb * nrb : (long long)nrb * (nrb + 1) / 2;
+      kernel<<<(unsigned)grid, 256, sm, st>>>(src, leaf, nrb, nkt, dense ? 0 : 1, (uint8_t*)out);
+      return cudaGetLastError();
+    };
+    if (precision == HSS_PREC_TF32X2)
+      return dense ? run(k_pack_pair<HSS_PREC_TF32X2, HSS_SRC_DENSE>) : run(k_pack_pair<HSS_PREC_TF32X2, HSS_SRC_LAPLACE>);
+    return dense ? run(k_pack_pair<HSS_PREC_BF16X3, HSS_SRC_DENSE>) : run(k_pack_pair<HSS_PREC_BF16X3, HSS_SRC_LAPLACE>);
+  }
   if (precision == HSS_PREC_TF32X2)
     k_pack_a<HSS_PREC_TF32X2><<<(unsigned)tiles, 256, 0, st>>>(src, leaf, nrb, nkt, (uint8_t*)out);
   else
@@ -952,7 +1125,8 @@ int sample_tc_ksplit(int n, int ncols, int precision) {
 }
 
 cudaError_t launch_sample_tc_packed(const void* A, const void* Rp, int n, int ncols, int precision,
-                                    int trans, int ksplit, double* S, long long lds, int* err, cudaStream_t st) {
+                                    int trans, int ksplit, double* S, double* Sc, long long lds, int* err,
+                                    cudaStream_t st) {
   if (n <= 0 || ncols <= 0) return cudaSuccess;
   TcPackedArgs a;
   a.A = (const uint8_t*)A;
@@ -967,12 +1141,13 @@ cudaError_t launch_sample_tc_packed(const void* A, const void* Rp, int n, int nc
   a.trans = trans;
   a.drain = DRAIN_PACKED;
   a.S = S;
+  a.Sc = Sc;
   a.lds = lds;
   a.atomic = a.ksplit > 1 ? 1 : 0;
   a.err = err;
-  const int gy = (ncols + a.N - 1) / a.N;
-  if (precision == HSS_PREC_TF32X2) return launch_packed_t<HSS_PREC_TF32X2>(a, a.nrb, gy, st);
-  if (precision == HSS_PREC_BF16X3) return launch_packed_t<HSS_PREC_BF16X3>(a, a.nrb, gy, st);
+  const int gy = (ncols + a.N - 1) / a.N, gx = (Sc ? 2 : 1) * a.nrb;
+  if (precision == HSS_PREC_TF32X2) return launch_packed_t<HSS_PREC_TF32X2>(a, gx, gy, st);
+  if (precision == HSS_PREC_BF16X3) return launch_packed_t<HSS_PREC_BF16X3>(a, gx, gy, st);
   return cudaErrorInvalidValue;
 }
 
