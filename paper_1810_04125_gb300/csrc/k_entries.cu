@@ -64,7 +64,14 @@ __device__ __forceinline__ double warp_sum8(double* a, int lane) {
   return s;
 }
 
-constexpr int EW = 4;   // warps of a path CTA
+// Warps of a path CTA by the largest rank.  Walking a path is a chain of small
+// products; with ranks of 100 and more four warps take several rounds of loads
+// per block, and sixteen hide more of them (ranks to 200, Laplace n = 3000: one
+// entry 448 us with 4 warps, 395 with 8, 219 with 16; 400 x 300 entries 854,
+// 874, 731); with small ranks twelve of the sixteen only wait (Toeplitz n = 8192:
+// 400 x 300 entries 104 us with 4 warps, 135 with 16).
+inline int path_warps(int kcap) { return kcap >= 96 ? 16 : 4; }
+constexpr int EW_MAX = 16;
 
 // Row (CTAs below nr) or column vectors of the nested basis along the path of
 // an index to the root.  A row stores W(level(a)) = u_a(i) B_ab for every
@@ -74,7 +81,7 @@ constexpr int EW = 4;   // warps of a path CTA
 // sums run along the blocks' contiguous direction: u B with eight columns of B
 // per warp and lanes along u, u U_p with a lane per column.  Rows and columns
 // go in one launch.
-__global__ void __launch_bounds__(32 * EW) k_entry_paths(const EntryNode* __restrict__ nodes,
+__global__ void __launch_bounds__(32 * EW_MAX) k_entry_paths(const EntryNode* __restrict__ nodes,
                                                          const int* __restrict__ leaf_of, int n,
                                                          const int* __restrict__ I, int nr, const int* __restrict__ J,
                                                          double* __restrict__ Wrow, double* __restrict__ Vcol, int kcap,
@@ -83,7 +90,7 @@ __global__ void __launch_bounds__(32 * EW) k_entry_paths(const EntryNode* __rest
   double* u = sm;
   double* u2 = sm + kcap;
   int* sp = (int*)(sm + 2 * kcap);
-  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, EW = blockDim.x / 32;
   const int side = (int)blockIdx.x >= nr, r = side ? blockIdx.x - nr : blockIdx.x;
   const int i = side ? J[r] : I[r];
   if (i < 0 || i >= n) {   // reported; the pair kernel skips the entry
@@ -258,7 +265,7 @@ cudaError_t launch_entry_paths(const EntryNode* nodes, const int* leaf_of, int n
   const size_t sm = (sizeof(double) * 2 + sizeof(int)) * (size_t)kcap;
   cudaError_t e = cudaFuncSetAttribute(k_entry_paths, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_entry_paths<<<nr + nc, 32 * EW, sm, st>>>(nodes, leaf_of, n, I, nr, J, Wrow, Vcol, kcap, lp1, err);
+  k_entry_paths<<<nr + nc, 32 * path_warps(kcap), sm, st>>>(nodes, leaf_of, n, I, nr, J, Wrow, Vcol, kcap, lp1, err);
   return cudaGetLastError();
 }
 
