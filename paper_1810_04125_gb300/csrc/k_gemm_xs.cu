@@ -53,6 +53,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "tc_common.cuh"
@@ -499,11 +500,12 @@ __device__ __forceinline__ double fixed_value(long long hi, long long lo, int e2
 // The tile's results (column-padded, in shared memory) to C: lanes along the
 // contiguous direction.
 constexpr int XLD = XS_TN + 1;
+template <int NR = XS_TM>
 __device__ __forceinline__ void store_tile(const GemmJob& jb, const double* sm, int i0, int j0, int t) {
   const bool row_major = jb.c_cs == 1;
   const double beta = jb.beta, gamma = jb.gamma;
-  for (int q = t; q < XS_TM * XS_TN; q += XW * 32) {
-    const int il = row_major ? q / XS_TN : q % XS_TM, jl = row_major ? q % XS_TN : q / XS_TM;
+  for (int q = t; q < NR * XS_TN; q += XW * 32) {
+    const int il = row_major ? q / XS_TN : q % NR, jl = row_major ? q % XS_TN : q / NR;
     const int i = i0 + il, jj = j0 + jl;
     if (i >= jb.M || jj >= jb.N) continue;
     double v = sm[il * XLD + jl];
@@ -521,20 +523,24 @@ __device__ __forceinline__ void store_tile(const GemmJob& jb, const double* sm, 
   }
 }
 
-// The tile by FP64 FMAs (operands the digits cannot hold): 512 threads, 4 x 4
-// outputs each, K staged 16 at a time.  Leaves alpha * sum in sm.
-__device__ void fp64_tile(const GemmJob& jb, double* sm, double* stage, int i0, int j0, int t) {
-  double (*As)[XS_TM + 2] = (double (*)[XS_TM + 2])stage;
-  double (*Bs)[XS_TN + 2] = (double (*)[XS_TN + 2])(stage + 16 * (XS_TM + 2));
-  const int tx = t % 16, ty = t / 16;
-  double acc[4][4];
+// NR rows of the tile by FP64 FMAs (operands the digits cannot hold): 512
+// threads, RX x CY outputs each, K staged 16 at a time, every output one chain
+// over K whatever NR.
+template <int RX, int CY>
+__device__ void fp64_rows(const GemmJob& jb, double* sm, int i0, int j0, int t) {
+  constexpr int TX = XS_TN / CY, NR = XW * 32 / TX * RX;
+  double* stage = sm + XS_TM * XLD;
+  double (*As)[NR + 2] = (double (*)[NR + 2])stage;
+  double (*Bs)[XS_TN + 2] = (double (*)[XS_TN + 2])(stage + 16 * (NR + 2));
+  const int tx = t % TX, ty = t / TX;
+  double acc[RX][CY];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < RX; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+    for (int b = 0; b < CY; ++b) acc[a][b] = 0.0;
   for (int l0 = 0; l0 < jb.K; l0 += 16) {
-    for (int q = t; q < 16 * XS_TM; q += XW * 32) {
-      const int il = q % XS_TM, kk = q / XS_TM, i = i0 + il, l = l0 + kk;
+    for (int q = t; q < 16 * NR; q += XW * 32) {
+      const int il = q % NR, kk = q / NR, i = i0 + il, l = l0 + kk;
       As[kk][il] = (i < jb.M && l < jb.K) ? op_row(jb.A, i)[(long long)l * jb.A.cs] : 0.0;
     }
     for (int q = t; q < 16 * XS_TN; q += XW * 32) {
@@ -544,25 +550,45 @@ __device__ void fp64_tile(const GemmJob& jb, double* sm, double* stage, int i0, 
     bar_drain();
 #pragma unroll 4
     for (int kk = 0; kk < 16; ++kk) {
-      double a[4], b[4];
+      double a[RX], b[CY];
 #pragma unroll
-      for (int x = 0; x < 4; ++x) { a[x] = As[kk][ty * 4 + x]; b[x] = Bs[kk][tx * 4 + x]; }
+      for (int x = 0; x < RX; ++x) a[x] = As[kk][ty * RX + x];
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < CY; ++x) b[x] = Bs[kk][tx * CY + x];
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] = __fma_rn(a[x], b[y], acc[x][y]);
+      for (int x = 0; x < RX; ++x)
+#pragma unroll
+        for (int y = 0; y < CY; ++y) acc[x][y] = __fma_rn(a[x], b[y], acc[x][y]);
     }
     bar_drain();
   }
 #pragma unroll
-  for (int x = 0; x < 4; ++x)
+  for (int x = 0; x < RX; ++x)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) sm[(ty * 4 + x) * XLD + tx * 4 + y] = jb.alpha * acc[x][y];
+    for (int y = 0; y < CY; ++y) sm[(ty * RX + x) * XLD + tx * CY + y] = jb.alpha * acc[x][y];
   bar_drain();
+  store_tile<NR>(jb, sm, i0, j0, t);
+}
+
+// Such a tile is shared by its CTAs by rows: those of its K segments, and
+// helpers (CTAs past the last unit, which leave at once when the digits hold
+// the tile).  One CTA takes 2.15 us per unit of K for the tile, and a level of
+// a deep tree has a dozen to fifty tiles: the projections of the Incrementing
+// strategy on the surface kernel (n = 4001), where the elements of one
+// column spread over more than 2^10, took 300 to 1500 us a product on 12 to 48
+// CTAs: 21.1 ms of 77 in all, 6.6 with the rows shared.
+__device__ void fp64_share(const GemmJob& jb, double* sm, int i0, int j0, int part, int parts, int t) {
+  const int ns = parts >= 8 ? 8 : (parts >= 4 ? 4 : (parts >= 2 ? 2 : 1));
+  const int r0 = i0 + part * (XS_TM / ns);
+  if (part >= ns || r0 >= jb.M) return;
+  if (ns == 8) fp64_rows<1, 2>(jb, sm, r0, j0, t);
+  else if (ns == 4) fp64_rows<1, 4>(jb, sm, r0, j0, t);
+  else if (ns == 2) fp64_rows<2, 4>(jb, sm, r0, j0, t);
+  else fp64_rows<4, 4>(jb, sm, r0, j0, t);
 }
 
 __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const int* __restrict__ prefix, int njobs,
-                                          int* flag, int* err) {
+                                          int nunits, int* flag, int* err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ GemmJob sj;
   __shared__ int s_bad, s_last;
@@ -572,7 +598,9 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
   uint64_t* tempty = tfull + XMW;
   uint32_t* tmem_slot = (uint32_t*)(tempty + XMW);
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-  const int ji = find_job(prefix, njobs, blockIdx.x);
+  // CTAs past the units are helpers of unit blockIdx.x % nunits
+  const int share = blockIdx.x / nunits, shares = gridDim.x / nunits, unit = blockIdx.x % nunits;
+  const int ji = find_job(prefix, njobs, unit);
   if (tid == 0) {
     sj = jobs[ji];
     s_bad = 0;
@@ -581,7 +609,7 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const int u = blockIdx.x - prefix[ji], nseg = sj.nseg;
+  const int u = unit - prefix[ji], nseg = sj.nseg;
   const int ntn = (sj.N + XS_TN - 1) / XS_TN;
   const int t = u / nseg, seg = u % nseg;   // column tiles fastest: the tiles of one row block share A through L2
   const int ti = t / ntn, tj = t % ntn, i0 = ti * XS_TM, j0 = tj * XS_TN;
@@ -600,13 +628,12 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
   if (s_bad) {
     if (flag) {
       if (tid == 0) atomicOr(flag, 1);
-    } else if (seg == 0 && warp > XMW) {
-      const int t512 = tid - (1 + XMW) * 32;
-      fp64_tile(sj, tile_sm, tile_sm + XS_TM * XLD, i0, j0, t512);
-      store_tile(sj, tile_sm, i0, j0, t512);
+    } else if (warp > XMW) {
+      fp64_share(sj, tile_sm, i0, j0, seg + nseg * share, nseg * shares, tid - (1 + XMW) * 32);
     }
     return;
   }
+  if (share > 0) return;
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(512u)
@@ -739,7 +766,9 @@ cudaError_t launch_xs_mm(const GemmJob* jobs_dev, const int* prefix_dev, int njo
   const size_t sm = (size_t)XNS * XSTAGE + 8 * (2 * XNS + 2 * XMW) + 16;
   cudaError_t e = cudaFuncSetAttribute(k_xs_mm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_xs_mm<<<nunits, XTHREADS, sm, st>>>(jobs_dev, prefix_dev, njobs, flag, err);
+  // helpers where the units leave SMs idle (with a flag the caller falls back)
+  const int shares = flag || nunits > 304 ? 1 : std::min(8, 608 / nunits);
+  k_xs_mm<<<nunits * shares, XTHREADS, sm, st>>>(jobs_dev, prefix_dev, njobs, nunits, flag, err);
   return cudaGetLastError();
 }
 

@@ -129,3 +129,23 @@ def test_product_columns(torch, nrhs, transpose):
             assert np.array_equal(np.isfinite(a), np.isfinite(b)) and not np.isfinite(a).all()
         else:   # both within a few hundred roundings of terms bounded by |H||x|
             assert np.abs(a - b).max() <= 1e-13 * np.abs(src.to_dense()).sum(axis=1).max() * np.abs(X[:, j]).max()
+
+
+# columns that the digits cannot hold, with the rows of a tile shared by 8, 4, 2
+# and 1 CTAs (as the columns make more tiles): against the same product by tasks,
+# both sums of the same terms in FP64
+@pytest.mark.parametrize("nrhs", [256, 640, 1300, 2600])
+def test_shared_rows(torch, nrhs):
+    from paper_1810_04125_gb300 import hss
+    import gpu_util as gu
+    n = 800
+    src = w.dense_source(np.random.default_rng(1).standard_normal((n, n)))
+    H = hss.hss_compress(gu.device_source(src), hss.make_opts(100, 1e-12, 1e-13, 64, 64, n, hss.HSS_DOUBLING))
+    rng = np.random.default_rng(5)
+    X = gu.col_major(rng.standard_normal((n, nrhs)) * 10.0 ** -rng.uniform(0, 12, (n, 1)))
+    Y, Z = (torch.empty((nrhs, n), dtype=torch.float64, device=gu.dev()).t() for _ in range(2))
+    hss.hss_matvec(H, X, Y)
+    for j in range(0, nrhs, 4):
+        hss.hss_matvec(H, X[:, j:j + 4], Z[:, j:j + 4])
+    bound = 1e-13 * np.abs(src.to_dense()).sum(axis=1).max() * np.abs(X.cpu().numpy()).max(axis=0)
+    assert np.all(np.abs((Y - Z).cpu().numpy()) <= bound)
