@@ -181,8 +181,17 @@ __global__ void __launch_bounds__(NT) k_inc_qr(const IncJob* __restrict__ jobs) 
 //    reflector): one reduction of [V^T V, V^T E] per block (its P partials
 //    added by slices over the group, then read back by all), E <- E -
 //    V (T (V^T E)).
-// The P partial sums of a value are added in rank order, so all CTAs hold
+// The P partial sums of a value are added in a fixed order, so all CTAs hold
 // identical scalars.  Same tests, same outputs as k_inc_qr.
+//
+// A column is a chain: dots, barrier, sums of the partials, square root and
+// divisions, update.  The FP64 instructions on it (64 clocks of a scheduler's
+// pipe each) are kept few: eight dots of a warp are summed over its lanes
+// together, the partials of a value by four lanes, the two divisions in two
+// warps, and c(j) is read from the CTA that owns it.  The blocks of 64 columns
+// of the surface kernel n = 4001 (groups of 32 CTAs): 640 to 520 us a launch,
+// 19.6 to 15.1 ms a compression.  Groups of at least 16 or 32 rows per CTA
+// instead of 8 took 15.3 and 17.2 ms.
 constexpr int GR_BUDGET = 6144;   // doubles of V (and of E) per CTA: rows x b
 constexpr int GR_BMAX = 1024;     // widest block of the group form (tau table)
 constexpr int QB = 16;            // reflectors per block of the Q formation
@@ -249,6 +258,25 @@ __device__ double bsum(double v, double* sh) {
   double t = 0.0;
   for (int w = 0; w < NW; ++w) t += sh[w];
   return t;
+}
+
+// Eight sums over a warp: lane l's a[x] are its parts of sum x, the return value
+// is sum l / 4.  9 additions (each occupies the scheduler's FP64 pipe for 64
+// clocks) where eight butterflies take 40.
+__device__ __forceinline__ double warp_sum8(double* a, int lane) {
+#pragma unroll
+  for (int h = 4; h >= 1; h /= 2) {
+    const bool up = (lane & (4 * h)) != 0;
+#pragma unroll
+    for (int x = 0; x < h; ++x) {
+      const double keep = up ? a[x + h] : a[x], give = up ? a[x] : a[x + h];
+      a[x] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+    }
+  }
+  double s = a[0];
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  return s;
 }
 
 // reflectors per block of the Q formation for a block of beff columns
@@ -341,36 +369,60 @@ __global__ void __launch_bounds__(NT, 2) k_inc_group(const IncJob* __restrict__ 
     const int nc = b - j;
     const bool ownj = j >= r0 && j < r0 + nr;
     double* out = slot(parity, rank);
-    for (int c = warp; c < nc; c += NW) {   // a warp per column
+    {   // a warp per eight columns, their sums over the lanes at once
       const double* xc = V + (size_t)j * RB;
-      const double* cc = V + (size_t)(j + c) * RB;
-      double w = 0.0;
-      for (int i = lane; i < nr; i += 32)
-        if (r0 + i >= j) w = __fma_rn(xc[i], cc[i], w);
-      w = warp_sum(w);
-      if (lane == 0) {
-        __stcg(out + c, w);
-        __stcg(out + nc + c, ownj ? cc[j - r0] : 0.0);
+      const int i0 = max(0, j - r0);
+      for (int c0 = 8 * warp; c0 < nc; c0 += 8 * NW) {
+        const double* cc = V + (size_t)(j + c0) * RB;
+        double a[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) a[x] = 0.0;
+        for (int i = i0 + lane; i < nr; i += 32) {
+          const double xi = xc[i];
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+            if (c0 + x < nc) a[x] = __fma_rn(xi, cc[i + (size_t)x * RB], a[x]);
+        }
+        const double w = warp_sum8(a, lane);
+        if ((lane & 3) == 0 && c0 + lane / 4 < nc) __stcg(out + c0 + lane / 4, w);
       }
+      if (ownj)
+        for (int c = tid; c < nc; c += NT) __stcg(out + nc + c, V[(j - r0) + (size_t)(j + c) * RB]);
     }
     if (!gbar(jb.bar, P, epoch, err, &s_ok, jb.wait_ns)) return;
-    for (int t = tid; t < 2 * nc; t += NT) {   // the P partials of a value, in rank order
-      const double w = sum_partials(slot(parity, 0) + t, S1, P);
-      if (t < nc) dd[t] = w;
-      else gg[t - nc] = w;
+    // the P partials of a value by four lanes (one lane's chain of 32 additions
+    // took 2000 clocks); c(j) from the CTA that owns row j
+    for (int t0 = 0; t0 < nc; t0 += NT / 4) {
+      const int t = t0 + tid / 4;
+      double w = 0.0;
+      if (t < nc) {
+        const double* base = slot(parity, 0) + t;
+        for (int q = tid & 3; q < P; q += 32) {
+          double v[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) v[u] = q + 4 * u < P ? __ldcg(base + (size_t)(q + 4 * u) * S1) : 0.0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (q + 4 * u < P) w += v[u];
+        }
+      }
+      w += __shfl_xor_sync(0xffffffffu, w, 2);
+      w += __shfl_xor_sync(0xffffffffu, w, 1);
+      if (t < nc && (tid & 3) == 0) dd[t] = w;
     }
+    for (int t = tid; t < nc; t += NT) gg[t] = __ldcg(slot(parity, j / RB) + nc + t);
     parity ^= 1;
     __syncthreads();
-    if (tid == 0) {
+    if (tid == 0 || tid == 32) {   // (two warps: the divisions run side by side)
       const double alpha = sqrt(dd[0]), x0 = gg[0];
-      double beta = 0.0, tau = 0.0, scal = 0.0;
-      if (alpha != 0.0) {
-        beta = x0 >= 0.0 ? -alpha : alpha;
-        tau = (beta - x0) / beta;
-        scal = 1.0 / (x0 - beta);
+      const double beta = x0 >= 0.0 ? -alpha : alpha;
+      if (tid == 32) {
+        s_sc[3] = alpha != 0.0 ? 1.0 / (x0 - beta) : 0.0;
+      } else {
+        const double tau = alpha != 0.0 ? (beta - x0) / beta : 0.0;
+        s_sc[0] = alpha; s_sc[1] = alpha != 0.0 ? beta : 0.0; s_sc[2] = tau;
+        s_taus[j] = tau;
       }
-      s_sc[0] = alpha; s_sc[1] = beta; s_sc[2] = tau; s_sc[3] = scal;
-      s_taus[j] = tau;
     }
     __syncthreads();
     const double alpha = s_sc[0], beta = s_sc[1], tau = s_sc[2], scal = s_sc[3];
