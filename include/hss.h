@@ -382,9 +382,11 @@ hss_status hss_load(const char* path, hss_matrix* out);
  * of a call (packed operands, job lists, temporaries) come stream-ordered
  * from a memory pool of the library's own per context, which keeps freed
  * memory reserved, at most the largest set of work buffers one call held at
- * once (the device's default pool is not touched).
+ * once (the device's default pool is not touched).  Up to sixteen pinned
+ * read-back buffers of 64 KB stay for later calls too.
  * This call returns the chunks cached for the current device with cudaFree
- * and, after waiting for the device, trims that pool to nothing. */
+ * and the pinned buffers of its context and, after waiting for the device,
+ * trims that pool to nothing. */
 hss_status hss_release_cached(void);
 const char* hss_status_str(hss_status s);
 const char* hss_last_error(void);
