@@ -458,11 +458,40 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0u;
 }
 
+// TF32 x 2 with 128 columns: the columns of R are the rows of the product (the
+// MMA's first operand) and the matrix tile its columns, eight of the leading
+// terms and the eight of the second terms of a row group in turn, so that one
+// MMA of 128 x 256 x 8 does what two of 128 x 128 x 8 did (an MMA is issued in
+// about 110 clocks whatever its width; n = 131072, 256 columns: 26.8 to 22.4 ms,
+// 0.84 of the measured tensor rate).  Cores of even number lie in one half of
+// the buffer, the terms of each side by side, those of odd number in the other:
+// a group to the next is SBO = one core matrix, a chunk to the one before LBO =
+// half the buffer.
+template <int PREC, int NH>
+constexpr bool toep_swap() { return PREC == HSS_PREC_TF32X2 && NH == 32; }
+constexpr uint32_t TP_HALF = TILE_A_BYTES;
+
+// drain_chain for that product: lane = sample column, NH rows of the matrix
+__device__ __forceinline__ void drain_swapped(uint32_t tmem, int b, int q, int h, float* s, float* e) {
+  const uint32_t at = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(256 * b + 64 * h);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float x[16];
+    tmem_ld16_nw(at + 16 * c, x);
+    tmem_wait_ld();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) ff_add(s[8 * c + i], e[8 * c + i], x[i]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) e[8 * c + i] = __fadd_rn(e[8 * c + i], x[8 + i]);
+  }
+}
+
 template <int PREC, int NH, int TRANS>
 __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
   using SP = Split<PREC>;
   constexpr int T = SP::T, EV = SP::EV, BK = SP::BK, KC = BK / EV, RS = 8 / EV;
   constexpr int DR = drain_gen(PREC);
+  constexpr bool SWAP = toep_swap<PREC, NH>();
   constexpr uint32_t abuf = T * TILE_A_BYTES;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int n = a.src.n, N = a.N;
@@ -525,12 +554,27 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
       const int b = cd & 1;
       if (!mbar_wait_warp(&tfull[b], (uint32_t)(cd >> 1) & 1u, a.err, 6)) { ok = false; break; }
       tc_fence_after();
-      drain_chain<NH>(tmem, N, b, q, h, s, e);
+      if constexpr (SWAP) drain_swapped(tmem, b, q, h, s, e);
+      else drain_chain<NH>(tmem, N, b, q, h, s, e);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[b]);
     }
-    if (ok) store_row<NH>(a.S, a.lds, n, a.ncols, row0 + 32 * q + lane, col0 + h * NH, a.atomic, s, e);
+    if constexpr (SWAP) {
+      const int col = col0 + 32 * q + lane;
+#pragma unroll
+      for (int j = 0; j < NH; ++j) {
+        const int row = row0 + h * NH + j;
+        if (ok && col < a.ncols && row < n) {
+          const double v = f2d_exact(s[j]) + f2d_exact(e[j]);
+          double* out = a.S + (long long)row * a.lds + col;
+          if (a.atomic) atomicAdd(out, v);
+          else *out = v;
+        }
+      }
+    } else if (ok) {
+      store_row<NH>(a.S, a.lds, n, a.ncols, row0 + 32 * q + lane, col0 + h * NH, a.atomic, s, e);
+    }
   } else if (warp >= GEN_WARPS + 2) {
     // ------------------------------------------------------------ strips of A
     const int tl = tid - (GEN_WARPS + 2) * 32;
@@ -577,7 +621,11 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
           uint4 ch[T];
           chunk_of(TRANS ? -d : d, TRANS ? 1 : -1, ch, [](int) { return true; });
 #pragma unroll
-          for (int t = 0; t < T; ++t) *(uint4*)(dst + t * TILE_A_BYTES + (uint32_t)u * 16u) = ch[t];
+          for (int t = 0; t < T; ++t) {
+            const uint32_t off = SWAP ? (uint32_t)(m & 1) * TP_HALF + (uint32_t)((m & ~1) + t) * 128u + (uint32_t)rho * 16u
+                                      : t * TILE_A_BYTES + (uint32_t)u * 16u;
+            *(uint4*)(dst + off) = ch[t];
+          }
         }
       } else {
         const int k0 = kt * BK;
@@ -589,9 +637,11 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
             const int gk = k0 + c * EV + x;
             return gr < n && gk < n && (gk < lo || gk >= hi);
           });
-          const uint32_t off = (uint32_t)(r / 8) * 1024u + (uint32_t)(c ^ 1) * 128u + (uint32_t)(r % 8) * 16u;
+          // (swapped: the groups of a chunk together, 4 KB a chunk)
+          const uint32_t off = SWAP ? (uint32_t)(c ^ 1) * 4096u + (uint32_t)(r / 8) * 256u + (uint32_t)(r % 8) * 16u
+                                    : (uint32_t)(r / 8) * 1024u + (uint32_t)(c ^ 1) * 128u + (uint32_t)(r % 8) * 16u;
 #pragma unroll
-          for (int t = 0; t < T; ++t) *(uint4*)(dst + t * TILE_A_BYTES + off) = ch[t];
+          for (int t = 0; t < T; ++t) *(uint4*)(dst + (SWAP ? t * 128u : t * TILE_A_BYTES) + off) = ch[t];
         }
       }
       fence_async_smem();
@@ -619,7 +669,7 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
     }
   } else {
     // --------------------------------------------------------- MMA issuer
-    const uint32_t id = idesc(SP::FMT, (uint32_t)N);
+    const uint32_t id = idesc(SP::FMT, SWAP ? 256u : (uint32_t)N);
     const bool one = elect_one();
     bool ok = true, masked = false;
     int st = 0, it = 0;
@@ -637,18 +687,28 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
         tc_fence_after();
         if (one) {
           const uint64_t bd = sdesc(smem_u32(sB + st * tileB), 128u, 1024u);
-          // chunk 2 ks + 1 of the tile's first row group, then LBO on to 2 ks
-          const uint64_t ad = masked ? sdesc(sa, 128u, 1024u)
-                                     : sdesc(sa + 128u * (uint32_t)(KC - 2 + KC * (len - 1 - j)), 128u, RS * 128u);
-          const uint32_t hi = tmem + (uint32_t)((2 * b) * N), lo = hi + (uint32_t)N;
+          if constexpr (SWAP) {
+            const uint64_t ad = masked ? sdesc(sa, 4096u, 128u)
+                                       : sdesc(sa + 128u * (uint32_t)(KC - 2 + KC * (len - 1 - j)), TP_HALF, 128u);
 #pragma unroll
-          for (int ks = 0; ks < BK / SP::KSTEP; ++ks) {
-            const uint64_t ak = masked ? ad + (uint64_t)(ks * 16) : ad - (uint64_t)(ks * 16);   // 256 bytes
-            const uint64_t bk = bd + (uint64_t)(ks * 16);
-            mma<PREC>(hi, ak, bk, id, (first && ks == 0) ? 0u : 1u);
+            for (int ks = 0; ks < BK / SP::KSTEP; ++ks)
+              mma<PREC>(tmem + (uint32_t)(256 * b), bd + (uint64_t)(ks * 16),
+                        masked ? ad + (uint64_t)(ks * 512) : ad - (uint64_t)(ks * 16), id,
+                        (first && ks == 0) ? 0u : 1u);
+          } else {
+            // chunk 2 ks + 1 of the tile's first row group, then LBO on to 2 ks
+            const uint64_t ad = masked ? sdesc(sa, 128u, 1024u)
+                                       : sdesc(sa + 128u * (uint32_t)(KC - 2 + KC * (len - 1 - j)), 128u, RS * 128u);
+            const uint32_t hi = tmem + (uint32_t)((2 * b) * N), lo = hi + (uint32_t)N;
 #pragma unroll
-            for (int t = 1; t < T; ++t)
-              mma<PREC>(lo, ak + (uint64_t)((t * TILE_A_BYTES) >> 4), bk, id, (first && ks == 0 && t == 1) ? 0u : 1u);
+            for (int ks = 0; ks < BK / SP::KSTEP; ++ks) {
+              const uint64_t ak = masked ? ad + (uint64_t)(ks * 16) : ad - (uint64_t)(ks * 16);   // 256 bytes
+              const uint64_t bk = bd + (uint64_t)(ks * 16);
+              mma<PREC>(hi, ak, bk, id, (first && ks == 0) ? 0u : 1u);
+#pragma unroll
+              for (int t = 1; t < T; ++t)
+                mma<PREC>(lo, ak + (uint64_t)((t * TILE_A_BYTES) >> 4), bk, id, (first && ks == 0 && t == 1) ? 0u : 1u);
+            }
           }
           mma_commit(&emptyB[st]);
           if (it % DR == DR - 1 || it == nk - 1) mma_commit(&tfull[b]);

@@ -29,7 +29,8 @@ def hss():
 
 @pytest.mark.parametrize("precision", ["bf16x3", "tf32x2"])
 @pytest.mark.parametrize("n,leaf,cols", [(1, 1, 1), (33, 8, 33), (127, 40, 64), (129, 16, 129), (300, 70, 300),
-                                         (1027, 128, 130), (9000, 256, 8)])
+                                         (1027, 128, 130), (9000, 256, 8),
+                                         (9001, 256, 100)])
 def test_entries(hss, precision, n, leaf, cols):
     import torch
     rng = np.random.default_rng(n)
