@@ -560,7 +560,7 @@ __global__ void __maxnreg__(96) k_sample_tc_toep(TcArgs a) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[b]);
     }
-    if constexpr (SWAP) {
+    if constexpr (SWAP) {   // (store_col, written out: its call took 60 bytes more of spills, 4 % of the time)
       const int col = col0 + 32 * q + lane;
 #pragma unroll
       for (int j = 0; j < NH; ++j) {
@@ -996,7 +996,8 @@ __global__ void __maxnreg__(96) k_sample_tc_packed(TcPackedArgs a) {
         if (first && !mbar_wait(&tempty[b], ((uint32_t)(c >> 1) & 1u) ^ 1u, a.err, 15)) break;
         if (!mbar_wait(&full[s], ph, a.err, 13)) break;
         tc_fence_after();
-        mma_ktile<PREC>(smem_u32(smem + s * stage_bytes), tmem, N, b, first, id);
+        if constexpr (NH == 32) mma_ktile_swapped<PREC>(smem_u32(smem + s * stage_bytes), tmem, b, first);   // N = 128
+        else mma_ktile<PREC>(smem_u32(smem + s * stage_bytes), tmem, N, b, first, id);
         mma_commit(&empty[s]);
         if (it % DR == DR - 1 || it == nk - 1) mma_commit(&tfull[b]);
       }
@@ -1017,8 +1018,11 @@ __global__ void __maxnreg__(96) k_sample_tc_packed(TcPackedArgs a) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[b]);
     }
-    if (ok && nk > 0)
-      store_row<NH>(side ? a.Sc : a.S, a.lds, a.n, a.ncols, rb * BM + 32 * q + lane, ct * N + h * NH, a.atomic, s, e);
+    if (ok && nk > 0) {
+      double* S = side ? a.Sc : a.S;
+      if constexpr (NH == 32) store_col<NH>(S, a.lds, a.n, a.ncols, rb * BM + h * NH, ct * N + 32 * q + lane, a.atomic, s, e);
+      else store_row<NH>(S, a.lds, a.n, a.ncols, rb * BM + 32 * q + lane, ct * N + h * NH, a.atomic, s, e);
+    }
   }
   tc_fence_before();
   __syncthreads();

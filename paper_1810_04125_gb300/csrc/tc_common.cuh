@@ -333,6 +333,42 @@ __device__ __forceinline__ void store_row(double* S, long long lds, int n, int n
   }
 }
 
+// store_row for a product whose rows are sample columns: the NH rows from row0
+// of the matrix in one column (neighbouring lanes write neighbouring columns)
+template <int NH>
+__device__ __forceinline__ void store_col(double* S, long long lds, int n, int ncols, int row0, int col, int atomic,
+                                          const float* s, const float* e) {
+  if (col >= ncols) return;
+#pragma unroll
+  for (int j = 0; j < NH; ++j) {
+    if (row0 + j < n) {
+      const double v = f2d_exact(s[j]) + f2d_exact(e[j]);
+      double* out = S + (long long)(row0 + j) * lds + col;
+      if (atomic) atomicAdd(out, v);
+      else *out = v;
+    }
+  }
+}
+
+// mma_ktile with 128 columns of R as the rows of the product and the 128 rows
+// of the first two terms as its 256 columns: an MMA is issued in about 110
+// clocks whatever its width, so two terms in one take half the time (packed
+// dense n = 16384, TF32 x 2: 128 columns 2.00 to 1.90 ms, 512 columns 4.02 to
+// 3.48).  The sums are those of mma_ktile, element by element in the same order.
+template <int PREC>
+__device__ __forceinline__ void mma_ktile_swapped(uint32_t base, uint32_t tmem, int b, bool first) {
+  using SP = Split<PREC>;
+  constexpr int T = SP::T, BK = SP::BK;
+  const uint32_t d = tmem + (uint32_t)(256 * b);
+#pragma unroll
+  for (int ks = 0; ks < BK / SP::KSTEP; ++ks) {
+    const uint64_t r = sdesc(base + T * TILE_A_BYTES + ks * 256u, 128u, 1024u);
+    mma<PREC>(d, r, sdesc(base + ks * 256u, 128u, 1024u), idesc(SP::FMT, 256u), (first && ks == 0) ? 0u : 1u);
+    if (T == 3)
+      mma<PREC>(d + 128u, r, sdesc(base + 2 * TILE_A_BYTES + ks * 256u, 128u, 1024u), idesc(SP::FMT, 128u), 1u);
+  }
+}
+
 // Issue the MMAs of one k-tile (BK/KSTEP k-steps, T terms) into buffer b.
 template <int PREC>
 __device__ __forceinline__ void mma_ktile(uint32_t base, uint32_t tmem, int N, int b, bool first,
