@@ -291,10 +291,12 @@ def run_gpu(args):
     pk, pk_kind = peaks()
     fp64_src = "derived: 152 SMs x 2 FP64 FMA/clk x 2070 MHz"
     if args.precision == "fp64":
-        ach = s0.flop_sample / (s0.ms_sample / 1e3) / 1e12
-        r_sample = {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                    "frac": ach / FP64_PEAK_TFLOPS, "kernel": "k_sample_fp64", "peak_source": fp64_src,
-                    **dict(zip(("traffic", "traffic_profile"), traffic_from_profiles("k_sample_fp64_gauss8_n16384")))}
+        # exact-split products: 36 FP16 term products per FP64 one; a symmetric
+        # A is sampled on one side (sample_launches counts the products)
+        ach = s0.flop_sample * s0.sample_launches / (2 * (s0.n_adapt + 1)) / (s0.ms_sample / 1e3) / 1e12
+        r_sample = {"bound": "tensor", "achieved": ach, "peak": pk["bf16_tflops"] / 36, "unit": "TFLOP/s",
+                    "frac": ach / (pk["bf16_tflops"] / 36), "kernel": "k_xs_mm",
+                    "peak_source": f"{pk_kind} bf16_tflops (burst) / 36 term products", "traffic": None}
     else:
         ach = s0.bytes_sample / (s0.ms_sample / 1e3) / 1e9
         r_sample = {"bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
@@ -485,9 +487,10 @@ def _sampling_roofline(st, ns, terms, tc_peak, tc_src, pk, pk_kind):
         return {"bound": "hbm", "kernel": "k_sample_tc_packed", "achieved": ach, "peak": pk["hbm_gbs"],
                 "unit": "GB/s", "peak_source": f"{pk_kind} hbm_gbs (burst)",
                 "note": "bytes = packed A per pass and orientation + R + S, and the one-time split of A"}
-    ach = sum(s.flop_sample for s in st) * terms / (ms / 1e3) / 1e12
-    return {"bound": "tensor", "kernel": "k_sample_tc_gen", "achieved": ach, "peak": tc_peak, "unit": "TFLOP/s",
-            "peak_source": tc_src, "note": f"tensor work = {terms} term products x the sampled flops"}
+    # (a symmetric A is sampled on one side: sample_launches counts the products)
+    ach = sum(s.flop_sample * s.sample_launches / (2 * (s.n_adapt + 1)) for s in st) * terms / (ms / 1e3) / 1e12
+    return {"bound": "tensor", "kernel": "k_sample_tc_toep", "achieved": ach, "peak": tc_peak, "unit": "TFLOP/s",
+            "peak_source": tc_src, "note": f"tensor work = {terms} term products x the products formed"}
 
 
 def run_config(args):
@@ -616,13 +619,13 @@ def run_config(args):
             torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / args.steps
         useful = 4.0 * n * n * d0
-        ach = useful * terms / (ms / 1e3) / 1e12
+        ach = 0.5 * useful * terms / (ms / 1e3) / 1e12   # one product: these sources are symmetric, S^c is a copy
         out = {"metric": "sampling kernel alone: S^r, S^c of one pass (generated entries)", "value": useful / (ms / 1e3) / 1e12,
                "unit": "TFLOP/s", "ms_per_step": ms, "steps": args.steps, "warmup": args.warmup,
                "config": {"workload": CONFIG_WORKLOADS[c], "n": n, "columns": d0, "precision": prec, "leaf": leaf},
                "roofline": {"bound": "tensor", "achieved": ach, "peak": tc_peak, "unit": "TFLOP/s", "frac": ach / tc_peak,
-                            "kernel": "k_sample_tc_gen", "peak_source": tc_src,
-                            "note": f"tensor work = {terms} term products x 4 n^2 d0"},
+                            "kernel": "k_sample_tc_toep" if c == "c5" else "k_sample_tc", "peak_source": tc_src,
+                            "note": f"tensor work = {terms} term products x 2 n^2 d0"},
                "clocks": clocks.summary()}
         print(json.dumps(out), flush=True)
         return
