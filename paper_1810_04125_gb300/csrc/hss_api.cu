@@ -1327,22 +1327,22 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
       CK(launch_sample_tc(s, H->o.leaf, H->o.precision, 1, w, packR, H->Sg_c + c0, H->dmax, c.d_flag + 1, &at,
                           H->toep_terms, st));
     CKS(copy_samples());
-    c.launches += 1;
-    c.sample_launches += 1;
-    H->st.sample_launches += 1;
+    c.launches += one_side ? 1 : 2;
+    c.sample_launches += one_side ? 1 : 2;
+    H->st.sample_launches += one_side ? 1 : 2;
     CK(c.timer.mark(PH_RNG, st));
     CK(cudaFreeAsync(packR, st));
   }
   CK(c.timer.mark(PH_RNG, st));
   H->st.flop_sample += (H->o.symmetric ? 2.0 : 4.0) * (double)n * (double)n * (double)w;
-  // algorithmic bytes of the sampling kernels: A read once per orientation
+  // algorithmic bytes of the sampling kernels: A read once per product formed
   // (FP64: 8 B per entry; packed TF32x2: 8 B; packed BF16x3: 6 B), R read,
   // S written
   double abytes = 0.0;
   if (H->o.op) abytes = 0.0;   // the operator's own traffic is not the library's
   else if (H->src.kind == HSS_SRC_DENSE || (H->o.precision != HSS_PREC_FP64 && H->pack_decided == 1))
     abytes = (H->o.precision == HSS_PREC_BF16X3 ? 6.0 : 8.0) * n * (double)n;
-  H->st.bytes_sample += norient * (abytes + 2.0 * 8.0 * n * (double)w);
+  H->st.bytes_sample += (one_side ? 1 : 2) * (abytes + 2.0 * 8.0 * n * (double)w);
   int* flag = c.d_flag + 8 + H->slot;
   CK(launch_nonfinite(H->Sg_r, H->dmax, n, c0, c1, flag, st));
   if (!H->sym) CK(launch_nonfinite(H->Sg_c, H->dmax, n, c0, c1, flag, st));
