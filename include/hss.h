@@ -342,7 +342,8 @@ typedef struct hss_tuning {
                                  (default 2)                                   */
   int qrcp_min_cols;          /* a node side's QRCP group takes extra CTAs
                                  (beyond one per 256 columns) only while each
-                                 keeps at least this many columns (default 4) */
+                                 keeps at least this many columns (default
+                                 4); the plain form: half, but 4 suffice      */
   int qrcp_sm_ctas;           /* CTAs per SM of the QRCP group launches: 1
                                  (512 threads), 2 (256) or 4 (128); 0 = by
                                  qrcp_wide_max_sides (default 0)              */

@@ -1471,6 +1471,15 @@ hss_status run_qrcp(Ctx& c, const std::vector<QrcpReq>& reqs, std::vector<double
   // tuning fixes).  Shapes: 0 = 128 threads, four CTAs per SM; 1 = 256, two;
   // 2 = 512, one.
   const hss_tuning tun = tuning_get();
+  // The plain form takes half as many columns per CTA, down to 4: its levels have
+  // one side a node where A = A^T, so fewer and longer groups share the SMs
+  // (8 against 16 columns, ID phase: Gaussian 8-D n = 8192 148.0 to 141.3 ms,
+  // Toeplitz n = 1024 0.85 to 0.76; whole Laplace n = 4001 compressions 2.7 %
+  // faster to 2.7 % slower over four sample matrices; the mixed benchmark, both
+  // sides, 411.6 with either).
+  bool plain = true;
+  for (const QrcpReq& q : reqs) plain = plain && q.H->o.precision == HSS_PREC_FP64;
+  const int min_cols = plain ? std::max(std::min(tun.qrcp_min_cols, 4), tun.qrcp_min_cols / 2) : tun.qrcp_min_cols;
   int wide = (int)nj <= tun.qrcp_wide_max_sides ? 1 : 0;
   if (tun.qrcp_sm_ctas) wide = tun.qrcp_sm_ctas == 4 ? 0 : (tun.qrcp_sm_ctas == 2 ? 1 : 2);
   if (c.qrcp_cap_d != dmx || c.qrcp_cap_w != wide) {
@@ -1519,7 +1528,7 @@ hss_status run_qrcp(Ctx& c, const std::vector<QrcpReq>& reqs, std::vector<double
       auto top = pq.top();
       pq.pop();
       const size_t i = top.second;
-      if (mj[i] / (P[i] + 1) < tun.qrcp_min_cols) continue;   // keep enough columns per CTA
+      if (mj[i] / (P[i] + 1) < min_cols) continue;   // keep enough columns per CTA
       P[i]++;
       used++;
       pq.push({wk[i] / P[i], i});
