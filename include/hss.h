@@ -281,7 +281,9 @@ hss_status hss_compress_batched(const hss_source* A, const hss_opts* opts, int c
  * couples with B21^T, B12^T.  A partial result (HSS_ERR_NOT_CONVERGED)
  * couples the children of its uncompressed nodes through the dense blocks
  * it kept.  X, Y: device col-major n x nrhs (ldx, ldy >= n); Y is
- * overwritten.  Asynchronous on the stream. */
+ * overwritten.  Asynchronous on the stream, but for the handle's first
+ * product or entry call outside of a capture: it lays out the task lists and
+ * index tables that the handle keeps, and waits for the stream. */
 hss_status hss_matvec(hss_matrix H, int nrhs, const double* X, long long ldx,
                       double* Y, long long ldy, int transpose, void* stream);
 
@@ -296,7 +298,8 @@ hss_status hss_matvec(hss_matrix H, int nrhs, const double* X, long long ldx,
  * a partial result where they apply.  Cost: for each row index the products
  * along its path to the root (sum over its ancestors of k^2), and k per
  * entry.  I (nr), J (nc): device int arrays of indices in [0, n); out: device
- * col-major nr x nc, ld ldo >= nr.  Uses a temporary device buffer; returns
+ * col-major nr x nc, ld ldo >= nr.  Uses a temporary device buffer and the
+ * handle's index tables (see hss_matvec); returns
  * after a sync of the stream; HSS_ERR_ARG (entries left zero) when an index
  * is out of range. */
 hss_status hss_get_entries(hss_matrix H, int nr, const int* I, int nc, const int* J, double* out,

@@ -13,10 +13,11 @@
 // Every product of terms is exact in FP32; partial sums are kept short in
 // TMEM and carried in float-float registers (see "Accumulation" below).
 //
-// Two kernels share the tile format: the packed kernel streams a dense A that
-// was split once into canonical tiles (cp.async.bulk into an mbarrier ring);
-// the generating kernel computes the entries (Toeplitz table lookups, point
-// kernels) in its producer warps.  In both, one thread issues tcgen05.mma, the
+// Three kernels share the tile format: the packed kernel streams an A that was
+// split once into canonical tiles (cp.async.bulk into an mbarrier ring); the
+// generating kernel computes the entries of a point kernel in its producer
+// warps; the Toeplitz kernel reads every tile out of a strip of the few core
+// matrices that such tiles are made of.  One thread issues tcgen05.mma, the
 // R tile arrives pre-packed by bulk copy, and every mbarrier wait is bounded
 // (about 2 s of %globaltimer): on expiry the kernel records an error code,
 // leaves its loops, frees its TMEM and returns.
