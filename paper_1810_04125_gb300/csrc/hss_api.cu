@@ -698,6 +698,7 @@ GemmJob gemm_job() {
 
 // ---- exact-split FP64 products (k_gemm_xs.cu)
 constexpr size_t kXsCap = size_t(2) << 30;   // digits of the operands of one launch
+constexpr size_t kXsMask = sizeof(unsigned) * 2 * XS_TM;   // bits of a tile's elements
 constexpr int kSms = 152;
 constexpr size_t kXsKeep = size_t(4) << 30;  // digits of generated sources kept over a compression
 constexpr double kXsMinUs = 30.0;            // FP64-pipe time from which the exact-split launches pay
@@ -732,7 +733,7 @@ int xs_seg_ktiles(const std::vector<std::pair<long long, int>>& tiles) {
   return best;
 }
 
-// One launch set (maxima, digits, product) over jobs[b0..b1).
+// One launch set (maxima, digits, check, product) over the jobs.
 hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs) {
   const int nj = (int)jobs.size();
   std::vector<std::pair<long long, int>> tl;
@@ -740,8 +741,8 @@ hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs) {
     tl.push_back({(long long)((j.M + XS_TM - 1) / XS_TM) * ((j.N + XS_TN - 1) / XS_TN), (j.K + XS_BK - 1) / XS_BK});
   const int g = xs_seg_ktiles(tl);
   size_t nz = 8, np = 0;   // words of the zeroed region (word 0: the wait flag of calls without flags); packed bytes
-  std::vector<size_t> oea(nj), oeb(nj), onb(nj), ocnt(nj), ows(nj), opa(nj), opb(nj);
-  std::vector<int> pm(nj + 1, 0), pp(nj + 1, 0), pt(nj + 1, 0);
+  std::vector<size_t> oea(nj), oeb(nj), onb(nj), ocnt(nj), ost(nj), ows(nj), opa(nj), opb(nj), omk(nj);
+  std::vector<int> pm(nj + 1, 0), pp(nj + 1, 0), pt(nj + 1, 0), pc(nj + 1, 0);
   size_t nws = 0;
   for (int i = 0; i < nj; ++i) {
     GemmJob& j = jobs[i];
@@ -752,13 +753,16 @@ hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs) {
     oeb[i] = nz; nz += j.N;
     onb[i] = nz; nz += j.N;
     ocnt[i] = nz; nz += nrb * ncb;
+    ost[i] = nz; nz += nrb * ncb;
     ows[i] = nws;
     if (j.nseg > 1) nws += nrb * ncb * 2 * XS_TM * XS_TN;
     opa[i] = np; np += nrb * j.nkt * xs_tile_bytes(0);
     opb[i] = np; np += ncb * j.nkt * xs_tile_bytes(1);
+    omk[i] = np; np += nrb * ncb * kXsMask;
     pm[i + 1] = pm[i] + xs_max_units(j.M, j.N, j.K);
     pp[i + 1] = pp[i] + xs_pack_units(j.M, j.N, j.K);
     pt[i + 1] = pt[i] + (int)(nrb * ncb) * j.nseg;
+    pc[i + 1] = pc[i] + (int)(nrb * ncb);
   }
   const size_t zb = Scratch::rnd(sizeof(unsigned) * nz) + sizeof(unsigned long long) * nws;
   CK(c.xz.ensure(zb, c.st));
@@ -773,20 +777,25 @@ hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs) {
     j.ws = (unsigned long long*)(c.xz.p + Scratch::rnd(sizeof(unsigned) * nz)) + ows[i];
     j.pa = (unsigned char*)c.xp.p + opa[i];
     j.pb = (unsigned char*)c.xp.p + opb[i];
+    j.state = z + ost[i];
+    j.mask = (unsigned*)(c.xp.p + omk[i]);
   }
   Staging sg;
   const size_t oj = sg.put(jobs.data(), jobs.size() * sizeof(GemmJob));
   const size_t om = sg.put(pm.data(), sizeof(int) * (nj + 1));
   const size_t op = sg.put(pp.data(), sizeof(int) * (nj + 1));
   const size_t ot = sg.put(pt.data(), sizeof(int) * (nj + 1));
+  const size_t oc = sg.put(pc.data(), sizeof(int) * (nj + 1));
   char* dev;
   CKS(sg.send(c, &dev));
   CK(cudaMemsetAsync(c.xz.p, 0, zb, c.st));
   const GemmJob* dj = (const GemmJob*)(dev + oj);
   CK(launch_xs_max(dj, (const int*)(dev + om), nj, pm[nj], c.st));
   CK(launch_xs_pack(dj, (const int*)(dev + op), nj, pp[nj], c.st));
-  CK(launch_xs_mm(dj, (const int*)(dev + ot), nj, pt[nj], nullptr, c.d_flag ? c.d_flag + 5 : (int*)z, c.st));
-  c.launches += 3;
+  int* err = c.d_flag ? c.d_flag + 5 : (int*)z;
+  CK(launch_xs_check(dj, (const int*)(dev + oc), nj, pc[nj], err, c.st));
+  CK(launch_xs_mm(dj, (const int*)(dev + ot), nj, pt[nj], false, err, c.st));
+  c.launches += 4;
   return HSS_OK;
 }
 
@@ -1100,10 +1109,11 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
   const size_t onb = nz; nz += w;
   const size_t per_cnt = (size_t)chunk * ncb;
   const size_t ocnt = nz; nz += per_cnt * no * nchunk;
+  const size_t ost = nz; nz += per_cnt * no * nchunk;
   const size_t per_ws = nseg > 1 ? per_cnt * 2 * XS_TM * XS_TN : 0;
   const size_t zw = Scratch::rnd(sizeof(unsigned) * nz);
   const size_t zb = zw + sizeof(unsigned long long) * per_ws * no;
-  const size_t bB = (size_t)ncb * nkt * xs_tile_bytes(1);
+  const size_t bB = (size_t)ncb * nkt * xs_tile_bytes(1) + per_cnt * no * nchunk * kXsMask;
   if (c.xz.ensure(zb, st) != cudaSuccess ||
       c.xp.ensure(bB + (keep ? 0 : chunk * row_bytes * no), st) != cudaSuccess) {
     cudaGetLastError();   // no memory for the digits
@@ -1111,8 +1121,9 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
   }
   unsigned* z = (unsigned*)c.xz.p;
   unsigned long long* ws = (unsigned long long*)(c.xz.p + zw);
-  unsigned char* pB = (unsigned char*)c.xp.p;
-  unsigned char* pA = pB + bB;
+  unsigned* mask = (unsigned*)c.xp.p;
+  unsigned char* pB = (unsigned char*)c.xp.p + per_cnt * no * nchunk * kXsMask;
+  unsigned char* pA = (unsigned char*)c.xp.p + bB;
   unsigned* ea = keep ? keep->ea : z + oea;
   std::vector<GemmJob> jobs;
   GemmJob jr = gemm_job();   // R alone: maxima and digits
@@ -1126,6 +1137,7 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
   for (int q = 0; q < nchunk; ++q) {
     const int r0 = q * chunk * XS_TM, rows = std::min(n - r0, chunk * XS_TM);
     int units = 0;
+    std::vector<int> tiles(1, 0);
     pre.push_back(0);
     for (int o = 0; o < no; ++o) {
       GemmJob j = jr;
@@ -1137,10 +1149,15 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
       j.nseg = nseg;
       j.cnt = z + ocnt + (size_t)(q * no + o) * per_cnt;
       j.ws = ws + (size_t)o * per_ws;
+      j.state = z + ost + (size_t)(q * no + o) * per_cnt;
+      j.mask = mask + (size_t)(q * no + o) * per_cnt * (kXsMask / sizeof(unsigned));
       jobs.push_back(j);
-      units += (rows + XS_TM - 1) / XS_TM * ncb * nseg;
+      const int nt = (rows + XS_TM - 1) / XS_TM * ncb;
+      units += nt * nseg;
       pre.push_back(units);
+      tiles.push_back(tiles.back() + nt);
     }
+    pre.insert(pre.end(), tiles.begin(), tiles.end());
   }
   Staging sg;
   const size_t oj = sg.put(jobs.data(), jobs.size() * sizeof(GemmJob));
@@ -1168,13 +1185,24 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
       c.launches++;
     }
     if (nseg > 1 && q > 0) CK(cudaMemsetAsync(ws, 0, sizeof(unsigned long long) * per_ws * no, st));
-    const size_t op_q = 4 + (size_t)q * (no + 1);
-    CK(launch_xs_mm(dj + 1 + (size_t)q * no, dp + op_q, no, pre[op_q + no], (int*)z, err ? err : (int*)z + 1, st));
-    c.launches++;
+    const size_t op_q = 4 + (size_t)q * 2 * (no + 1), oc_q = op_q + no + 1;
+    const GemmJob* djq = dj + 1 + (size_t)q * no;
+    CK(launch_xs_check(djq, dp + oc_q, no, pre[oc_q + no], err ? err : (int*)z, st));
+    CK(launch_xs_mm(djq, dp + op_q, no, pre[op_q + no], true, err ? err : (int*)z, st));
+    c.launches += 2;
   }
   if (keep) keep->have = true;
-  // operands that the digits cannot hold: the FP64 kernel instead
-  CK(launch_sample_fp64(s, w, R, ldr, Sr, Sc, lds, st, (const int*)z));
+  // what the digits do not settle by the FP64 kernel (S^c: by its own tiles, or
+  // S^r's where it is the same)
+  XsTiles x[2];
+  for (int o = 0; o < no; ++o) {
+    x[o].state = z + ost + (size_t)o * per_cnt;
+    x[o].mask = mask + (size_t)o * per_cnt * (kXsMask / sizeof(unsigned));
+    x[o].stride = (long long)per_cnt * no;
+    x[o].chunk = chunk;
+    x[o].ncb = ncb;
+  }
+  CK(launch_sample_fp64(s, w, R, ldr, Sr, Sc, lds, st, &x[0], &x[no - 1]));
   c.launches += (Sr ? 1 : 0) + (Sc ? 1 : 0);
   *done = true;
   return HSS_OK;

@@ -89,6 +89,21 @@ struct GemmJob {
   unsigned* cnt;
   double* dup;
   int nseg;
+  // what every output tile still needs (XS_FMA, XS_PART; zeroed by the caller),
+  // and with XS_PART the elements the digits do not settle: 64 bits a row, 128
+  // rows a tile
+  unsigned* state;
+  unsigned* mask;
+};
+enum : unsigned { XS_FMA = 1u, XS_PART = 4u };
+// The tile states of a sampling call whose rows were cut into chunks of `chunk`
+// row blocks: tile (row block, column tile) at (rb / chunk) stride +
+// (rb % chunk) ncb + column tile.
+struct XsTiles {
+  const unsigned* state;
+  const unsigned* mask;
+  long long stride;
+  int chunk, ncb;
 };
 // One tile of an operand to pack: job, operand (0 = A, 1 = B), row tile, k tile.
 struct PackUnit { int job, which, tile, kt; };
@@ -211,10 +226,10 @@ struct ProdTask {
 // Launch wrappers (return cudaError_t of the launch).
 cudaError_t launch_random_normal(unsigned long long seed, int n, int col0, int ncols,
                                  double* R, long long ldr, int round_mode, cudaStream_t st);
-// only_if: device flag (may be null); the launch does nothing while it is 0
+// tr, tc: only what an exact-split call left out of Sr, Sc
 cudaError_t launch_sample_fp64(const SrcDev& src, int ncols, const double* R, long long ldr,
                                double* Sr, double* Sc, long long lds, cudaStream_t st,
-                               const int* only_if = nullptr);
+                               const XsTiles* tr = nullptr, const XsTiles* tc = nullptr);
 // tcgen05 mixed-precision sampling with entries generated in the kernel
 // (k_sample_tc.cu); Rp is R packed by launch_pack_r; *used_atomic tells
 // whether S had to be zeroed beforehand (K split across CTAs).  toep: for a
@@ -260,11 +275,14 @@ int xs_max_units(int M, int N, int K);
 int xs_pack_units(int M, int N, int K);
 cudaError_t launch_xs_max(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, cudaStream_t st);
 cudaError_t launch_xs_pack(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, cudaStream_t st);
-// flag == nullptr: a tile whose operands the digits cannot hold (non-finite,
-// or a column of B of uneven magnitude) is computed by FP64 FMAs in the same
-// launch; otherwise it is left out and *flag set (for the sampling, whose A
-// has no operand view).
-cudaError_t launch_xs_mm(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, int* flag, int* err,
+// Which results the digits settle to FP64's accuracy: the state of every tile,
+// before the product (prefix: tiles).
+cudaError_t launch_xs_check(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int ntiles, int* err,
+                            cudaStream_t st);
+// XS_FMA tiles and the marked elements of XS_PART tiles are computed by FP64 FMAs
+// in the same launch, or left out (leave: for the sampling, whose A has no
+// operand view, and whose FP64 kernel fills them in).
+cudaError_t launch_xs_mm(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, bool leave, int* err,
                          cudaStream_t st);
 // The sampling operand A - D^(L) (trans 0) or its transpose (1), rows
 // [row0, row0 + rows): the largest entry of every row (zeroed by the caller),

@@ -27,7 +27,8 @@
 // f = sum (b_p - 128) 2^(8 p): eight signed digits, exact in FP16.  The
 // columns of B are cut the same way.  With digit s = 0 the leading one, the
 // products of digits p and q weigh 2^-8(p+q); those with p + q <= 7 are
-// formed (the rest is below 2^-62 of the largest product).  Digit 0 is at most
+// formed (the rest is below 2^-57 of row maximum x column maximum a term, and
+// near 2^-60 for digits of either sign).  Digit 0 is at most
 // 2^6, the others 2^7, so the products of weight s >= 1 over K terms sum to
 // at most K s 2^14: exact in the FP32 accumulator for K up to 128.
 //
@@ -48,8 +49,20 @@
 //
 // What the digits cannot hold: NaN and Inf, and a column of B whose elements
 // are of uneven magnitude (fewer than 15/16 of them within 2^-10 of the
-// largest): there an element of C may be made of small terms only, which a
-// common scale would cut.  Such a tile is computed with FP64 FMAs.
+// largest).  Such a tile is computed with FP64 FMAs.
+//
+// What they do not settle.  The scales are those of whole rows and columns, so
+// an element of C keeps FP64's accuracy only if its own terms are not all small
+// against them: a row whose one large entry meets a zero of B has only terms
+// that were cut (with the row (1, 1e-20, ...) all of them).  In units of f, the
+// pairs left out are at most 7.03 2^62 a term and the operands' roundings 2^62,
+// together 2^65.01: K 2^65.01 in all.  FP64 FMAs guarantee K 2^-53 S, S = sum
+// |A(i,l) B(l,j)|, and the digits no less where S >= 2^118 (in f), an
+// 1/16 to 1/64 of (largest of the row) x (largest of the column).  k_xs_check
+// forms a lower bound of S for every element from the two leading digits, an
+// FP16 product that stops as soon as all elements of its tile have reached it
+// (for even data after the first 32 of K); elements that never do are computed
+// with FP64 FMAs, or, if they are more than one in eight, the whole tile.
 #include <cuda_fp16.h>
 #include <stdint.h>
 
@@ -500,26 +513,30 @@ __device__ __forceinline__ double fixed_value(long long hi, long long lo, int e2
 // The tile's results (column-padded, in shared memory) to C: lanes along the
 // contiguous direction.
 constexpr int XLD = XS_TN + 1;
+__device__ __forceinline__ void store_one(const GemmJob& jb, int i, int jj, double v) {
+  if (jb.beta != 0.0) {
+    const double c0 = op_row(jb.C0, i)[(long long)jj * jb.C0.cs];
+    v += jb.beta == 1.0 ? c0 : jb.beta * c0;
+  }
+  int r = jb.c_rows ? jb.c_rows[i] : i;
+  double* base = jb.C;
+  if (r >= jb.c_split) { base = jb.C2; r -= jb.c_split; }
+  const long long off = (long long)r * jb.c_rs + (long long)jj * jb.c_cs;
+  if (jb.gamma != 0.0) v += jb.gamma == 1.0 ? base[off] : jb.gamma * base[off];
+  base[off] = v;
+  if (jb.dup) jb.dup[off] = v;
+}
+// (mask: elements to leave out, or NULL)
 template <int NR = XS_TM>
-__device__ __forceinline__ void store_tile(const GemmJob& jb, const double* sm, int i0, int j0, int t) {
+__device__ __forceinline__ void store_tile(const GemmJob& jb, const double* sm, int i0, int j0, int t,
+                                           const unsigned* mask = nullptr) {
   const bool row_major = jb.c_cs == 1;
-  const double beta = jb.beta, gamma = jb.gamma;
   for (int q = t; q < NR * XS_TN; q += XW * 32) {
     const int il = row_major ? q / XS_TN : q % NR, jl = row_major ? q % XS_TN : q / NR;
     const int i = i0 + il, jj = j0 + jl;
     if (i >= jb.M || jj >= jb.N) continue;
-    double v = sm[il * XLD + jl];
-    if (beta != 0.0) {
-      const double c0 = op_row(jb.C0, i)[(long long)jj * jb.C0.cs];
-      v += beta == 1.0 ? c0 : beta * c0;
-    }
-    int r = jb.c_rows ? jb.c_rows[i] : i;
-    double* base = jb.C;
-    if (r >= jb.c_split) { base = jb.C2; r -= jb.c_split; }
-    const long long off = (long long)r * jb.c_rs + (long long)jj * jb.c_cs;
-    if (gamma != 0.0) v += gamma == 1.0 ? base[off] : gamma * base[off];
-    base[off] = v;
-    if (jb.dup) jb.dup[off] = v;
+    if (mask && (mask[2 * il + jl / 32] >> (jl % 32) & 1u)) continue;
+    store_one(jb, i, jj, sm[il * XLD + jl]);
   }
 }
 
@@ -587,11 +604,33 @@ __device__ void fp64_share(const GemmJob& jb, double* sm, int i0, int j0, int pa
   else fp64_rows<4, 4>(jb, sm, r0, j0, t);
 }
 
+// The marked elements of every nseg-th row of the tile by FP64 FMAs: a warp an
+// element, its lanes along K.
+__device__ __noinline__ void fix_rows(const GemmJob& jb, const unsigned* mask, int i0, int j0, int seg, int warp, int lane) {
+  for (int q = warp; seg + q * jb.nseg < XS_TM; q += XW) {
+    const int il = seg + q * jb.nseg, i = i0 + il;
+    if (i >= jb.M) return;
+    const double* a = op_row(jb.A, i);
+    for (int h = 0; h < 2; ++h) {
+      for (unsigned m = mask[2 * il + h]; m; m &= m - 1u) {   // (none past N)
+        const int jj = j0 + 32 * h + __ffs(m) - 1;
+        double v = 0.0;
+#pragma unroll 4
+        for (int l = lane; l < jb.K; l += 32)
+          v = __fma_rn(a[(long long)l * jb.A.cs], op_row(jb.B, l)[(long long)jj * jb.B.cs], v);
+#pragma unroll
+        for (int o = 16; o; o /= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) store_one(jb, i, jj, jb.alpha * v);
+      }
+    }
+  }
+}
+
 __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const int* __restrict__ prefix, int njobs,
-                                          int nunits, int* flag, int* err) {
+                                          int nunits, int leave, int* err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ GemmJob sj;
-  __shared__ int s_bad, s_last;
+  __shared__ int s_last;
   uint64_t* full = (uint64_t*)(smem + XNS * XSTAGE);
   uint64_t* empty = full + XNS;
   uint64_t* tfull = empty + XNS;    // one per issuing warp
@@ -603,7 +642,6 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
   const int ji = find_job(prefix, njobs, unit);
   if (tid == 0) {
     sj = jobs[ji];
-    s_bad = 0;
     for (int s = 0; s < XNS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], XMW); }
     for (int s = 0; s < XMW; ++s) { mbar_init(&tfull[s], 1); mbar_init(&tempty[s], XW); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -613,24 +651,11 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
   const int ntn = (sj.N + XS_TN - 1) / XS_TN;
   const int t = u / nseg, seg = u % nseg;   // column tiles fastest: the tiles of one row block share A through L2
   const int ti = t / ntn, tj = t % ntn, i0 = ti * XS_TM, j0 = tj * XS_TN;
-  // operands the digits cannot hold?
-  if (tid < XS_TM) {
-    if (i0 + tid < sj.M && sj.ea[i0 + tid] >= HI_INF) s_bad = 1;
-  } else if (tid < XS_TM + XS_TN) {
-    const int c = j0 + tid - XS_TM;
-    if (c < sj.N) {
-      const unsigned key = sj.eb[c];
-      if (key >= HI_INF || (key != 0u && (unsigned long long)sj.nb[c] * 16ull < 15ull * (unsigned)sj.K)) s_bad = 1;
-    }
-  }
-  __syncthreads();
+  const unsigned state = sj.state[t];
   double* tile_sm = (double*)smem;   // the results, once the stages are done with
-  if (s_bad) {
-    if (flag) {
-      if (tid == 0) atomicOr(flag, 1);
-    } else if (warp > XMW) {
+  if (state & XS_FMA) {
+    if (!leave && warp > XMW)
       fp64_share(sj, tile_sm, i0, j0, seg + nseg * share, nseg * shares, tid - (1 + XMW) * 32);
-    }
     return;
   }
   if (share > 0) return;
@@ -727,13 +752,160 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
       }
     }
     bar_drain();   // (every drain warp is here: all products and copies are done)
-    if (last) store_tile(sj, tile_sm, i0, j0, t512);
+    const unsigned* mask = state & XS_PART ? sj.mask + (size_t)t * (2 * XS_TM) : nullptr;
+    if (last) store_tile(sj, tile_sm, i0, j0, t512, mask);
+    if (mask && !leave) fix_rows(sj, mask, i0, j0, seg, warp - 1 - XMW, lane);
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  }
+}
+
+// ------------------------------------------------- what the digits settle
+// One CTA per tile.  The magnitude of an element by its two leading digits,
+// h = max(|d0 + d1 / 256| - 2^-9, 0) <= |f| 2^-56 up to two roundings to FP16
+// (the digits below are at most 1.004 2^-9), so sum h_A h_B, with 64 for the
+// 2^118 of S above and 1.5 % for the roundings, is a lower bound of S.  One
+// k-tile first, then three at a time, from the tile's own place outwards
+// (matrices that decay have their large entries near the diagonal).  Bound by
+// the latency of its few loads: 5 to 11 us a launch (dense n = 6001, 200 columns:
+// 1.39 to 1.40 ms for the call; a product of 2048 columns with twelve launch
+// sets 3.75 to 3.87).
+constexpr int CKT = 3;                                   // most k-tiles a round
+constexpr uint32_t CK_SMEM = CKT * (XA + XB);
+constexpr int CK_MOST = XS_TM * XS_TN / 8;               // elements to compute one by one
+constexpr float CK_ENOUGH = 65.0f;
+
+__device__ __forceinline__ uint32_t lead_mag(uint32_t d0, uint32_t d1) {   // two FP16 digits each
+  const __half2 v = __hfma2(*(const __half2*)&d1, __half2half2(__ushort_as_half((unsigned short)0x1C00)),   // 2^-8
+                            *(const __half2*)&d0);
+  const __half2 h = __hmax2(__hsub2(__habs2(v), __float2half2_rn(0.00197f)), __float2half2_rn(0.0f));
+  return *(const uint32_t*)&h;
+}
+
+__global__ void __launch_bounds__(256, 5) k_xs_check(const GemmJob* __restrict__ jobs, const int* __restrict__ prefix,
+                                                     int njobs, int* err) {
+  __shared__ __align__(1024) uint8_t smem[CK_SMEM];
+  __shared__ GemmJob sj;
+  __shared__ uint64_t bar;
+  __shared__ uint32_t s_tmem;
+  __shared__ unsigned s_free[2], s_cnt;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  int ji = 0;   // (one round of loads up to 256 jobs; find_job's chain is eight)
+  for (int j = tid; j - tid < njobs; j += 256) ji += __syncthreads_count(j < njobs && prefix[j + 1] <= (int)blockIdx.x);
+  if (tid == 0) {
+    sj = jobs[ji];
+    s_cnt = 0u;
+    mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                 "r"((uint32_t)XS_TN)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    tc_fence_before();
+  }
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_tmem;
+  const int t = blockIdx.x - prefix[ji], ntn = (sj.N + XS_TN - 1) / XS_TN;
+  const int ti = t / ntn, tj = t % ntn, i0 = ti * XS_TM, j0 = tj * XS_TN;
+  const int nkt = sj.nkt, kt0 = (i0 + XS_TM / 2) / XS_BK % nkt;
+  const uint8_t* gA = sj.pa + (size_t)ti * nkt * (XD * (size_t)XA);
+  const uint8_t* gB = sj.pb + (size_t)tj * nkt * (XD * (size_t)XB);
+  uint4 d[3][2];   // a thread's 16-byte chunks of one k-tile: two of A, one of B, both digits
+  auto fetch = [&](int k) {   // kt0, kt0 + 1, kt0 - 1, kt0 + 2, ...
+    int kg = kt0 + (k & 1 ? (k + 1) / 2 : -(k / 2));   // (-nkt < . < 2 nkt)
+    if (kg >= nkt) kg -= nkt;
+    if (kg < 0) kg += nkt;
+    const uint8_t* pa = gA + (size_t)kg * (XD * (size_t)XA) + tid * 16;
+    const uint8_t* pb = gB + (size_t)kg * (XD * (size_t)XB) + tid * 16;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      d[0][x] = *(const uint4*)(pa + x * XA);
+      d[1][x] = *(const uint4*)(pa + x * XA + 4096);
+      d[2][x] = *(const uint4*)(pb + x * XB);
+    }
+  };
+  fetch(0);
+  // operands the digits cannot hold; rows and columns of zeros have no terms
+  int bad = 0;
+  if (tid < XS_TM) {
+    bad = i0 + tid < sj.M && sj.ea[i0 + tid] >= HI_INF;
+  } else if (tid < XS_TM + XS_TN) {
+    const int c = j0 + tid - XS_TM;
+    const unsigned key = c < sj.N ? sj.eb[c] : 0u;
+    bad = key >= HI_INF || (key != 0u && (unsigned long long)sj.nb[c] * 16ull < 15ull * (unsigned)sj.K);
+    const unsigned fr = __ballot_sync(0xffffffffu, key == 0u);
+    if (lane == 0) s_free[(tid - XS_TM) / 32] = fr;
+  }
+  bad = __syncthreads_or(bad);
+  const int row = 32 * (warp % 4) + lane, h = warp / 4;   // a thread's row and half of the columns
+  const bool row_free = i0 + row >= sj.M || sj.ea[i0 + row] == 0u;
+  const unsigned col_free = s_free[h];
+  unsigned fail = 0u;
+  bool ok = true;
+  int more = !bad;
+  for (int it = 0, done = 0; done < nkt && more; ++it) {
+    const int nk = it ? min(CKT, nkt - done) : 1;
+    if (it == 1) fetch(done);
+    for (int kt = 0; kt < nk; ++kt) {
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+        *(uint4*)(smem + (x < 2 ? kt * XA + x * 4096u : CKT * XA + kt * XB) + tid * 16u) =
+            make_uint4(lead_mag(d[x][0].x, d[x][1].x), lead_mag(d[x][0].y, d[x][1].y),
+                       lead_mag(d[x][0].z, d[x][1].z), lead_mag(d[x][0].w, d[x][1].w));
+      if (it && done + kt + 1 < nkt) fetch(done + kt + 1);   // (for the next round, too, while this one is multiplied)
+    }
+    fence_async_smem();
+    __syncthreads();
+    if (warp == 0) {
+      if (elect_one()) {
+        tc_fence_after();
+        const uint32_t id = idesc(0u, (uint32_t)XS_TN);
+        for (int kt = 0; kt < nk; ++kt) {
+          const uint64_t ad = sdesc(smem_u32(smem + kt * XA), 128u, 512u);
+          const uint64_t bd = sdesc(smem_u32(smem + CKT * XA + kt * XB), 128u, 512u);
+#pragma unroll
+          for (int ks = 0; ks < XS_BK / 16; ++ks)
+            mma_f16(tmem, ad + (uint64_t)(ks * 16), bd + (uint64_t)(ks * 16), id, it + kt + ks > 0 ? 1u : 0u);
+        }
+        mma_commit(&bar);
+      }
+      __syncwarp();
+    }
+    ok = mbar_wait_warp(&bar, (uint32_t)it & 1u, err, 37);
+    tc_fence_after();
+    fail = 0u;
+    if (ok) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        float v[16];
+        tmem_ld16_nw(tmem + ((uint32_t)(32 * (warp % 4)) << 16) + (uint32_t)(32 * h + 16 * c), v);
+        tmem_wait_ld();
+#pragma unroll
+        for (int x = 0; x < 16; ++x) fail |= v[x] >= CK_ENOUGH ? 0u : 1u << (16 * c + x);
+      }
+      fail = row_free ? 0u : fail & ~col_free;
+    }
+    tc_fence_before();
+    if (__syncthreads_or(!ok)) { ok = false; break; }
+    more = __syncthreads_or(fail != 0u);
+    done += nk;
+  }
+  if (more && ok) {
+    atomicAdd(&s_cnt, (unsigned)__popc(fail));
+    sj.mask[(size_t)t * (2 * XS_TM) + 2 * row + h] = fail;
+  }
+  __syncthreads();
+  if (tid == 0 && (bad || !ok || more)) sj.state[t] = !bad && ok && s_cnt <= CK_MOST ? XS_PART : XS_FMA;
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)XS_TN) : "memory");
   }
 }
 
@@ -760,15 +932,22 @@ cudaError_t launch_xs_pack(const GemmJob* jobs_dev, const int* prefix_dev, int n
   return cudaGetLastError();
 }
 
-cudaError_t launch_xs_mm(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, int* flag, int* err,
+cudaError_t launch_xs_check(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int ntiles, int* err,
+                            cudaStream_t st) {
+  if (ntiles <= 0) return cudaSuccess;
+  k_xs_check<<<ntiles, 256, 0, st>>>(jobs_dev, prefix_dev, njobs, err);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_xs_mm(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, bool leave, int* err,
                          cudaStream_t st) {
   if (nunits <= 0) return cudaSuccess;
   const size_t sm = (size_t)XNS * XSTAGE + 8 * (2 * XNS + 2 * XMW) + 16;
   cudaError_t e = cudaFuncSetAttribute(k_xs_mm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  // helpers where the units leave SMs idle (with a flag the caller falls back)
-  const int shares = flag || nunits > 304 ? 1 : std::min(8, 608 / nunits);
-  k_xs_mm<<<nunits * shares, XTHREADS, sm, st>>>(jobs_dev, prefix_dev, njobs, nunits, flag, err);
+  // helpers where the units leave SMs idle
+  const int shares = leave || nunits > 304 ? 1 : std::min(8, 608 / nunits);
+  k_xs_mm<<<nunits * shares, XTHREADS, sm, st>>>(jobs_dev, prefix_dev, njobs, nunits, leave ? 1 : 0, err);
   return cudaGetLastError();
 }
 

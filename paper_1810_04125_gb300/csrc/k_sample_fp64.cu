@@ -18,11 +18,43 @@ namespace {
 
 constexpr int BM = 64, BN = 64, BK = 16;
 
+// Of the tile's rows, the elements marked in mask (64 bits a row of the 128-row
+// tile that holds this one): a warp an element, its lanes along k.
 template <bool TRANS>
+__device__ __noinline__ void marked_elements(const SrcDev& src, int ncols, const double* R, long long ldr, double* S,
+                                             long long lds, const unsigned* mask) {
+  const int lane = threadIdx.x % 32;
+  for (int il = threadIdx.x / 32; il < BM; il += 8) {
+    const int i = blockIdx.x * BM + il, im = (blockIdx.x % 2) * BM + il;
+    if (i >= src.n) return;
+    for (int h = 0; h < 2; ++h) {
+      for (unsigned m = mask[2 * im + h]; m; m &= m - 1u) {
+        const int c = blockIdx.y * BN + 32 * h + __ffs(m) - 1;
+        if (c >= ncols) break;
+        double v = 0.0;
+#pragma unroll 4
+        for (int k = lane; k < src.n; k += 32)
+          if (src.leaf_id[k] != src.leaf_id[i])
+            v = __fma_rn(TRANS ? entry(src, k, i) : entry(src, i, k), R[k + (long long)c * ldr], v);
+#pragma unroll
+        for (int o = 16; o; o /= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) S[(long long)i * lds + c] = v;
+      }
+    }
+  }
+}
+
+// GATED: only what `only` asks for.
+template <bool TRANS, bool GATED>
 __global__ void __launch_bounds__(256) k_sample_fp64(SrcDev src, int ncols, const double* __restrict__ R,
                                                      long long ldr, double* __restrict__ S, long long lds,
-                                                     const int* only_if) {
-  if (only_if && *only_if == 0) return;
+                                                     XsTiles only) {
+  if (GATED) {   // (64 x 64 tiles here, 128 x 64 there)
+    const int rb = blockIdx.x / 2;
+    const long long t = (rb / only.chunk) * only.stride + (long long)(rb % only.chunk) * only.ncb + blockIdx.y;
+    if (only.state[t] & XS_PART) marked_elements<TRANS>(src, ncols, R, ldr, S, lds, only.mask + 256 * t);
+    if (!(only.state[t] & XS_FMA)) return;
+  }
   __shared__ double As[BK][BM + 2];
   __shared__ double Rs[BK][BN + 2];
   const int n = src.n;
@@ -82,12 +114,19 @@ __global__ void __launch_bounds__(256) k_sample_fp64(SrcDev src, int ncols, cons
 }  // namespace
 
 cudaError_t launch_sample_fp64(const SrcDev& src, int ncols, const double* R, long long ldr,
-                               double* Sr, double* Sc, long long lds, cudaStream_t st, const int* only_if) {
+                               double* Sr, double* Sc, long long lds, cudaStream_t st, const XsTiles* tr,
+                               const XsTiles* tc) {
   if (src.kind < HSS_SRC_DENSE || src.kind > HSS_SRC_LAPLACE) return cudaErrorInvalidValue;   // no entries on the device
   if (src.n <= 0 || ncols <= 0) return cudaSuccess;
   dim3 grid((src.n + BM - 1) / BM, (ncols + BN - 1) / BN);
-  if (Sr) k_sample_fp64<false><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sr, lds, only_if);
-  if (Sc) k_sample_fp64<true><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sc, lds, only_if);
+  if (tr && tc) {
+    if (Sr) k_sample_fp64<false, true><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sr, lds, *tr);
+    if (Sc) k_sample_fp64<true, true><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sc, lds, *tc);
+    return cudaGetLastError();
+  }
+  const XsTiles all = {};
+  if (Sr) k_sample_fp64<false, false><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sr, lds, all);
+  if (Sc) k_sample_fp64<true, false><<<grid, 256, 0, st>>>(src, ncols, R, ldr, Sc, lds, all);
   return cudaGetLastError();
 }
 
