@@ -89,13 +89,14 @@ struct GemmJob {
   unsigned* cnt;
   double* dup;
   int nseg;
-  // what every output tile still needs (XS_FMA, XS_PART; zeroed by the caller),
+  // what every output tile still needs (XS_FMA, XS_PART; XS_WAIT: a wait of one
+  // of its CTAs ran out; zeroed by the caller),
   // and with XS_PART the elements the digits do not settle: 64 bits a row, 128
   // rows a tile
   unsigned* state;
   unsigned* mask;
 };
-enum : unsigned { XS_FMA = 1u, XS_PART = 4u };
+enum : unsigned { XS_FMA = 1u, XS_WAIT = 2u, XS_PART = 4u };
 // The tile states of a sampling call whose rows were cut into chunks of `chunk`
 // row blocks: tile (row block, column tile) at (rb / chunk) stride +
 // (rb % chunk) ncb + column tile.
@@ -281,7 +282,8 @@ cudaError_t launch_xs_check(const GemmJob* jobs_dev, const int* prefix_dev, int 
                             cudaStream_t st);
 // XS_FMA tiles and the marked elements of XS_PART tiles are computed by FP64 FMAs
 // in the same launch, or left out (leave: for the sampling, whose A has no
-// operand view, and whose FP64 kernel fills them in).
+// operand view, and whose FP64 kernel fills them in), as is a tile whose waits
+// ran out (*err records the first).
 cudaError_t launch_xs_mm(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, bool leave, int* err,
                          cudaStream_t st);
 // The sampling operand A - D^(L) (trans 0) or its transpose (1), rows

@@ -63,6 +63,10 @@
 // FP16 product that stops as soon as all elements of its tile have reached it
 // (for even data after the first 32 of K); elements that never do are computed
 // with FP64 FMAs, or, if they are more than one in eight, the whole tile.
+//
+// A wait that runs out (2 s) loses no result: the tile's last CTA, once its own
+// copies and products are over, computes it with FP64 FMAs.  Calls that return
+// a status after their work also report the wait (err).
 #include <cuda_fp16.h>
 #include <stdint.h>
 
@@ -544,7 +548,7 @@ __device__ __forceinline__ void store_tile(const GemmJob& jb, const double* sm, 
 // threads, RX x CY outputs each, K staged 16 at a time, every output one chain
 // over K whatever NR.
 template <int RX, int CY>
-__device__ void fp64_rows(const GemmJob& jb, double* sm, int i0, int j0, int t) {
+__device__ void fp64_rows(const GemmJob& jb, double* sm, int i0, int j0, int t, const unsigned* mask) {
   constexpr int TX = XS_TN / CY, NR = XW * 32 / TX * RX;
   double* stage = sm + XS_TM * XLD;
   double (*As)[NR + 2] = (double (*)[NR + 2])stage;
@@ -584,7 +588,7 @@ __device__ void fp64_rows(const GemmJob& jb, double* sm, int i0, int j0, int t) 
 #pragma unroll
     for (int y = 0; y < CY; ++y) sm[(ty * RX + x) * XLD + tx * CY + y] = jb.alpha * acc[x][y];
   bar_drain();
-  store_tile<NR>(jb, sm, i0, j0, t);
+  store_tile<NR>(jb, sm, i0, j0, t, mask);
 }
 
 // Such a tile is shared by its CTAs by rows: those of its K segments, and
@@ -594,14 +598,16 @@ __device__ void fp64_rows(const GemmJob& jb, double* sm, int i0, int j0, int t) 
 // strategy on the surface kernel (n = 4001), where the elements of one
 // column spread over more than 2^10, took 300 to 1500 us a product on 12 to 48
 // CTAs: 21.1 ms of 77 in all, 6.6 with the rows shared.
-__device__ void fp64_share(const GemmJob& jb, double* sm, int i0, int j0, int part, int parts, int t) {
+// (mask: see store_tile; with one part only)
+__device__ __noinline__ void fp64_share(const GemmJob& jb, double* sm, int i0, int j0, int part, int parts, int t,
+                                        const unsigned* mask = nullptr) {
   const int ns = parts >= 8 ? 8 : (parts >= 4 ? 4 : (parts >= 2 ? 2 : 1));
   const int r0 = i0 + part * (XS_TM / ns);
   if (part >= ns || r0 >= jb.M) return;
-  if (ns == 8) fp64_rows<1, 2>(jb, sm, r0, j0, t);
-  else if (ns == 4) fp64_rows<1, 4>(jb, sm, r0, j0, t);
-  else if (ns == 2) fp64_rows<2, 4>(jb, sm, r0, j0, t);
-  else fp64_rows<4, 4>(jb, sm, r0, j0, t);
+  if (ns == 8) fp64_rows<1, 2>(jb, sm, r0, j0, t, nullptr);
+  else if (ns == 4) fp64_rows<1, 4>(jb, sm, r0, j0, t, nullptr);
+  else if (ns == 2) fp64_rows<2, 4>(jb, sm, r0, j0, t, nullptr);
+  else fp64_rows<4, 4>(jb, sm, r0, j0, t, mask);
 }
 
 // The marked elements of every nseg-th row of the tile by FP64 FMAs: a warp an
@@ -630,20 +636,22 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
                                           int nunits, int leave, int* err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ GemmJob sj;
-  __shared__ int s_last;
+  __shared__ int s_last, s_fail, s_redo;
   uint64_t* full = (uint64_t*)(smem + XNS * XSTAGE);
   uint64_t* empty = full + XNS;
   uint64_t* tfull = empty + XNS;    // one per issuing warp
   uint64_t* tempty = tfull + XMW;
-  uint32_t* tmem_slot = (uint32_t*)(tempty + XMW);
+  uint64_t* idle = tempty + XMW;    // one per issuing warp: its last product is done
+  uint32_t* tmem_slot = (uint32_t*)(idle + XMW);
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   // CTAs past the units are helpers of unit blockIdx.x % nunits
   const int share = blockIdx.x / nunits, shares = gridDim.x / nunits, unit = blockIdx.x % nunits;
   const int ji = find_job(prefix, njobs, unit);
   if (tid == 0) {
     sj = jobs[ji];
+    s_fail = s_redo = 0;
     for (int s = 0; s < XNS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], XMW); }
-    for (int s = 0; s < XMW; ++s) { mbar_init(&tfull[s], 1); mbar_init(&tempty[s], XW); }
+    for (int s = 0; s < XMW; ++s) { mbar_init(&tfull[s], 1); mbar_init(&tempty[s], XW); mbar_init(&idle[s], 1); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -674,7 +682,8 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
     if (lane == 0) {
       const uint8_t* gA = sj.pa + ((size_t)ti * sj.nkt + kt0) * (XD * (size_t)XA);
       const uint8_t* gB = sj.pb + ((size_t)tj * sj.nkt + kt0) * (XD * (size_t)XB);
-      for (int it = 0; it < nk; ++it) {
+      int it = 0;
+      for (; it < nk; ++it) {
         const int st = it % XNS;
         if (!mbar_wait(&empty[st], ((uint32_t)(it / XNS) & 1u) ^ 1u, err, 31)) break;
         uint8_t* sp = smem + st * XSTAGE;
@@ -682,6 +691,8 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
         bulk_g2s(sp, gA + (size_t)it * (XD * XA), XD * XA, &full[st]);
         bulk_g2s(sp + XD * XA, gB + (size_t)it * (XD * XB), XD * XB, &full[st]);
       }
+      // (no copy is under way when this CTA goes on, whatever the others gave up)
+      for (int c = max(0, it - XNS); c < it; ++c) mbar_wait(&full[c % XNS], (uint32_t)(c / XNS) & 1u, err, 35);
     }
   } else if (warp <= XMW) {
     const uint32_t id = idesc(0u, (uint32_t)XS_TN);   // FP16 operands
@@ -689,6 +700,9 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
     if (warp == 1) issue_weights<0, 7, 3>(smem, full, empty, tfull, tempty, tmem, id, nk, one, err);
     else if (warp == 2) issue_weights<1, 6, 4>(smem, full, empty, tfull, tempty, tmem, id, nk, one, err);
     else issue_weights<2, 5, 2, 1, 0>(smem, full, empty, tfull, tempty, tmem, id, nk, one, err);
+    if (one) mma_commit(&idle[warp - 1]);
+    __syncwarp();
+    mbar_wait_warp(&idle[warp - 1], 0u, err, 36);
   } else {
     const int q = warp % 4, h = (warp - 1 - XMW) / 4, t512 = tid - (1 + XMW) * 32;
     unsigned long long hi[XNH], lo[XNH];
@@ -702,11 +716,21 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
       if (ok && chain_end(1, it, nk)) ok = drain_weights<1, 6, 4>(tfull, tempty, c1++, ta, lane, hi, lo, err);
       if (ok && chain_end(2, it, nk)) ok = drain_weights<2, 5, 2, 1, 0>(tfull, tempty, c2++, ta, lane, hi, lo, err);
     }
+#ifdef HSS_TEST_LOST_WAIT   // tests: as if the waits of every other tile's last segment had run out
+    if ((t & 1) && seg == nseg - 1) {
+      ok = false;
+      if (lane == 0) atomicCAS(err, 0, 99);
+    }
+#endif
     // the offset of the raw values of weights 0 .. 2, once per chain
     const unsigned long long bias = (unsigned long long)MAGIC * 0x01010100ull * (unsigned long long)c2;
 #pragma unroll
     for (int x = 0; x < XNH; ++x) hi[x] -= bias;
-    bool last = ok;
+    if (!ok && lane == 0) {
+      s_fail = 1;
+      atomicOr(sj.state + t, XS_WAIT);   // (for the tile's last CTA)
+    }
+    bool last = true;
     if (nseg > 1) {
       // K is split: exact integer sums in global memory, the last CTA to
       // arrive writes the tile
@@ -720,9 +744,12 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
       }
       __threadfence();
       bar_drain();
-      if (t512 == 0) s_last = atomicAdd(sj.cnt + t, 1u) == (unsigned)(nseg - 1) ? 1 : 0;
+      if (t512 == 0) {
+        s_last = atomicAdd(sj.cnt + t, 1u) == (unsigned)(nseg - 1) ? 1 : 0;
+        if (s_last && (atomicOr(sj.state + t, 0u) & XS_WAIT)) s_fail = 1;
+      }
       bar_drain();
-      last = ok && s_last != 0;
+      last = s_last != 0;
       if (last) {
         __threadfence();
 #pragma unroll
@@ -732,12 +759,8 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
         }
       }
     }
-    // a wait that gave up anywhere in the call: the result is NaN, not a
-    // partial sum (callers that read err report it)
-    const bool failed = !ok || *(volatile int*)err != 0;
     const int il = 32 * q + lane, i = i0 + il;
-    if (failed) last = nseg == 1 || last || !ok;
-    if (last) {
+    if (last && ok) {
       const int eA = scale_exp(i < sj.M ? sj.ea[i] : 0u);
       const bool neg = sj.alpha == -1.0;
       const double alpha = neg ? 1.0 : sj.alpha;
@@ -746,14 +769,14 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
         const int jl = h * XNH + x, jj = j0 + jl;
         const int eB = scale_exp(jj < sj.N ? sj.eb[jj] : 0u);
         // E_a + E_b - 70 with E = e - 1021
-        double v = fixed_value((long long)hi[x], (long long)lo[x], eA + eB - 2042 - 70, neg);
-        if (failed) v = __longlong_as_double(0x7FF8000000000000ll);
+        const double v = fixed_value((long long)hi[x], (long long)lo[x], eA + eB - 2042 - 70, neg);
         tile_sm[il * XLD + jl] = alpha == 1.0 ? v : alpha * v;
       }
     }
-    bar_drain();   // (every drain warp is here: all products and copies are done)
+    bar_drain();   // (every drain warp is here: unless one gave up, all products and copies are done)
     const unsigned* mask = state & XS_PART ? sj.mask + (size_t)t * (2 * XS_TM) : nullptr;
-    if (last) store_tile(sj, tile_sm, i0, j0, t512, mask);
+    if (last && !s_fail) store_tile(sj, tile_sm, i0, j0, t512, mask);
+    else if (last && t512 == 0) s_redo = 1;
     if (mask && !leave) fix_rows(sj, mask, i0, j0, seg, warp - 1 - XMW, lane);
   }
   tc_fence_before();
@@ -761,6 +784,13 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  }
+  if (s_redo && warp > XMW) {
+    if (leave) {
+      if (lane == 0) atomicOr(sj.state + t, XS_FMA);
+    } else {
+      fp64_share(sj, tile_sm, i0, j0, 0, 1, tid - (1 + XMW) * 32, state & XS_PART ? sj.mask + (size_t)t * (2 * XS_TM) : nullptr);
+    }
   }
 }
 
@@ -847,7 +877,7 @@ __global__ void __launch_bounds__(256, 5) k_xs_check(const GemmJob* __restrict__
   const int row = 32 * (warp % 4) + lane, h = warp / 4;   // a thread's row and half of the columns
   const bool row_free = i0 + row >= sj.M || sj.ea[i0 + row] == 0u;
   const unsigned col_free = s_free[h];
-  unsigned fail = 0u;
+  unsigned fail = 0u, rounds = 0u;   // (rounds: products waited for)
   bool ok = true;
   int more = !bad;
   for (int it = 0, done = 0; done < nkt && more; ++it) {
@@ -896,6 +926,7 @@ __global__ void __launch_bounds__(256, 5) k_xs_check(const GemmJob* __restrict__
     if (__syncthreads_or(!ok)) { ok = false; break; }
     more = __syncthreads_or(fail != 0u);
     done += nk;
+    ++rounds;
   }
   if (more && ok) {
     atomicAdd(&s_cnt, (unsigned)__popc(fail));
@@ -904,6 +935,7 @@ __global__ void __launch_bounds__(256, 5) k_xs_check(const GemmJob* __restrict__
   __syncthreads();
   if (tid == 0 && (bad || !ok || more)) sj.state[t] = !bad && ok && s_cnt <= CK_MOST ? XS_PART : XS_FMA;
   if (warp == 1) {
+    if (!ok) mbar_wait_warp(&bar, rounds & 1u, err, 38);   // (the products under way)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)XS_TN) : "memory");
   }
@@ -942,7 +974,7 @@ cudaError_t launch_xs_check(const GemmJob* jobs_dev, const int* prefix_dev, int 
 cudaError_t launch_xs_mm(const GemmJob* jobs_dev, const int* prefix_dev, int njobs, int nunits, bool leave, int* err,
                          cudaStream_t st) {
   if (nunits <= 0) return cudaSuccess;
-  const size_t sm = (size_t)XNS * XSTAGE + 8 * (2 * XNS + 2 * XMW) + 16;
+  const size_t sm = (size_t)XNS * XSTAGE + 8 * (2 * XNS + 3 * XMW) + 16;
   cudaError_t e = cudaFuncSetAttribute(k_xs_mm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   // helpers where the units leave SMs idle
