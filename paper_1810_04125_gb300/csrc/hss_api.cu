@@ -457,7 +457,8 @@ struct DevBuf {
     }
     p = nullptr;
     cap = 0;
-    const size_t sz = std::max(bytes + bytes / 2, size_t(1) << 20);
+    // (room to grow, up to 64 MB of it: digits take gigabytes)
+    const size_t sz = std::max(bytes + std::min(bytes / 2, size_t(64) << 20), size_t(1) << 20);
     cudaError_t e = dmalloc_async((void**)&p, sz, st);
     if (e != cudaSuccess) return e;
     cap = sz;
@@ -733,8 +734,10 @@ int xs_seg_ktiles(const std::vector<std::pair<long long, int>>& tiles) {
   return best;
 }
 
-// One launch set (maxima, digits, check, product) over the jobs.
-hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs) {
+// One launch set (maxima, digits, check, product) over the jobs; without memory
+// for their digits they are left to the FP64 tile kernel (rest), which needs
+// none.
+hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs, std::vector<GemmJob>& rest) {
   const int nj = (int)jobs.size();
   std::vector<std::pair<long long, int>> tl;
   for (const GemmJob& j : jobs)
@@ -765,8 +768,11 @@ hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs) {
     pc[i + 1] = pc[i] + (int)(nrb * ncb);
   }
   const size_t zb = Scratch::rnd(sizeof(unsigned) * nz) + sizeof(unsigned long long) * nws;
-  CK(c.xz.ensure(zb, c.st));
-  CK(c.xp.ensure(np, c.st));
+  if (c.xz.ensure(zb, c.st) != cudaSuccess || c.xp.ensure(np, c.st) != cudaSuccess) {
+    cudaGetLastError();
+    rest.insert(rest.end(), jobs.begin(), jobs.end());
+    return HSS_OK;
+  }
   unsigned* z = (unsigned*)c.xz.p;
   for (int i = 0; i < nj; ++i) {
     GemmJob& j = jobs[i];
@@ -837,7 +843,7 @@ hss_status run_gemms(Ctx& c, const std::vector<GemmJob>& all_jobs, const char* t
           continue;
         }
         if (bytes + xs_job_bytes(j) > kXsCap) {
-          CKS(xs_launch(c, std::move(xs)));
+          CKS(xs_launch(c, std::move(xs), rest));
           xs.clear();
           bytes = 0;
         }
@@ -846,7 +852,7 @@ hss_status run_gemms(Ctx& c, const std::vector<GemmJob>& all_jobs, const char* t
         flop += 2.0 * j.M * j.N * j.K;
       }
       const size_t nxs = xs.size();
-      if (!xs.empty()) CKS(xs_launch(c, std::move(xs)));
+      if (!xs.empty()) CKS(xs_launch(c, std::move(xs), rest));
       if (c.trace) {
         CK(cudaEventRecord(c.trace_ev[1], c.st));
         CK(cudaEventSynchronize(c.trace_ev[1]));

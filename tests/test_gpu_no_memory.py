@@ -1,0 +1,40 @@
+"""What needs no memory of its own does not fail for want of it: the digits of
+the exact-split products are used where they can be allocated."""
+import pytest
+
+import fake_alloc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+
+
+WIDE_PRODUCT = r"""
+n = 1500
+P = w.uniform_points(n, 3, seed=2)
+P = P[hss.hss_rcb_order(P, 100)]
+A = w.gaussian_kernel(P, 1.0, 0.5).to_dense()
+H = hss.hss_compress(gu.device_source(w.dense_source(A)), hss.make_opts(100, 1e-9, 1e-12, 64, 64, n, hss.HSS_DOUBLING))
+X = gu.col_major(np.random.default_rng(1).standard_normal((n, 1600)))
+for tr in (False, True):
+    Y, Z = (torch.empty((1600, n), dtype=torch.float64, device=gu.dev()).t() for _ in range(2))
+    hss.hss_matvec(H, X, Y, transpose=tr)
+    before = fake.fake_refused()
+    fake.fake_largest(1 << 20, 1)   # the node vectors' buffer, but no digits
+    hss.hss_matvec(H, X, Z, transpose=tr)
+    torch.cuda.synchronize()
+    fake.fake_largest(-1, 0)
+    assert fake.fake_refused() > before
+    d = (Y - Z).abs().cpu().numpy()
+    # the same sums of at most n terms in FP64, over the levels
+    assert np.all(d <= 1e-12 * (np.abs(A).sum(axis=1).max() * np.abs(X.cpu().numpy()).max())), d.max()
+"""
+
+
+def test_wide_product_without_digits(tmp_path):
+    fake_alloc.run(WIDE_PRODUCT, tmp_path)
