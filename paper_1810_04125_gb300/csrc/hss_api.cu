@@ -1214,6 +1214,26 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
   return HSS_OK;
 }
 
+// The FP64 sampling, in slabs of columns whose digits take at most kXsCap bytes
+// (and those of A as much again).  A slab that xs_sample leaves takes the FP64
+// kernel.
+hss_status sample_plain(Ctx& c, const SrcDev& s, int w, const double* R, long long ldr, double* Sr, double* Sc,
+                        long long lds, XsKeep* keep, int* err) {
+  const size_t col_tile = (size_t)((s.n + XS_BK - 1) / XS_BK) * xs_tile_bytes(1);
+  const int slab = XS_TN * (int)std::max<size_t>(1, std::min<size_t>(kXsCap / col_tile, (size_t)w / XS_TN + 1));
+  for (int c0 = 0; c0 < w; c0 += slab) {
+    const int wc = std::min(slab, w - c0);
+    const double* Rc = R + (long long)c0 * ldr;
+    double *Src = Sr ? Sr + c0 : nullptr, *Scc = Sc ? Sc + c0 : nullptr;
+    bool done = false;
+    CKS(xs_sample(c, s, wc, Rc, ldr, Src, Scc, lds, keep, err, &done));
+    if (done) continue;
+    CK(launch_sample_fp64(s, wc, Rc, ldr, Src, Scc, lds, c.st));
+    c.launches += (Sr ? 1 : 0) + (Sc ? 1 : 0);
+  }
+  return HSS_OK;
+}
+
 // Storage for the digits of a generated source over a whole compression
 // (made at its first sampling pass): up to kXsKeep bytes for all matrices of
 // the call; NULL: not kept, made again by every pass.
@@ -1294,12 +1314,7 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
   } else if (H->o.precision == HSS_PREC_FP64) {
     CK(c.timer.mark(PH_SAMPLE, st));
     double* Sc = H->sym ? nullptr : H->Sg_c + c0;
-    bool xs = false;
-    CKS(xs_sample(c, s, w, Rc, n, H->Sg_r + c0, Sc, H->dmax, xs_keep(c, H), c.d_flag + 5, &xs));
-    if (!xs) {
-      CK(launch_sample_fp64(s, w, Rc, n, H->Sg_r + c0, Sc, H->dmax, st));
-      c.launches += norient;
-    }
+    CKS(sample_plain(c, s, w, Rc, n, H->Sg_r + c0, Sc, H->dmax, xs_keep(c, H), c.d_flag + 5));
     c.sample_launches += norient;
     H->st.sample_launches += norient;
   } else if (use_packed(H)) {
@@ -3418,10 +3433,7 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   SrcDev s = make_src(*A, d_lid);
   if (precision == HSS_PREC_FP64) {
     Ctx c(st);
-    bool xs = false;
-    hss_status e = xs_sample(c, s, ncols, R, ldr, Sr, Sc, lds, nullptr, nullptr, &xs);
-    if (e == HSS_OK && !xs && launch_sample_fp64(s, ncols, R, ldr, Sr, Sc, lds, st) != cudaSuccess)
-      e = fail(HSS_ERR_CUDA, "FP64 sampling launch failed");
+    const hss_status e = sample_plain(c, s, ncols, R, ldr, Sr, Sc, lds, nullptr, nullptr);
     cudaFreeAsync(d_lid, st);
     return e;
   }

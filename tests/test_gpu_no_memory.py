@@ -38,3 +38,24 @@ for tr in (False, True):
 
 def test_wide_product_without_digits(tmp_path):
     fake_alloc.run(WIDE_PRODUCT, tmp_path)
+
+
+MANY_COLUMNS = r"""
+n, nc = 4096, 70000   # digits of R: 4.6 GB
+src = gu.device_source(w.toeplitz_cos(n))
+R = torch.randn((nc, n), dtype=torch.float64, device=gu.dev(), generator=torch.Generator(device=gu.dev()).manual_seed(1)).t()
+S = [torch.full((n, nc), float("nan"), dtype=torch.float64, device=gu.dev()) for _ in range(2)]
+T = [torch.empty((n, 100), dtype=torch.float64, device=gu.dev()) for _ in range(2)]
+held = fake.fake_held()
+fake.fake_peak(1)
+hss.hss_sample_offdiag(src, 128, 0, R, *S)
+torch.cuda.synchronize()
+assert fake.fake_peak(1) - held < 5e9, fake.fake_peak(0)   # two caps of 2^31 bytes, and bookkeeping
+for c in (0, 32700, 65400, nc - 100):   # slabs of 32768
+    hss.hss_sample_offdiag(src, 128, 0, R[:, c:c + 100], *T)
+    assert all(torch.equal(s[:, c:c + 100], t) for s, t in zip(S, T))
+"""
+
+
+def test_digits_of_many_columns(tmp_path):
+    fake_alloc.run(MANY_COLUMNS, tmp_path)
