@@ -151,12 +151,25 @@ cudaError_t lib_pool(cudaMemPool_t* out) {
   return cudaSuccess;
 }
 
+// Gives back what the compression that runs on this thread holds for speed
+// alone (digits of operands, the pool's idle memory) when an allocation fails;
+// true: worth another try.
+bool give_back_spare();
+
 template <class T>
 cudaError_t dmalloc_async(T** p, size_t bytes, cudaStream_t st) {
   cudaMemPool_t pool = nullptr;
   cudaError_t e = lib_pool(&pool);
   if (e != cudaSuccess) return e;
-  return cudaMallocFromPoolAsync((void**)p, bytes, pool, st);
+  e = cudaMallocFromPoolAsync((void**)p, bytes, pool, st);
+  if (e != cudaSuccess && give_back_spare()) e = cudaMallocFromPoolAsync((void**)p, bytes, pool, st);
+  return e;
+}
+
+cudaError_t dmalloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess && give_back_spare()) e = cudaMalloc(p, bytes);
+  return e;
 }
 
 // Pinned read-back buffers of the usual size outlive their call, up to
@@ -219,7 +232,7 @@ struct Arena {
             break;
           }
       }
-      if (!p && cudaMalloc(&p, sz) != cudaSuccess) return nullptr;
+      if (!p && dmalloc(&p, sz) != cudaSuccess) return nullptr;
       chunks.push_back({p, sz});
       cur = (char*)p;
       left = sz;
@@ -271,7 +284,7 @@ struct Scratch {
     // from the pool up to kScratchPool, so that the pool holds little more for
     // it; larger ones are given back to the system at the end of the call
     pooled = sz <= kScratchPool;
-    e = pooled ? dmalloc_async(&base, sz, st) : cudaMalloc(&base, sz);
+    e = pooled ? dmalloc_async(&base, sz, st) : dmalloc((void**)&base, sz);
     if (e != cudaSuccess) {
       base = nullptr;
       return e;
@@ -494,6 +507,9 @@ struct Ctx {
   PhaseTimer timer;
   long long launches = 0, sample_launches = 0, bytes_h2d = 0, bytes_d2h = 0;
   size_t xs_kept = 0;      // bytes of digits kept by the matrices of the call (XsKeep)
+  std::vector<hss_matrix_s*> xs_keepers;
+  bool xs_keep_none = false;   // they were given back: made again by every pass from then on
+  bool xs_busy = false;    // pointers into xz, xp or kept digits are in use
   bool trace = false;      // HSS_TRACE=1: one stderr line per launch of the batched phases
   cudaEvent_t trace_ev[2] = {nullptr, nullptr};
   int qrcp_cap = -1, qrcp_cap_d = -1, qrcp_cap_w = -1, qrcp_nsm = 0, qrcp_per = 0;
@@ -549,6 +565,38 @@ struct Ctx {
     return HSS_OK;
   }
 };
+
+// The compression that runs on this thread (a user's callback may start another).
+thread_local Ctx* t_ctx = nullptr;
+struct CtxScope {
+  Ctx* before;
+  explicit CtxScope(Ctx* c) : before(t_ctx) { t_ctx = c; }
+  ~CtxScope() { t_ctx = before; }
+};
+struct XsBusy {
+  Ctx& c;
+  bool before;
+  explicit XsBusy(Ctx& x) : c(x), before(x.xs_busy) { c.xs_busy = true; }
+  ~XsBusy() { c.xs_busy = before; }
+};
+
+bool give_back_spare() {
+  cudaGetLastError();
+  Ctx* c = t_ctx;
+  if (!c || c->xs_busy) return false;
+  for (hss_matrix_s* H : c->xs_keepers) {
+    if (H->xs.pa[0]) cudaFreeAsync(H->xs.pa[0], c->st);
+    H->xs = XsKeep();
+    c->xs_keep_none = true;
+  }
+  c->xs_keepers.clear();
+  c->xs_kept = 0;
+  c->xz.release(c->st);
+  c->xp.release(c->st);
+  cudaMemPool_t pool = nullptr;
+  return cudaStreamSynchronize(c->st) == cudaSuccess && lib_pool(&pool) == cudaSuccess &&
+         cudaMemPoolTrimTo(pool, 0) == cudaSuccess;
+}
 
 SrcDev make_src(const hss_source& s, const int* leaf_id) {
   SrcDev d;
@@ -768,8 +816,12 @@ hss_status xs_launch(Ctx& c, std::vector<GemmJob> jobs, std::vector<GemmJob>& re
     pc[i + 1] = pc[i] + (int)(nrb * ncb);
   }
   const size_t zb = Scratch::rnd(sizeof(unsigned) * nz) + sizeof(unsigned long long) * nws;
+  XsBusy busy(c);
+  CK(c.jobs.ensure(nj * (sizeof(GemmJob) + 4 * sizeof(int)) + 4096, c.st));   // (no allocation while the digits are held)
   if (c.xz.ensure(zb, c.st) != cudaSuccess || c.xp.ensure(np, c.st) != cudaSuccess) {
     cudaGetLastError();
+    c.xz.release(c.st);
+    c.xp.release(c.st);
     rest.insert(rest.end(), jobs.begin(), jobs.end());
     return HSS_OK;
   }
@@ -1089,6 +1141,8 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
   *done = false;
   const int n = s.n;
   if (n < 192 || w <= 0 || n > (1 << 22) || (n + 127) / 128 > 65535) return HSS_OK;
+  XsBusy busy(c);
+  if (keep && !keep->pa[0]) keep = nullptr;   // (given back)
   cudaStream_t st = c.st;
   const bool sym = symmetric_source(s);
   struct Orient { int trans; double* S; double* dup; };
@@ -1120,9 +1174,12 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
   const size_t zw = Scratch::rnd(sizeof(unsigned) * nz);
   const size_t zb = zw + sizeof(unsigned long long) * per_ws * no;
   const size_t bB = (size_t)ncb * nkt * xs_tile_bytes(1) + per_cnt * no * nchunk * kXsMask;
+  CK(c.jobs.ensure((1 + (size_t)no * nchunk) * (sizeof(GemmJob) + 4 * sizeof(int)) + 16 * (size_t)nchunk + 4096, st));
   if (c.xz.ensure(zb, st) != cudaSuccess ||
       c.xp.ensure(bB + (keep ? 0 : chunk * row_bytes * no), st) != cudaSuccess) {
     cudaGetLastError();   // no memory for the digits
+    c.xz.release(st);
+    c.xp.release(st);
     return HSS_OK;
   }
   unsigned* z = (unsigned*)c.xz.p;
@@ -1242,13 +1299,15 @@ XsKeep* xs_keep(Ctx& c, hss_matrix_s* H) {
   if (H->xs.pa[0]) return &H->xs;
   const size_t one = (size_t)((H->n + XS_TM - 1) / XS_TM) * ((H->n + XS_BK - 1) / XS_BK) * xs_tile_bytes(0);
   const size_t need = one + Scratch::rnd(sizeof(unsigned) * 2 * (size_t)H->n);
-  if (H->n < 192 || c.xs_kept + need > kXsKeep) return nullptr;
+  if (H->n < 192 || c.xs_keep_none || c.xs_kept + need > kXsKeep) return nullptr;
+  XsBusy busy(c);   // (not at the cost of what others keep)
   char* p = nullptr;
   if (dmalloc_async(&p, need, c.st) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
   c.xs_kept += need;
+  c.xs_keepers.push_back(H);
   H->xs.pa[0] = H->xs.pa[1] = (unsigned char*)p;   // a point kernel's two orientations are one
   H->xs.ea = (unsigned*)(p + one);
   return &H->xs;
@@ -2190,6 +2249,7 @@ hss_status keep_dense_blocks(Ctx& c, hss_matrix_s* H) {
   for (auto& t : H->nodes)
     if (!t.leaf && t.state != HSS_COMPRESSED)
       need += 2.0 * 8.0 * (double)H->nodes[t.ch[0]].size * (double)H->nodes[t.ch[1]].size;
+  give_back_spare();   // (free memory without what the samples' digits took)
   size_t fr = 0, tot = 0;
   CK(cudaMemGetInfo(&fr, &tot));
   if (need > 0.5 * (double)fr) return HSS_OK;
@@ -2333,6 +2393,7 @@ hss_status find_symmetric(Ctx& c, const std::vector<const hss_source*>& A, const
 // flags per round of sampling.
 hss_status compress_all(Ctx& c, const std::vector<const hss_source*>& A, const std::vector<const hss_opts*>& O,
                         std::vector<hss_matrix_s*>& Hs) {
+  CtxScope scope(&c);
   CKS(c.flags((int)Hs.size()));
   CK(c.timer.mark(PH_OTHER, c.st));
   ExtractSet leafD;
@@ -2578,7 +2639,7 @@ hss_status hss_compress_batched(const hss_source* A, const hss_opts* opts, int c
   }
   cudaStream_t st = (cudaStream_t)stream;
   // Groups of matrices compressed in lockstep, each group's estimated device
-  // memory (samples, R, bases, packed tensor-core operand) within 60 % of
+  // memory (samples, R, bases, packed tensor-core operand, digits) within 60 % of
   // the free memory; largest first.
   std::vector<int> order(count);
   for (int i = 0; i < count; ++i) order[i] = i;
@@ -2589,7 +2650,17 @@ hss_status hss_compress_batched(const hss_source* A, const hss_opts* opts, int c
     if (opts[i].strategy == HSS_INCREMENTING) b += 8.0 * n * dm * 2.0;   // bases Q
     if (opts[i].precision != HSS_PREC_FP64 && A[i].kind == HSS_SRC_DENSE)
       b += (double)packed_a_bytes(A[i].n, opts[i].precision, 2);
+    // digits of a generated source's entries, kept over the compression
+    if (opts[i].precision == HSS_PREC_FP64 && (A[i].kind == HSS_SRC_GAUSS || A[i].kind == HSS_SRC_LAPLACE) &&
+        16.0 * n * n <= (double)kXsKeep)
+      b += 16.0 * n * n;
     return b;
+  };
+  // digits of the operands of one launch, which the matrices of a group share
+  auto workspace = [&](int i) {
+    const double n = A[i].n, dm = std::min(opts[i].d_max, A[i].n);
+    if (opts[i].precision != HSS_PREC_FP64) return 0.0;
+    return std::min(32.0 * n * n, (double)kXsCap) + std::min(16.0 * n * dm, (double)kXsCap);
   };
   size_t fr = 0, tot = 0;
   CK(cudaMemGetInfo(&fr, &tot));
@@ -2615,8 +2686,13 @@ hss_status hss_compress_batched(const hss_source* A, const hss_opts* opts, int c
   int at = -1;
   for (size_t g0 = 0; g0 < order.size() && first == HSS_OK;) {
     size_t g1 = g0;
-    double used = 0.0;
-    while (g1 < order.size() && (g1 == g0 || used + footprint(order[g1]) <= budget)) used += footprint(order[g1++]);
+    double used = 0.0, work = 0.0;
+    for (; g1 < order.size(); ++g1) {
+      const double w = std::max(work, workspace(order[g1]));
+      if (g1 > g0 && used + footprint(order[g1]) + w > budget) break;
+      used += footprint(order[g1]);
+      work = w;
+    }
     std::vector<hss_matrix_s*> Hs;
     std::vector<const hss_source*> As;
     std::vector<const hss_opts*> Os;

@@ -59,3 +59,41 @@ for c in (0, 32700, 65400, nc - 100):   # slabs of 32768
 
 def test_digits_of_many_columns(tmp_path):
     fake_alloc.run(MANY_COLUMNS, tmp_path)
+
+
+COMPRESSION = r"""
+import gc
+n, leaf = 4096, 64
+P = w.uniform_points(n, 3, seed=2)
+P = gu.col_major(P[hss.hss_rcb_order(P, leaf)])
+src = hss.points_source(w.SRC_GAUSS, P, 0.5, 1.0)
+X = gu.col_major(np.random.default_rng(1).standard_normal((n, 3)))
+
+def compress():
+    hss.hss_release_cached()
+    gc.collect()
+    H = hss.hss_compress(src, hss.make_opts(leaf, 1e-6, 1e-10, 64, 64, 2048, hss.HSS_DOUBLING))
+    Y = torch.empty((3, n), dtype=torch.float64, device=gu.dev()).t()
+    hss.hss_matvec(H, X, Y)
+    return H.ranks(), Y.cpu().numpy()
+
+compress()
+hss.hss_release_cached()
+held = fake.fake_held()
+fake.fake_peak(1)
+ranks, Y = compress()
+peak = fake.fake_peak(1) - held
+digits = 16 * n * n
+hss.hss_release_cached()
+fake.fake_budget(peak - digits * 8 // 10 - (fake.fake_held() - held))
+before = fake.fake_refused()
+ranks2, Z = compress()
+assert fake.fake_refused() > before
+assert ranks == ranks2
+assert np.linalg.norm(Y - Z) <= 1e-12 * np.linalg.norm(Y), np.linalg.norm(Y - Z) / np.linalg.norm(Y)
+"""
+
+
+def test_compression_gives_its_digits_back(tmp_path):
+    """A compression that fits without the digits it keeps for speed fits."""
+    fake_alloc.run(COMPRESSION, tmp_path)
