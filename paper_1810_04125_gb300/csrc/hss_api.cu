@@ -408,8 +408,8 @@ struct ProdPlan {
   struct Phase { int first, count, tiles; };
   std::vector<Phase> phases[2];
   size_t rows[2] = {0, 0};   // buffer rows of a product
-  double elems = 0.0;        // generator elements read by a product
-  int sets = 0;              // of its phases, those with sums of 8 terms or more
+  double elems[2] = {0.0, 0.0};   // generator elements read by a product
+  int sets[2] = {0, 0};      // of its phases, those with sums of 8 terms or more
 };
 
 struct hss_matrix_s {
@@ -3146,7 +3146,7 @@ const ProdPlan* get_plan(hss_matrix_s* H, cudaStream_t st) {
       P.phases[tr].clear();
       if (tr) second = tasks.size();
       std::vector<ProdTask> q;
-      if (!H->partial) prod_tasks(H, tr != 0, ipr, ipc, q, P.phases[tr], &P.rows[tr], &P.elems, &P.sets);
+      if (!H->partial) prod_tasks(H, tr != 0, ipr, ipc, q, P.phases[tr], &P.rows[tr], &P.elems[tr], &P.sets[tr]);
       tasks.insert(tasks.end(), q.begin(), q.end());
     }
     P.tasks[0] = (const ProdTask*)(base + o_task);
@@ -3203,8 +3203,8 @@ const ProdPlan* get_plan(hss_matrix_s* H, cudaStream_t st) {
 // us against 650, 32 columns 1130 against 679; Gaussian 3-D n = 5003 (19
 // sets): 256 columns 793 us against 1650.
 bool prod_by_tasks(const ProdPlan& P, bool tr, int nrhs) {
-  const double flop = 2.0 * P.elems * nrhs;
-  return nrhs <= 65535 * 8 && 3.0 * P.phases[tr].size() + flop / 0.85e6 <= 60.0 * P.sets + flop / 20e6;
+  const double flop = 2.0 * P.elems[tr] * nrhs;
+  return nrhs <= 65535 * 8 && 3.0 * P.phases[tr].size() + flop / 0.85e6 <= 60.0 * P.sets[tr] + flop / 20e6;
 }
 
 }  // namespace
