@@ -395,12 +395,13 @@ struct XsKeep {
 }  // namespace
 
 // What the products and the entry extraction of a handle read besides its
-// generators, laid out on the device at the first such call and kept (in the
-// handle's arena) until the handle is freed: the nodes with the inverse pivot
+// generators, laid out on the device at the first such call and kept until the
+// handle is freed, in a buffer of just their size: the nodes with the inverse pivot
 // orders, the leaf of every index, and for H X and H^T X the task lists of
 // every phase (first task, count, 16-row tiles of its largest).
 struct ProdPlan {
   bool ready = false;
+  char* mem = nullptr;
   EntryNode* nodes = nullptr;
   int* leaf_of = nullptr;
   int kcap = 1;
@@ -450,6 +451,10 @@ struct hss_matrix_s {
     if (toep_terms) cudaFree(toep_terms);
     if (pts) cudaFree(pts);
     if (xs.pa[0]) cudaFree(xs.pa[0]);
+    if (plan.mem) {   // (from the pool, whose memory cudaFree does not wait for)
+      cudaDeviceSynchronize();
+      cudaFree(plan.mem);
+    }
     arena.release();
   }
 };
@@ -3106,15 +3111,19 @@ void prod_tasks(const hss_matrix_s* H, bool tr, const std::vector<const int*>& i
 
 // The handle's plan, made at the first call that needs it (from any thread;
 // it is complete on the device before the lock is given up, so that calls on
-// other streams may use it at once).  NULL when there is no memory for it, or
-// when it would have to be made during a stream capture.
-const ProdPlan* get_plan(hss_matrix_s* H, cudaStream_t st) {
+// other streams may use it at once).  NULL, and why (a status with its message
+// in g_err), when there is no memory for it, when the handle's pivots are no
+// permutations, or when it would have to be made during a stream capture.
+const ProdPlan* get_plan(hss_matrix_s* H, cudaStream_t st, hss_status* why = nullptr) {
+  hss_status ignored;
+  if (!why) why = &ignored;
   std::lock_guard<std::mutex> lock(H->plan_mu);
   ProdPlan& P = H->plan;
   if (P.ready) return &P;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
+    *why = fail(HSS_ERR_CUDA, "the index tables of the handle cannot be laid out during a stream capture");
     return nullptr;
   }
   const int nn = (int)H->nodes.size(), n = H->n;
@@ -3157,9 +3166,10 @@ const ProdPlan* get_plan(hss_matrix_s* H, cudaStream_t st) {
   ntask = tasks.size();
   const size_t o_inv = o_task + Scratch::rnd(sizeof(ProdTask) * ntask);
   const size_t o_leaf = o_inv + Scratch::rnd(sizeof(int) * std::max<size_t>(ninv, 1));
-  char* base = (char*)H->arena.alloc(o_leaf + sizeof(int) * n);
-  if (!base) {
+  char* base = nullptr;
+  if (dmalloc_async(&base, o_leaf + sizeof(int) * n, st) != cudaSuccess) {
     cudaGetLastError();
+    *why = fail(HSS_ERR_NOMEM, "no device memory for the index tables of the handle");
     return nullptr;
   }
   make(base);
@@ -3181,16 +3191,25 @@ const ProdPlan* get_plan(hss_matrix_s* H, cudaStream_t st) {
     }
   }
   if (ntask) memcpy(host.data() + o_task, tasks.data(), sizeof(ProdTask) * ntask);
-  int herr = 1;
-  if (cudaMemcpyAsync(base, host.data(), o_inv, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemsetAsync(base + o_inv, 0xff, sizeof(int) * std::max<size_t>(ninv, 1), st) != cudaSuccess ||
-      launch_inv_piv((const EntryNode*)(base + o_nodes), nn, (int*)base, st) != cudaSuccess ||
-      launch_leaf_of((const EntryNode*)(base + o_nodes), nn, (int*)(base + o_leaf), st) != cudaSuccess ||
-      cudaMemcpyAsync(&herr, base, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess || herr) {
+  int herr = 0;
+  auto run = [&]() -> hss_status {
+    CK(cudaMemcpyAsync(base, host.data(), o_inv, cudaMemcpyHostToDevice, st));
+    CK(cudaMemsetAsync(base + o_inv, 0xff, sizeof(int) * std::max<size_t>(ninv, 1), st));   // -1: no position
+    CK(launch_inv_piv((const EntryNode*)(base + o_nodes), nn, (int*)base, st));
+    CK(launch_leaf_of((const EntryNode*)(base + o_nodes), nn, (int*)(base + o_leaf), st));
+    CK(cudaMemcpyAsync(&herr, base, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (herr) return fail(HSS_ERR_CUDA, "inconsistent pivots in the handle (code %d)", herr);
+    return HSS_OK;
+  };
+  *why = run();
+  if (*why != HSS_OK) {
     cudaGetLastError();
-    return nullptr;   // (pivots that are no permutation: the general paths report it)
+    cudaStreamSynchronize(st);
+    cudaFreeAsync(base, st);
+    return nullptr;
   }
+  P.mem = base;
   P.nodes = (EntryNode*)(base + o_nodes);
   P.leaf_of = (int*)(base + o_leaf);
   P.ready = true;
@@ -3403,8 +3422,9 @@ hss_status hss_get_entries(hss_matrix H, int nr, const int* I, int nc, const int
   if (!I || !J || !out) return fail(HSS_ERR_ARG, "NULL argument");
   cudaStream_t st = (cudaStream_t)stream;
   const int n = H->n;
-  const ProdPlan* P = get_plan(H, st);
-  if (!P) return fail(HSS_ERR_NOMEM, "the index tables of the handle could not be laid out on the device");
+  hss_status why = HSS_OK;
+  const ProdPlan* P = get_plan(H, st, &why);
+  if (!P) return why;
   const int kcap = P->kcap, lp1 = H->max_level + 1;
   // rows and columns in chunks whose path vectors take at most 512 MB each
   // (and at most 65535 columns: one grid row per column)

@@ -97,3 +97,35 @@ assert np.linalg.norm(Y - Z) <= 1e-12 * np.linalg.norm(Y), np.linalg.norm(Y - Z)
 def test_compression_gives_its_digits_back(tmp_path):
     """A compression that fits without the digits it keeps for speed fits."""
     fake_alloc.run(COMPRESSION, tmp_path)
+
+
+ENTRIES = r"""
+n = 6000   # one leaf: its block fills the handle's last chunk of memory
+A = w.toeplitz_cos(n).to_dense()
+src = gu.device_source(w.dense_source(A))
+H = hss.hss_compress(src, hss.make_opts(n, 1e-6, 1e-10, 16, 16, 16, hss.HSS_DOUBLING))
+I, J = (torch.arange(k, n, 997, device=gu.dev(), dtype=torch.int32) for k in (0, 5))
+out = torch.empty((J.numel(), I.numel()), dtype=torch.float64, device=gu.dev()).t()
+X = gu.col_major(np.eye(n)[:, :3])
+Y = torch.empty((3, n), dtype=torch.float64, device=gu.dev()).t()
+fake.fake_budget(64 << 20)
+hss.hss_get_entries(H, I, J, out)
+hss.hss_matvec(H, X, Y)
+torch.cuda.synchronize()
+assert np.array_equal(out.cpu().numpy(), A[np.ix_(I.cpu().numpy(), J.cpu().numpy())])
+assert np.array_equal(Y.cpu().numpy(), A[:, :3])
+held = fake.fake_held()
+fake.fake_budget(0)
+for call in (lambda: hss.hss_get_entries(G, I, J, out), lambda: hss.hss_matvec(H, X, Y)):
+    G = H
+    try:
+        call()
+    except hss.HSSError as e:
+        assert e.status in (2, 3)
+assert fake.fake_held() == held
+"""
+
+
+def test_tables_of_a_handle(tmp_path):
+    """The first entries of a handle take memory of their own size, not a chunk."""
+    fake_alloc.run(ENTRIES, tmp_path)
