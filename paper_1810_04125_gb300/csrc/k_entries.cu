@@ -76,11 +76,13 @@ constexpr int EW_MAX = 16;
 // Row (CTAs below nr) or column vectors of the nested basis along the path of
 // an index to the root.  A row stores W(level(a)) = u_a(i) B_ab for every
 // ancestor a whose parent is COMPRESSED, a column v_a(j).  Wrow, Vcol:
-// (count x (levels + 1) x kcap) doubles; shared memory 2 kcap doubles and kcap
-// ints.  Bound by the FP64 pipe (sum of k_a k_b + k_a k_p per level) once the
+// (count x (levels + 1) x kcap) doubles; shared memory 2 kcap doubles and, where
+// they fit too (HAVE_SP), kcap ints for the positions, which are read from the
+// tables again otherwise (ranks above 11600).  Bound by the FP64 pipe (sum of k_a k_b + k_a k_p per level) once the
 // sums run along the blocks' contiguous direction: u B with eight columns of B
 // per warp and lanes along u, u U_p with a lane per column.  Rows and columns
 // go in one launch.
+template <bool HAVE_SP>
 __global__ void __launch_bounds__(32 * EW_MAX) k_entry_paths(const EntryNode* __restrict__ nodes,
                                                          const int* __restrict__ leaf_of, int n,
                                                          const int* __restrict__ I, int nr, const int* __restrict__ J,
@@ -124,15 +126,17 @@ __global__ void __launch_bounds__(32 * EW_MAX) k_entry_paths(const EntryNode* __
     // the rows of U_p for the up-step: positions of a's rows in p's pivot order
     const bool top = p.parent < 0;   // a is a child of the root
     const int kp = side ? p.kc : p.kr, mp = side ? p.mc : p.mr;
+    const int* inv = top ? nullptr : (side ? p.ipivc : p.ipivr) + (first ? 0 : (side ? b.kc : b.kr));
+    auto checked = [&](int q) {
+      const int pos = inv[q];
+      return pos < 0 || pos >= mp ? -1 : pos;   // (not a permutation: never from a compression)
+    };
+    auto place = [&](int q) { return HAVE_SP ? sp[q] : checked(q); };
     if (!top) {
-      const int* inv = (side ? p.ipivc : p.ipivr) + (first ? 0 : (side ? b.kc : b.kr));
       for (int q = tid; q < ka; q += 32 * EW) {
-        int pos = inv[q];
-        if (pos < 0 || pos >= mp) {   // not a permutation (never from a compression)
-          atomicCAS(err, 0, 2);
-          pos = -1;
-        }
-        sp[q] = pos;
+        const int pos = checked(q);
+        if (pos < 0) atomicCAS(err, 0, 2);
+        if (HAVE_SP) sp[q] = pos;
       }
       for (int c = tid; c < kp; c += 32 * EW) u2[c] = 0.0;
     }
@@ -172,18 +176,18 @@ __global__ void __launch_bounds__(32 * EW_MAX) k_entry_paths(const EntryNode* __
         double m[8];
 #pragma unroll
         for (int x = 0; x < 8; ++x) {
-          const int pos = q0 + x < ka ? sp[q0 + x] : -1;
+          const int pos = q0 + x < ka ? place(q0 + x) : -1;
           m[x] = pos >= kp && c < kp ? X[c + (long long)(pos - kp) * kp] : 0.0;
         }
 #pragma unroll
         for (int x = 0; x < 8; ++x)
-          if (q0 + x < ka && sp[q0 + x] >= kp) s = __fma_rn(u[q0 + x], m[x], s);
+          if (q0 + x < ka && place(q0 + x) >= kp) s = __fma_rn(u[q0 + x], m[x], s);
       }
       if (c < kp) u2[c] = s;
     }
     __syncthreads();
     for (int q = tid; q < ka; q += 32 * EW)   // the skeleton rows: each position once
-      if (sp[q] >= 0 && sp[q] < kp) u2[sp[q]] += u[q];
+      if (const int pos = place(q); pos >= 0 && pos < kp) u2[pos] += u[q];
     double* tmp = u;
     u = u2;
     u2 = tmp;
@@ -262,10 +266,12 @@ cudaError_t launch_inv_piv(const EntryNode* nodes, int nn, int* err, cudaStream_
 cudaError_t launch_entry_paths(const EntryNode* nodes, const int* leaf_of, int n, const int* I, int nr, const int* J,
                                int nc, double* Wrow, double* Vcol, int kcap, int lp1, int* err, cudaStream_t st) {
   if (nr + nc <= 0) return cudaSuccess;
-  const size_t sm = (sizeof(double) * 2 + sizeof(int)) * (size_t)kcap;
-  cudaError_t e = cudaFuncSetAttribute(k_entry_paths, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const bool have_sp = (sizeof(double) * 2 + sizeof(int)) * (size_t)kcap <= size_t(227) << 10;
+  const size_t sm = (sizeof(double) * 2 + (have_sp ? sizeof(int) : 0)) * (size_t)kcap;
+  auto* f = have_sp ? k_entry_paths<true> : k_entry_paths<false>;
+  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_entry_paths<<<nr + nc, 32 * path_warps(kcap), sm, st>>>(nodes, leaf_of, n, I, nr, J, Wrow, Vcol, kcap, lp1, err);
+  f<<<nr + nc, 32 * path_warps(kcap), sm, st>>>(nodes, leaf_of, n, I, nr, J, Wrow, Vcol, kcap, lp1, err);
   return cudaGetLastError();
 }
 

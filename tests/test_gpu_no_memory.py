@@ -116,8 +116,7 @@ assert np.array_equal(out.cpu().numpy(), A[np.ix_(I.cpu().numpy(), J.cpu().numpy
 assert np.array_equal(Y.cpu().numpy(), A[:, :3])
 held = fake.fake_held()
 fake.fake_budget(0)
-for call in (lambda: hss.hss_get_entries(G, I, J, out), lambda: hss.hss_matvec(H, X, Y)):
-    G = H
+for call in (lambda: hss.hss_get_entries(H, I, J, out), lambda: hss.hss_matvec(H, X, Y)):
     try:
         call()
     except hss.HSSError as e:
