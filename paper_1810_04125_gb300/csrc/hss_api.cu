@@ -1129,7 +1129,11 @@ bool use_packed(hss_matrix_s* H) {
   if (H->src.kind == HSS_SRC_DENSE) return true;
   if (H->pack_decided < 0) {
     size_t fr = 0, tot = 0;
-    const size_t pb = packed_a_bytes(H->n, H->o.precision, H->sym || H->same_samples ? 1 : 2);
+    // (a Toeplitz matrix above the size at which both orientations fit is sampled
+    // out of its 2 n - 1 diagonals, although one orientation may fit: at n =
+    // 100000 that would be 80 GB)
+    const bool one = (H->sym || H->same_samples) && H->src.kind != HSS_SRC_TOEPLITZ;
+    const size_t pb = packed_a_bytes(H->n, H->o.precision, one ? 1 : 2);
     H->pack_decided = (cudaMemGetInfo(&fr, &tot) == cudaSuccess && (double)pb <= 0.4 * (double)fr) ? 1 : 0;
   }
   return H->pack_decided == 1;

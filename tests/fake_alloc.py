@@ -7,7 +7,8 @@ fake_budget(bytes) sets the budget over what is held at that moment (< 0: none),
 fake_largest(bytes, k) the largest single allocation from a memory pool (< 0:
 any) after k more that are larger,
 fake_peak(1) returns the most held since the last such call and starts anew,
-fake_refused() the number of refusals."""
+fake_refused() the number of refusals; fake_free(bytes) what cudaMemGetInfo
+reports as free (< 0: the truth)."""
 import os
 import subprocess
 import sys
@@ -78,6 +79,16 @@ int cudaFreeAsync(void* p, void* st) {
   return f(p, st);
 }
 
+static long long free_bytes = -1;
+int cudaMemGetInfo(size_t* fr, size_t* tot) {
+  static int (*f)(size_t*, size_t*);
+  if (!f) f = dlsym(RTLD_NEXT, "cudaMemGetInfo");
+  int e = f(fr, tot);
+  if (!e && free_bytes >= 0) *fr = (size_t)free_bytes;
+  return e;
+}
+
+void fake_free(long long n) { free_bytes = n; }
 void fake_budget(long long n) {
   pthread_mutex_lock(&mu);
   budget = n < 0 ? -1 : held + n;
@@ -102,7 +113,7 @@ HEAD = r"""
 import ctypes, os, sys
 sys.path[:0] = [{root!r}, {root!r} + "/tests"]
 fake = ctypes.CDLL({shim!r})
-fake.fake_budget.argtypes = [ctypes.c_longlong]
+fake.fake_budget.argtypes = fake.fake_free.argtypes = [ctypes.c_longlong]
 fake.fake_largest.argtypes = [ctypes.c_longlong] * 2
 for f in ("fake_peak", "fake_held", "fake_refused"):
     getattr(fake, f).restype = ctypes.c_longlong

@@ -128,3 +128,24 @@ assert fake.fake_held() == held
 def test_tables_of_a_handle(tmp_path):
     """The first entries of a handle take memory of their own size, not a chunk."""
     fake_alloc.run(ENTRIES, tmp_path)
+
+
+TOEPLITZ = r"""
+n = 4096   # one orientation of the packed terms: 134 MB, both: 268
+src = hss.toeplitz_source(torch.from_numpy(w.toeplitz_cos(n).col).to(gu.dev()))
+opts = hss.make_opts(128, 1e-4, 1e-8, 128, 128, 1024, hss.HSS_DOUBLING, hss.HSS_PREC_TF32X2)
+hss.hss_compress(src, opts)
+bytes_ = []
+for free in (4 << 30, 500 << 20):   # 0.4 of it: room for both, for one
+    hss.hss_release_cached()
+    fake.fake_free(free)
+    st = hss.hss_compress(src, opts).stats()
+    fake.fake_free(-1)
+    bytes_.append(st.bytes_sample - 16.0 * n * st.d_final)
+print(bytes_)
+assert bytes_[0] > 0 and bytes_[1] == 0   # A's own traffic, counted where it is packed
+"""
+
+
+def test_toeplitz_is_not_packed_where_one_orientation_fits(tmp_path):
+    fake_alloc.run(TOEPLITZ, tmp_path)
