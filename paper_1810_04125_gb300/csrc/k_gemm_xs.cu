@@ -319,8 +319,10 @@ __global__ void __launch_bounds__(256) k_xs_src_max(SrcDev src, unsigned* out, u
         if (r2 < best) best = r2;
       }
     if (any) {
-      // the formulas of entry() at the smallest distance
-      const double v = src.kind == HSS_SRC_GAUSS ? exp(-best / (2.0 * src.p0 * src.p0))
+      // the formulas of entry() at the smallest distance; exp is within an ulp but
+      // not promised to be monotone, so the entry at a larger distance may be a
+      // little above it (and in the next binade, for which the digits have no room)
+      const double v = src.kind == HSS_SRC_GAUSS ? exp(-best / (2.0 * src.p0 * src.p0)) * (1.0 + 0x1p-50)
                                                  : 1.0 / (4.0 * 3.141592653589793 * sqrt(best));
       km = nan ? HI_INF : mag_key(v);
     }

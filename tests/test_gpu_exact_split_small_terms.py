@@ -77,6 +77,27 @@ def test_narrow_gaussian_kernel(torch):
         assert np.all(np.abs(s - f.cpu().numpy()) <= bound)
 
 
+def test_gaussian_entries_around_powers_of_two(torch):
+    """Entries within a few ulps of 2^-k, on both sides of it: the scale of a row
+    holds all of them (against the FMA kernel, as above)."""
+    import gpu_util as gu
+    from paper_1810_04125_gb300 import hss
+    m, leaf, nc = 256, 64, 70
+    k = 1 + np.arange(m) % 7
+    x = np.sqrt(2.0 * k * np.log(2.0)) * (1.0 + (np.arange(m) - m // 2) * 2.0 ** -53)
+    P = np.stack([np.concatenate([1e-9 * np.arange(m) * 2.0 ** -30, x]), np.zeros(2 * m)], axis=1)
+    src = w.gaussian_kernel(P, 1.0, 1.0)
+    R = w.gaussian_matrix(4, 2 * m, 0, nc)
+    S = _sample(torch, src, leaf, R)
+    ref = [torch.empty((2 * m, nc), dtype=torch.float64, device=gu.dev()) for _ in range(2)]
+    hss.hss_sample_offdiag_noalloc(gu.device_source(src), leaf, 0, gu.col_major(R), *ref)
+    A = src.to_dense()
+    A[_leaf_mask(2 * m, leaf)] = 0.0
+    bound = 2 * (2 * m + 2) * 2.0 ** -53 * (np.abs(A) @ np.abs(R)) * (1 + 1e-9)
+    for s, f in zip(S, ref):
+        assert np.all(np.abs(s - f.cpu().numpy()) <= bound)
+
+
 @pytest.mark.parametrize("nrhs,transpose", [(1000, False), (1000, True)])
 def test_wide_product(torch, nrhs, transpose):
     """Diagonal entries of 1e13 against zeros of X: the rows of H X there are
