@@ -108,7 +108,8 @@ __global__ void __launch_bounds__(256) k_asymmetric(const double* __restrict__ a
                                                     int* flag) {
   __shared__ unsigned long long t[64][65];
   const int bi = blockIdx.x, bj = blockIdx.y;
-  if (bi > bj || *(volatile int*)flag) return;
+  if (bi > bj) return;
+  if (__syncthreads_or(*(volatile int*)flag)) return;   // (the block as a whole: others set it meanwhile)
   const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
   const unsigned long long* p = (const unsigned long long*)a;
   unsigned long long v[16];

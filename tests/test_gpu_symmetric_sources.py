@@ -81,3 +81,14 @@ def test_one_bit_of_difference(hss, i, j):
     X = np.random.default_rng(0).standard_normal((333, 5))
     for Y, B in zip(got, (A, A.T)):
         assert np.linalg.norm(Y - B @ X) <= 1e-5 * np.linalg.norm(B @ X)
+
+
+def test_difference_in_every_tile(hss):
+    """Tiles that see the flag set by others while they begin."""
+    A = w.gaussian_kernel(_points(hss, 1900), 0.3, 0.5).to_dense()
+    A += np.triu(1e-9 * np.random.default_rng(3).random(A.shape))
+    got, per, _ = _run(hss, w.dense_source(A), 0)
+    assert per == 2
+    X = np.random.default_rng(0).standard_normal((1900, 5))
+    for Y, B in zip(got, (A, A.T)):
+        assert np.linalg.norm(Y - B @ X) <= 1e-5 * np.linalg.norm(B @ X)
