@@ -1343,10 +1343,14 @@ hss_status sample_columns(Ctx& c, hss_matrix_s* H, int c0, int c1) {
   SrcDev s = make_src(H->src, H->leaf_id);
   const double* Rc = H->R + (long long)c0 * n;
   if (H->src.kind == HSS_SRC_LAPLACE && H->o.precision != HSS_PREC_FP64) {
-    if (!H->pts) {
-      CK(dmalloc_async(&H->pts, sizeof(float4) * 2 * (size_t)n, st));
-      CK(launch_split_points(s, H->pts, st));
-      c.launches++;
+    if (!H->pts) {   // (without memory for them: the same bits from the points)
+      if (dmalloc_async(&H->pts, sizeof(float4) * 2 * (size_t)n, st) == cudaSuccess) {
+        CK(launch_split_points(s, H->pts, st));
+        c.launches++;
+      } else {
+        cudaGetLastError();
+        H->pts = nullptr;
+      }
     }
     s.pts = H->pts;
   }
@@ -3556,6 +3560,20 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
   // A point kernel is symmetric: one orientation serves both sides; a dense A
   // has two, unless only its own is asked for.
   const int orients = packed && Sc ? 2 : 1;
+  CK(dmalloc_async(&pR, packed_r_bytes(n, ncols, precision), st));
+  CK(launch_pack_r(Rr, n, n, ncols, precision, A->kind == HSS_SRC_TOEPLITZ, pR, st));
+  // (what can be done without comes last: the split points, the same bits
+  // without them, and the packed tiles of a generated source)
+  float4* pts = nullptr;
+  if (A->kind == HSS_SRC_LAPLACE) {
+    if (dmalloc_async(&pts, sizeof(float4) * 2 * (size_t)n, st) == cudaSuccess) {
+      CK(launch_split_points(s, pts, st));
+      s.pts = pts;
+    } else {
+      cudaGetLastError();
+      pts = nullptr;
+    }
+  }
   if ((A->kind == HSS_SRC_LAPLACE || A->kind == HSS_SRC_GAUSS) && precision == HSS_PREC_BF16X3) {
     const size_t pb = packed_a_bytes(n, precision, 1);
     if (pb <= (size_t(4) << 30)) {
@@ -3566,14 +3584,6 @@ hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int 
       }
     }
   }
-  float4* pts = nullptr;
-  if (A->kind == HSS_SRC_LAPLACE) {
-    CK(dmalloc_async(&pts, sizeof(float4) * 2 * (size_t)n, st));
-    CK(launch_split_points(s, pts, st));
-    s.pts = pts;
-  }
-  CK(dmalloc_async(&pR, packed_r_bytes(n, ncols, precision), st));
-  CK(launch_pack_r(Rr, n, n, ncols, precision, A->kind == HSS_SRC_TOEPLITZ, pR, st));
   if (packed) {
     if (!pA) CK(dmalloc_async(&pA, packed_a_bytes(n, precision, orients), st));
     CK(launch_pack_a(s, leaf, precision, orients, pA, st));

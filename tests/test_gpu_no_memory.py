@@ -149,3 +149,28 @@ assert bytes_[0] > 0 and bytes_[1] == 0   # A's own traffic, counted where it is
 
 def test_toeplitz_is_not_packed_where_one_orientation_fits(tmp_path):
     fake_alloc.run(TOEPLITZ, tmp_path)
+
+
+LAPLACE = r"""
+n, nc = 3000, 64
+P = w.laplace_kernel(w.uniform_points(n, 3, seed=2)).points
+src = hss.points_source(w.SRC_LAPLACE, gu.col_major(P[hss.hss_rcb_order(P, 100)]), 1.0)
+R = gu.col_major(w.gaussian_matrix(1, n, 0, nc))
+tiles = 3 * 16384 * -(-n // 128) * -(-n // 64)   # the packed matrix
+out = []
+for over in (None, tiles - 60000, 0, -60000):   # all; tiles at the cost of what comes after; no tiles; no split points either
+    S = [torch.full((n, nc), float("nan"), dtype=torch.float64, device=gu.dev()) for _ in range(2)]
+    if over is not None:   # leaf table, rounded R, packed R, split points
+        fake.fake_budget(4 * n + 8 * n * nc + 4 + 128 * 64 * -(-n // 64) + 32 * n + 1000 + over)
+    hss.hss_sample_offdiag(src, 100, hss.HSS_PREC_BF16X3, R, *S)
+    torch.cuda.synchronize()
+    fake.fake_budget(-1)
+    out.append(S)
+assert fake.fake_refused() >= 3
+assert all(torch.equal(a, b) for S in out[1:] for a, b in zip(S, out[0]))
+"""
+
+
+def test_mixed_samples_without_packed_tiles(tmp_path):
+    """Tiles and split points are for speed: the samples are the same bits."""
+    fake_alloc.run(LAPLACE, tmp_path)
