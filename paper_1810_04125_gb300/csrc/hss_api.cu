@@ -1214,6 +1214,7 @@ hss_status xs_sample(Ctx& c, const SrcDev& s, int w, const double* R, long long 
     for (int o = 0; o < no; ++o) {
       GemmJob j = jr;
       j.M = rows;
+      j.row0 = r0;
       j.C = O[o].S + (long long)r0 * lds; j.c_rs = lds; j.c_cs = 1;
       j.dup = O[o].dup ? O[o].dup + (long long)r0 * lds : nullptr;
       j.ea = ea + (size_t)O[o].trans * n + r0;

@@ -95,6 +95,7 @@ struct GemmJob {
   // rows a tile
   unsigned* state;
   unsigned* mask;
+  int row0;   // place of the first row along K (a chunk of rows of a square matrix)
 };
 enum : unsigned { XS_FMA = 1u, XS_WAIT = 2u, XS_PART = 4u };
 // The tile states of a sampling call whose rows were cut into chunks of `chunk`

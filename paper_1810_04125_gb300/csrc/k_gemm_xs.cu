@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(256, 5) k_xs_check(const GemmJob* __restrict__
   const uint32_t tmem = s_tmem;
   const int t = blockIdx.x - prefix[ji], ntn = (sj.N + XS_TN - 1) / XS_TN;
   const int ti = t / ntn, tj = t % ntn, i0 = ti * XS_TM, j0 = tj * XS_TN;
-  const int nkt = sj.nkt, kt0 = (i0 + XS_TM / 2) / XS_BK % nkt;
+  const int nkt = sj.nkt, kt0 = (sj.row0 + i0 + XS_TM / 2) / XS_BK % nkt;
   const uint8_t* gA = sj.pa + (size_t)ti * nkt * (XD * (size_t)XA);
   const uint8_t* gB = sj.pb + (size_t)tj * nkt * (XD * (size_t)XB);
   uint4 d[3][2];   // a thread's 16-byte chunks of one k-tile: two of A, one of B, both digits
