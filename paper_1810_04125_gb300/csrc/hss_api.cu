@@ -475,9 +475,16 @@ struct DevBuf {
     }
     p = nullptr;
     cap = 0;
-    // (room to grow, up to 64 MB of it: digits take gigabytes)
-    const size_t sz = std::max(bytes + std::min(bytes / 2, size_t(64) << 20), size_t(1) << 20);
+    // room to grow, up to 512 MB of it (digits take gigabytes, and every growth
+    // of them about a millisecond: with 64 MB the samples of a dense n = 16384
+    // compression took 38 ms instead of 35), or none
+    size_t sz = std::max(bytes + std::min(bytes / 2, size_t(512) << 20), size_t(1) << 20);
     cudaError_t e = dmalloc_async((void**)&p, sz, st);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      sz = bytes;
+      e = dmalloc_async((void**)&p, sz, st);
+    }
     if (e != cudaSuccess) return e;
     cap = sz;
     return cudaSuccess;
