@@ -14,8 +14,18 @@
  *    "row-major" means element (i, j) at p[i*ld + j].
  *  - Work is issued on the caller's CUDA stream (NULL = legacy default
  *    stream).  Calls return after their last stream synchronisation,
- *    except hss_matvec, hss_random_normal and hss_sample_offdiag, which
- *    are asynchronous on that stream.
+ *    except hss_matvec, hss_random_normal and hss_sample_offdiag (FP64),
+ *    which are asynchronous on that stream.
+ *  - FP64 products (the plain form's samples, merges, reductions and test
+ *    projections, hss_matvec) are sums of FMAs or, where they are large
+ *    enough, exact sums of products of digits cut to the scale of a row of
+ *    one operand and a column of the other.  Either way a result that sums K
+ *    terms a b is within (K + 2) 2^-53 sum |a b| of the exact one: results
+ *    that the digits would not settle to that are computed with FMAs.  Which
+ *    of the two is used follows the sizes of the whole call, so the last bits
+ *    of a column of hss_matvec can change with nrhs, and those of a
+ *    compression in a batch with the other matrices (pivots between columns
+ *    that are equal to rounding follow such bits).
  */
 #ifndef HSS_H
 #define HSS_H
@@ -283,7 +293,9 @@ hss_status hss_compress_batched(const hss_source* A, const hss_opts* opts, int c
  * it kept.  X, Y: device col-major n x nrhs (ldx, ldy >= n); Y is
  * overwritten.  Asynchronous on the stream, but for the handle's first
  * product or entry call outside of a capture: it lays out the task lists and
- * index tables that the handle keeps, and waits for the stream. */
+ * index tables that the handle keeps (a buffer of their size, until hss_free),
+ * and waits for the stream.  Without memory for them, or for the digits of a
+ * wide product, the product is formed without. */
 hss_status hss_matvec(hss_matrix H, int nrhs, const double* X, long long ldx,
                       double* Y, long long ldy, int transpose, void* stream);
 
@@ -301,7 +313,8 @@ hss_status hss_matvec(hss_matrix H, int nrhs, const double* X, long long ldx,
  * col-major nr x nc, ld ldo >= nr.  Uses a temporary device buffer and the
  * handle's index tables (see hss_matvec); returns
  * after a sync of the stream; HSS_ERR_ARG (entries left zero) when an index
- * is out of range. */
+ * is out of range, HSS_ERR_NOMEM when there is no memory for the tables,
+ * HSS_ERR_CUDA on a stream that is being captured. */
 hss_status hss_get_entries(hss_matrix H, int nr, const int* I, int nc, const int* J, double* out,
                            long long ldo, void* stream);
 
@@ -417,13 +430,16 @@ hss_status hss_random_normal(unsigned long long seed, int n, int col0, int ncols
  * Sc = (A - D^(L))^T R, where D^(L) = blockdiag of the leaves of the halving
  * tree with the given leaf size.  R: device col-major n x ncols (ldr);
  * Sr, Sc: device row-major n x ncols (row stride lds >= ncols); either may
- * be NULL to skip it.  precision: HSS_PREC_*.  Asynchronous. */
+ * be NULL to skip it.  precision: HSS_PREC_*.  Asynchronous in the FP64 form,
+ * whose device waits lose no result: a tile whose wait runs out is computed
+ * again.  The mixed forms return after a sync of the stream. */
 hss_status hss_sample_offdiag(const hss_source* A, int leaf, int precision, int ncols,
                               const double* R, long long ldr, double* Sr, double* Sc,
                               long long lds, void* stream);
 
 /* The same computation as hss_sample_offdiag in its FP64 form (same
- * arguments, same results; precision must be HSS_PREC_FP64 — the mixed
+ * arguments; sums of FP64 FMAs, so the same results to rounding and not bit
+ * for bit; precision must be HSS_PREC_FP64 — the mixed
  * forms stage their split operands in temporary buffers, so they return
  * HSS_ERR_UNSUPPORTED here), for callers that cannot let a library allocate
  * device memory:

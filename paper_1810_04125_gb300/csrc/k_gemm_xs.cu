@@ -13,7 +13,7 @@
 //
 // Measured (one GB300, both orientations, digits made in the call): a dense
 // n = 6001 by 200 columns 37.3 ms on the FP64 pipe (k_sample_fp64, 0.77
-// TFLOP/s, its last wave half empty) -> 1.38 ms; n = 8192 by 1024 columns 7.4
+// TFLOP/s, its last wave half empty) -> 1.40 ms; n = 8192 by 1024 columns 7.4
 // ms (37 TFLOP/s), of which the product kernel 6.7 ms (41 TFLOP/s, 3750
 // clocks per k-tile: near the 3456 in which shared memory can deliver the
 // 72 MMA operand pairs), the digits 0.48 and the maxima 0.11 ms (the latter
@@ -57,7 +57,7 @@
 // that were cut (with the row (1, 1e-20, ...) all of them).  In units of f, the
 // pairs left out are at most 7.03 2^62 a term and the operands' roundings 2^62,
 // together 2^65.01: K 2^65.01 in all.  FP64 FMAs guarantee K 2^-53 S, S = sum
-// |A(i,l) B(l,j)|, and the digits no less where S >= 2^118 (in f), an
+// |A(i,l) B(l,j)|, and the digits no less where S >= 2^118 (in f), a
 // 1/16 to 1/64 of (largest of the row) x (largest of the column).  k_xs_check
 // forms a lower bound of S for every element from the two leading digits, an
 // FP16 product that stops as soon as all elements of its tile have reached it
@@ -800,12 +800,12 @@ __global__ void __maxnreg__(96) k_xs_mm(const GemmJob* __restrict__ jobs, const 
 // One CTA per tile.  The magnitude of an element by its two leading digits,
 // h = max(|d0 + d1 / 256| - 2^-9, 0) <= |f| 2^-56 up to two roundings to FP16
 // (the digits below are at most 1.004 2^-9), so sum h_A h_B, with 64 for the
-// 2^118 of S above and 1.5 % for the roundings, is a lower bound of S.  One
-// k-tile first, then three at a time, from the tile's own place outwards
-// (matrices that decay have their large entries near the diagonal).  Bound by
-// the latency of its few loads: 5 to 11 us a launch (dense n = 6001, 200 columns:
-// 1.39 to 1.40 ms for the call; a product of 2048 columns with twelve launch
-// sets 3.75 to 3.87).
+// 2^118 of S above and 1.5 % for the roundings and the 0.01 of the exponent, is a
+// lower bound of S.  One k-tile first, then three at a time, from the tile's own
+// place outwards (matrices that decay have their large entries near the
+// diagonal).  Bound by the latency of its few loads: 5 to 11 us a launch (dense
+// n = 6001, 200 columns: 1.39 to 1.40 ms for the call; a product of 2048 columns
+// with twelve launch sets 3.73 to 3.84).
 constexpr int CKT = 3;                                   // most k-tiles a round
 constexpr uint32_t CK_SMEM = CKT * (XA + XB);
 constexpr int CK_MOST = XS_TM * XS_TN / 8;               // elements to compute one by one
